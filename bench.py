@@ -43,8 +43,9 @@ if ROOT not in sys.path:
 # Each set holds the SHA-256 of the kernel sources it was measured on; the
 # bench recomputes it and marks the roofline's counts stale when the
 # sources have changed since.
-#   FP64: 342 DFMA + 137 DMUL + 37 DADD per step (six right-hand sides
-#   included) = 516 FP64-pipe instructions, 858 FLOP (DFMA = 2).  The
+#   FP64: 342 multiply-adds, 137 products and 37 sums per step (six
+#   right-hand sides included; products and sums issue as DFMAs too) = 516
+#   FP64-pipe instructions of the one-thread kernel, 858 FLOP.  The
 #   DFMA-chain peak runs one DFMA per pipe slot, so pipe_frac below is the
 #   fraction of the FP64 pipe's instruction rate the kernel uses.
 FP64_FLOP_PER_STEP = 858
@@ -57,11 +58,11 @@ FP32_FLOP_PER_STEP = 1004
 FP32_THREAD_INSTR_PER_STEP = 787
 KERNEL_SOURCES = {
     64: ["integrate.cu", "elem64.cuh", "ff.cuh", "texp.cuh", "exp2_table.inc",
-         "dp5_tableau.cuh", "step_ctrl.cuh", "pair_force.cuh"],
+         "dp5_tableau.cuh", "step_ctrl.cuh", "pair_force.cuh", "regop.cuh"],
     32: ["integrate32.cu", "dp5_tableau.cuh"],
 }
 COUNTS_SOURCE_SHA256 = {
-    64: "130d7d1db1e117053912a66c771d9e78751bcc0dba47250e833458f06a8fefb4",
+    64: "d5c569ad3189817afd99549d55eb8ecb1a26b4d4691dcbe3ce9f99dc33bb0e57",
     32: "70e2932855a88f714f4f7b48b180d82a8b03cd6726c5035bdfd2c9d94b9bb1c1",
 }
 # DRAM bytes per trajectory of the integrator: ncu dram__bytes_read.sum +

@@ -4,7 +4,7 @@
  * The library integrates very many independent atom-diatom trajectories
  * A + BC -> products with the QCT method of Koots & Perez-Rios, "PyQCAMS:
  * Python Quasi-Classical Atom-Molecule Scattering" (Comput. Phys. Commun.),
- * one trajectory per CUDA thread on sm_103a:
+ * one or several CUDA threads per trajectory on sm_103a:
  *   - initial states from Bohr-Sommerfeld (v, j) levels with random
  *     orientation and vibrational phase (Sec. 2.1, Eqs. 5-7);
  *   - Hamilton's equations in Jacobi coordinates (Sec. 2, Eqs. 2-4) under
@@ -140,25 +140,27 @@ typedef struct {
                           stop test (used to test the integrator) */
   int32_t precision;   /* 64 = FP64 integrator; 32 = FP32 integrator with
                           compensated (Kahan) state updates */
-  int32_t persistent;  /* 1 = persistent refill-queue launch (finished lanes
-                          take the next trajectory from a device counter);
-                          0 = one thread per trajectory;
+  int32_t persistent;  /* 0 and 1: FP64 adaptive runs choose the launch by the
+                          batch (one thread per trajectory with a refill
+                          queue, or three and six lanes per trajectory; the
+                          results are the same bits on every path); FP32: 1 =
+                          persistent refill-queue launch (finished lanes take
+                          the next trajectory from a device counter), 0 = one
+                          thread per trajectory;
                           2 = three lanes per trajectory, 3 = six lanes
-                          per trajectory (FP64 adaptive steps only, else
-                          QCAMS_E_INVALID; block and blocks_per_sm are not
-                          used): a step takes about 2.8x (3.4x) fewer
-                          warp-wide FP64 instructions, for batches too
-                          small to fill the GPU (below ~10,000
-                          trajectories); a warp holds 10 (5) trajectories
-                          instead of 32 */
+                          per trajectory, from start to end (FP64 adaptive
+                          steps only, else QCAMS_E_INVALID; block and
+                          blocks_per_sm are not used); sums in an order of
+                          their own */
   int32_t block;       /* threads per block (0 = 128) */
-  int32_t blocks_per_sm; /* resident blocks per SM the integrator variant is
-                            compiled for (its __launch_bounds__ minimum, which
-                            caps registers per thread; 0 = 1).  Supported
-                            (block, blocks_per_sm): (128,1) (64,1) (128,3)
-                            (64,6) (64,7) (256,1); qcams_autotune picks one.
-                            The persistent grid is the resulting occupancy
-                            times the SM count. */
+  int32_t blocks_per_sm; /* resident blocks per SM the one-thread kernel of
+                            large all-Morse FP64 batches is compiled for (its
+                            __launch_bounds__ minimum, which caps registers
+                            per thread; 0 = 1).  Supported (block,
+                            blocks_per_sm): (128,1) (64,1) (128,3) (64,6)
+                            (64,7) (256,1); qcams_autotune picks one.  The
+                            persistent grid is the resulting occupancy times
+                            the SM count. */
   int32_t pad;
 } qcams_integ;
 

@@ -48,10 +48,10 @@ cudaError_t ctx_get(Ctx** out) {
   if (e == cudaSuccess) e = cudaMalloc(&c->level_flag, kLevelCells);
   if (e == cudaSuccess) e = cudaMalloc(&c->level_valid, kLevelCells);
   if (e == cudaSuccess) e = cudaMemset(c->level_valid, 0, kLevelCells);
-  if (e == cudaSuccess) e = cudaMalloc(&c->counters, sizeof(unsigned long long) * 8);
+  if (e == cudaSuccess) e = cudaMalloc(&c->counters, sizeof(unsigned long long) * kCounters);
   if (e == cudaSuccess) e = cudaMalloc(&c->req_out, sizeof(qcams_level) * kMaxLevelsReq);
   if (e == cudaSuccess) e = cudaMalloc(&c->req_in, sizeof(int32_t) * 3 * kMaxLevelsReq);
-  if (e == cudaSuccess) e = cudaMemset(c->counters, 0, sizeof(unsigned long long) * 8);
+  if (e == cudaSuccess) e = cudaMemset(c->counters, 0, sizeof(unsigned long long) * kCounters);
   for (int k = 0; k < 4 && e == cudaSuccess; ++k) e = cudaEventCreate(&c->ev[k]);
   if (e != cudaSuccess) {
     cudaFree(c->shapes); cudaFree(c->levels); cudaFree(c->level_flag); cudaFree(c->counters);
@@ -1030,7 +1030,8 @@ int qcams_autotune(const qcams_system* sys, int32_t n_sys, const qcams_integ* in
     e = copy_all(false);
     if (e == cudaSuccess) e = cudaEventRecord(ctx->ev[0], st);
     if (e == cudaSuccess)
-      e = launch_integrate(ss, ctx->shapes, tip, d, 64, mode, block, bps, *ctx, st);
+      e = mode == 1 ? launch_integrate_shape(ss, ctx->shapes, tip, d, block, bps, *ctx, st)
+                    : launch_integrate(ss, ctx->shapes, tip, d, 64, mode, block, bps, *ctx, st);
     if (e == cudaSuccess) e = cudaEventRecord(ctx->ev[1], st);
     unsigned long long cnt[2] = {0, 0};
     if (e == cudaSuccess)

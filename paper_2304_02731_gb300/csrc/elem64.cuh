@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include "ff.cuh"
+#include "regop.cuh"
 #include "texp.cuh"
 
 namespace qcams {
@@ -27,7 +28,8 @@ namespace {
 // multiply of the significands, so e costs one FMA.  y0/2 and 3y0/8 are
 // built on the integer / FP32 pipes (3y0/8 only multiplies e, so its FP32
 // rounding does not matter).  FP64 work: e, then two FMAs of the series.
-__device__ __forceinline__ double rsqrt_seeded(double s, float& rf) {
+template <class OP = OpPlain>
+__device__ __forceinline__ double rsqrt_seeded(double s, float& rf, const OP& op = OP()) {
   const unsigned hi = (unsigned)__double2hiint(s), lo = (unsigned)__double2loint(s);
   // biased exponent in [897, 1150] <=> FP32 normal (sign bit set: out of range)
   const bool in_range = (hi >> 20) - 897u < 254u;
@@ -50,7 +52,7 @@ __device__ __forceinline__ double rsqrt_seeded(double s, float& rf) {
   // P << (6 - top) puts the leading bit at bit 52, where it adds one to the
   // exponent field: hence the bias 1022 instead of 1023
   const double Y = __longlong_as_double((long long)(P << (6 - top)) + ((2 * ey + top + 1022) << 52));
-  const double e = fma(-s, Y, 1.0);
+  const double e = fma(-s, Y, op.one());
   const double c = fma(e, y38, y0h);
   return fma(e, c, y0);
 }
@@ -74,19 +76,21 @@ constexpr float kExpInvLf = (float)kExpInvL;
 // integer pipe, r_h^2 split exactly by an FMA) and r^3/6 <= 1.5e-12 in
 // FP32, then w is rebuilt as a double on the integer pipe.  FP64 work: the
 // reduction, r + w, and the table product.
-__device__ __forceinline__ double texp_hint(double x, float xa, const double* __restrict__ T) {
+template <class OP = OpPlain>
+__device__ __forceinline__ double texp_hint(double x, float xa, const double* __restrict__ T,
+                                            const OP& op = OP()) {
   const float kf = fmaf(xa, kExpInvLf, 12582912.0f);   // 1.5 * 2^23 + k
   const int k = __float_as_int(kf) - 0x4B400000;
   const unsigned kb = __float_as_uint(kf - 12582912.0f);   // k as an FP32 value, exact
   const unsigned khi = (kb & 0x80000000u) | (((kb & 0x7fffffffu) >> 3) + (896u << 20));
   const double kd = __hiloint2double(kb ? (int)khi : 0, (int)(kb << 29));
-  const double r = fma(-kd, kExpL1, x);
+  const double r = fma(-kd, op.exp_l1(), x);
   float rh, rl;
   split_ff(r, rh, rl);
   const float P = __fmul_rn(rh, rh);
   const float Pl = fmaf(2.0f * rh, rl, fmaf(rh, rh, -P));   // r^2 = P + Pl to 2^-46
   const float cub = (P * rh) * (1.0f / 6.0f);
-  const double p = r + ff_to_double(0.5f * P, fmaf(0.5f, Pl, cub));
+  const double p = op.add(r, ff_to_double(0.5f * P, fmaf(0.5f, Pl, cub)));
   const double Tj = T[k & (kExpTableSize - 1)];
   const double y = fma(Tj, p, Tj);
   const double ex = __hiloint2double(__double2hiint(y) + ((k >> 11) << 20), __double2loint(y));

@@ -1,6 +1,9 @@
 // Trajectory integrator: Hamilton's equations (Sec. 2, Eqs. 3-4) in Jacobi
 // coordinates, one trajectory per thread, Dormand-Prince 5(4) with a
 // per-lane adaptive step (Sec. 3.2: SciPy's solve_ivp RK45 step control).
+// Large all-Morse batches run here until their queue is empty; what is left,
+// and every other batch, runs the same arithmetic with several lanes per
+// trajectory (integrate_grp.cu; launch_stages below).
 //
 // GB300 design:
 //  * The state (12 doubles) and the stage derivatives live in registers;
@@ -19,9 +22,11 @@
 //  * Persistent mode: a finished lane takes the next trajectory index from a
 //    device counter, with one atomicAdd per warp for all lanes that need
 //    work (ballot + popc), so warps stay full until the queue drains.
-//  * GB300 issues one warp-wide FP64 instruction per 64 cycles per SM
+//  * GB300 issues one warp-wide FP64 instruction per 64 to 76 cycles per SM
 //    sub-partition (1/64 of the FP32 rate), so the kernel is bound by the
-//    number of FP64-pipe instructions per step.  Everything that does not
+//    number of FP64-pipe instructions per step, and by their form: products
+//    and sums are DFMAs on registers (regop.cuh), which took the 200,000-lane
+//    sweep sample from 1.01 to 1.08 G attempts/s.  Everything that does not
 //    need 53-bit arithmetic runs on the integer / FP32 pipes: the step-size
 //    controller's error norm (magnitudes taken from the doubles' exponent and
 //    leading mantissa bits, ratios in FP32), the stop tests (integer compares
@@ -39,6 +44,7 @@
 //    base) and the embedded error estimate.  The new state (stage 7, v_n+1)
 //    keeps its FP64 sums.
 #include <cuda_runtime.h>
+#include <cstdint>
 
 #include "qcams_device.cuh"
 #include "qcams_internal.h"
@@ -69,29 +75,29 @@ constexpr unsigned FULL = 0xffffffffu;
 // ---------------------------------------------------------------------------
 template <bool MORSE>
 __device__ __forceinline__ void accel(const DevSys& S, const double* __restrict__ T,
-                                      const double* x, double* a, double* s2) {
+                                      const double* x, double* a, double* s2, const OpReg& op) {
   const double rab0 = x[0], rab1 = x[1], rab2 = x[2];
   const double rbc0 = fma(-S.cB, x[0], x[3]), rbc1 = fma(-S.cB, x[1], x[4]),
                rbc2 = fma(-S.cB, x[2], x[5]);
   const double rca0 = fma(S.cA, x[0], x[3]), rca1 = fma(S.cA, x[1], x[4]),
                rca2 = fma(S.cA, x[2], x[5]);
-  s2[0] = fma(rab0, rab0, fma(rab1, rab1, rab2 * rab2));
-  s2[1] = fma(rbc0, rbc0, fma(rbc1, rbc1, rbc2 * rbc2));
-  s2[2] = fma(rca0, rca0, fma(rca1, rca1, rca2 * rca2));
-  const double u0 = pair_u<MORSE>(S.pair[0], s2[0], T);
-  const double u1 = pair_u<MORSE>(S.pair[1], s2[1], T);
-  const double u2 = pair_u<MORSE>(S.pair[2], s2[2], T);
-  const double f0 = (MORSE ? S.kf_morse[0] : S.kf[0]) * u0;
-  const double f1 = (MORSE ? S.kf_morse[1] : S.kf[1]) * u1;
-  const double f2 = (MORSE ? S.kf_morse[2] : S.kf[2]) * u2;
-  const double h1 = (MORSE ? S.kf_morse[3] : S.kf[3]) * u1;
-  const double h2 = (MORSE ? S.kf_morse[4] : S.kf[4]) * u2;
-  a[0] = fma(f0, rab0, fma(f1, rbc0, f2 * rca0));
-  a[1] = fma(f0, rab1, fma(f1, rbc1, f2 * rca1));
-  a[2] = fma(f0, rab2, fma(f1, rbc2, f2 * rca2));
-  a[3] = fma(h1, rbc0, h2 * rca0);
-  a[4] = fma(h1, rbc1, h2 * rca1);
-  a[5] = fma(h1, rbc2, h2 * rca2);
+  s2[0] = fma(rab0, rab0, fma(rab1, rab1, op.mul(rab2, rab2)));
+  s2[1] = fma(rbc0, rbc0, fma(rbc1, rbc1, op.mul(rbc2, rbc2)));
+  s2[2] = fma(rca0, rca0, fma(rca1, rca1, op.mul(rca2, rca2)));
+  const double u0 = pair_u<MORSE>(S.pair[0], s2[0], T, op);
+  const double u1 = pair_u<MORSE>(S.pair[1], s2[1], T, op);
+  const double u2 = pair_u<MORSE>(S.pair[2], s2[2], T, op);
+  const double f0 = op.mul(MORSE ? S.kf_morse[0] : S.kf[0], u0);
+  const double f1 = op.mul(MORSE ? S.kf_morse[1] : S.kf[1], u1);
+  const double f2 = op.mul(MORSE ? S.kf_morse[2] : S.kf[2], u2);
+  const double h1 = op.mul(MORSE ? S.kf_morse[3] : S.kf[3], u1);
+  const double h2 = op.mul(MORSE ? S.kf_morse[4] : S.kf[4], u2);
+  a[0] = fma(f0, rab0, fma(f1, rbc0, op.mul(f2, rca0)));
+  a[1] = fma(f0, rab1, fma(f1, rbc1, op.mul(f2, rca1)));
+  a[2] = fma(f0, rab2, fma(f1, rbc2, op.mul(f2, rca2)));
+  a[3] = fma(h1, rbc0, op.mul(h2, rca0));
+  a[4] = fma(h1, rbc1, op.mul(h2, rca1));
+  a[5] = fma(h1, rbc2, op.mul(h2, rca2));
 }
 
 // Position of stage s (1-based, s >= 2) from base = rho + h c_s v.
@@ -100,10 +106,10 @@ __device__ __forceinline__ void accel(const DevSys& S, const double* __restrict_
 // zero in exact arithmetic are skipped (stage 2 has no acceleration term).
 template <int s>
 __device__ __forceinline__ void stage_x(const double* base, const double (*acc)[6], double hh,
-                                        double* x) {
+                                        double* x, const OpReg& op) {
   double w[s > 2 ? s - 2 : 1];
 #pragma unroll
-  for (int q = 1; q <= s - 2; ++q) w[q - 1] = dpA2Zero(s, q) ? 0.0 : hh * kT.a2[s][q];
+  for (int q = 1; q <= s - 2; ++q) w[q - 1] = dpA2Zero(s, q) ? 0.0 : op.mul(hh, kT.a2[s][q]);
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
     double xi = base[i];
@@ -116,13 +122,13 @@ __device__ __forceinline__ void stage_x(const double* base, const double (*acc)[
 // The same for stages 2 and 3 (c_s < 1), forming rho + h c_s v per component.
 template <int s>
 __device__ __forceinline__ void stage_x(const double* rho, const double* vel, const double (*acc)[6],
-                                        double h, double hh, double* x) {
+                                        double h, double hh, double* x, const OpReg& op) {
   static_assert(s == 2 || s == 3, "stages 4-6 use stage_x_ff, 7 the FP64 form");
-  const double hc = h * dpC(s);
+  const double hc = op.mul(h, dpC(s));
   double base[6];
 #pragma unroll
   for (int i = 0; i < 6; ++i) base[i] = fma(hc, vel[i], rho[i]);
-  stage_x<s>(base, acc, hh, x);
+  stage_x<s>(base, acc, hh, x, op);
 }
 
 // Position of stage s = 4, 5, 6: base + h^2 sum_q (A^2)_{sq} a_q, the sum
@@ -133,7 +139,7 @@ __device__ __forceinline__ void stage_x(const double* rho, const double* vel, co
 // keep FP64 sums.
 template <int s>
 __device__ __forceinline__ void stage_x_ff(const double* base, const double (*acc)[6], float hhh,
-                                           float hhl, double* x) {
+                                           float hhl, double* x, const OpReg& op) {
   static_assert(s >= 4 && s <= 6, "stages 4-6");
   float wh[s - 2], wl[s - 2];
 #pragma unroll
@@ -152,7 +158,7 @@ __device__ __forceinline__ void stage_x_ff(const double* base, const double (*ac
       split_ff(acc[q - 1][i], ah, al);
       ff_dot_acc(sm, cm, wh[q - 1], wl[q - 1], ah, al);
     }
-    x[i] = base[i] + ff_to_double(sm, cm);
+    x[i] = op.add(base[i], ff_to_double(sm, cm));
   }
 }
 
@@ -170,35 +176,40 @@ template <bool MORSE>
 __device__ __forceinline__ void dp_step(const DevSys& S, const double* __restrict__ T,
                                         const double* rho, const double* vel, double (*acc)[6],
                                         double h, double* xn, double* vn, float* er, float* ev,
-                                        double* s2) {
-  const double hh = h * h;
+                                        double* s2, const OpReg& op, const double* sB) {
+  const double hh = op.mul(h, h);
   float hhh, hhl;
   split_ff(hh, hhh, hhl);
   double x[6];
-  stage_x<2>(rho, vel, acc, h, hh, x);
-  accel<MORSE>(S, T, x, acc[1], s2);
-  stage_x<3>(rho, vel, acc, h, hh, x);
-  accel<MORSE>(S, T, x, acc[2], s2);
+  stage_x<2>(rho, vel, acc, h, hh, x, op);
+  accel<MORSE>(S, T, x, acc[1], s2, op);
+  stage_x<3>(rho, vel, acc, h, hh, x, op);
+  accel<MORSE>(S, T, x, acc[2], s2, op);
   double base[6];
+  const double hc4 = op.mul(h, dpC(4)), hc5 = op.mul(h, dpC(5));
 #pragma unroll
-  for (int i = 0; i < 6; ++i) base[i] = fma(h * dpC(4), vel[i], rho[i]);
-  stage_x_ff<4>(base, acc, hhh, hhl, x);
-  accel<MORSE>(S, T, x, acc[3], s2);
+  for (int i = 0; i < 6; ++i) base[i] = fma(hc4, vel[i], rho[i]);
+  stage_x_ff<4>(base, acc, hhh, hhl, x, op);
+  accel<MORSE>(S, T, x, acc[3], s2, op);
 #pragma unroll
-  for (int i = 0; i < 6; ++i) base[i] = fma(h * dpC(5), vel[i], rho[i]);
-  stage_x_ff<5>(base, acc, hhh, hhl, x);
-  accel<MORSE>(S, T, x, acc[4], s2);
+  for (int i = 0; i < 6; ++i) base[i] = fma(hc5, vel[i], rho[i]);
+  stage_x_ff<5>(base, acc, hhh, hhl, x, op);
+  accel<MORSE>(S, T, x, acc[4], s2, op);
 #pragma unroll
   for (int i = 0; i < 6; ++i) base[i] = fma(h, vel[i], rho[i]);   // c_6 = c_7 = 1
-  stage_x_ff<6>(base, acc, hhh, hhl, x);
-  accel<MORSE>(S, T, x, acc[5], s2);
-  stage_x<7>(base, acc, hh, xn);
-  accel<MORSE>(S, T, xn, acc[6], s2);
+  stage_x_ff<6>(base, acc, hhh, hhl, x, op);
+  accel<MORSE>(S, T, x, acc[5], s2, op);
+  stage_x<7>(base, acc, hh, xn, op);
+  accel<MORSE>(S, T, xn, acc[6], s2, op);
+  // the weights b_q as register operands
+  double bq[7];
+#pragma unroll
+  for (int q = 1; q <= 6; ++q) bq[q] = static_cast<const volatile double*>(sB)[q];
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
-    double vb = kT.b[1] * acc[0][i];
+    double vb = op.mul(bq[1], acc[0][i]);
 #pragma unroll
-    for (int q = 3; q <= 6; ++q) vb = fma(kT.b[q], acc[q - 1][i], vb);
+    for (int q = 3; q <= 6; ++q) vb = fma(bq[q], acc[q - 1][i], vb);
     vn[i] = fma(h, vb, vel[i]);
     // (e^T A)_2 = e_2 = 0 and (e^T A)_7 = 0: a_2 never enters, a_7 only ev
     float es, ec, rs, rc, ah, al;
@@ -233,7 +244,7 @@ struct LaneState {
 // per trajectory, in FP64.
 template <bool MORSE>
 __device__ double initial_step(const DevSys& S, const double* __restrict__ T, const LaneState& L,
-                               double rtol, double atol) {
+                               double rtol, double atol, const OpReg& op) {
   double atv[2] = {atol * S.inv_mu12, atol * S.inv_mu123};
   double d0 = 0.0, d1 = 0.0;
 #pragma unroll
@@ -251,7 +262,7 @@ __device__ double initial_step(const DevSys& S, const double* __restrict__ T, co
   double x1[6], a1[6], s2[3];
 #pragma unroll
   for (int i = 0; i < 6; ++i) x1[i] = fma(h0, L.vel[i], L.rho[i]);
-  accel<MORSE>(S, T, x1, a1, s2);
+  accel<MORSE>(S, T, x1, a1, s2, op);
   double d2 = 0.0;
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
@@ -275,7 +286,7 @@ __device__ __forceinline__ bool runnable(int st) {
 template <bool MORSE>
 __device__ bool lane_load(const SysSet& sys, const IntegParams& ip, const double* __restrict__ T,
                           const DevBatch& B, int64_t i, LaneState& L,
-                          unsigned long long& rhs_count) {
+                          unsigned long long& rhs_count, const OpReg& op) {
   L.status = B.status[i];
   if (!runnable(L.status)) return false;
   L.sid = B.sys_id[i];
@@ -302,28 +313,30 @@ __device__ bool lane_load(const SysSet& sys, const IntegParams& ip, const double
   L.atv[0] = (float)(ip.atol * S.inv_mu12);
   L.atv[1] = (float)(ip.atol * S.inv_mu123);
   double s2[3];
-  accel<MORSE>(S, T, L.rho, L.acc[0], s2);
+  accel<MORSE>(S, T, L.rho, L.acc[0], s2, op);
   rhs_count += 1;
   if (!(L.h > 0.0)) {
-    L.h = initial_step<MORSE>(S, T, L, ip.rtol, ip.atol);
+    L.h = initial_step<MORSE>(S, T, L, ip.rtol, ip.atol, op);
     rhs_count += 1;
   }
   return true;
 }
 
 template <bool MORSE>
-__device__ void lane_store(const SysSet& sys, const DevBatch& B, int64_t i, const LaneState& L) {
+__device__ void lane_store(const SysSet& sys, const DevBatch& B, int64_t i, const LaneState& L,
+                           bool handoff = false) {
   const DevSys& S = sys.s[L.sid];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     B.y[k][i] = L.rho[k];
     B.y[3 + k][i] = L.rho[3 + k];
-    B.y[6 + k][i] = L.vel[k] * S.mu12;
-    B.y[9 + k][i] = L.vel[3 + k] * S.mu123;
+    B.y[6 + k][i] = handoff ? L.vel[k] : L.vel[k] * S.mu12;
+    B.y[9 + k][i] = handoff ? L.vel[3 + k] : L.vel[3 + k] * S.mu123;
   }
   B.t[i] = L.t;
   B.h[i] = L.h;
-  B.status[i] = static_cast<uint8_t>(L.status);
+  B.status[i] = static_cast<uint8_t>(
+      handoff ? kHandoff | (L.rejected ? kHandoffRejected : 0) : L.status);
   B.nsteps[i] = L.nacc;
   B.nrej[i] = L.nrej;
 }
@@ -343,7 +356,7 @@ __device__ void lane_store(const SysSet& sys, const DevBatch& B, int64_t i, cons
 template <bool MORSE>
 __device__ __forceinline__ void lane_attempt(const SysSet& sys, const DevShape* shapes,
                                              const IntegParams& ip, const double* __restrict__ T,
-                                             LaneState& L) {
+                                             LaneState& L, const OpReg& op, const double* sB) {
   const DevSys& S = sys.s[L.sid];
   {
     const int eh = (__double2hiint(L.h) >> 20) & 0x7ff;
@@ -355,7 +368,7 @@ __device__ __forceinline__ void lane_attempt(const SysSet& sys, const DevShape* 
   }
   double xn[6], vn[6], s2[3];
   float er[6], ev[6];
-  dp_step<MORSE>(S, T, L.rho, L.vel, L.acc, L.h, xn, vn, er, ev, s2);
+  dp_step<MORSE>(S, T, L.rho, L.vel, L.acc, L.h, xn, vn, er, ev, s2, op, sB);
   unsigned bad = 0, ignore = 0;
   float sum = 0.f;
   const float rt = ip.rtol_f, at = ip.atol_f;
@@ -429,33 +442,21 @@ __device__ __forceinline__ void flush_counters(unsigned long long rhs, unsigned 
   }
 }
 
-// One thread per trajectory.
-template <bool MORSE, int BLOCK, int MINB>
-__global__ void __launch_bounds__(BLOCK, MINB) k_integrate_plain(SysSet sys, const DevShape* shapes,
-                                                         IntegParams ip, DevBatch B,
-                                                         unsigned long long* counters) {
-  __shared__ double sT[kExpTableSize];
-  load_exp_table(sT);
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  unsigned long long rhs = 0, steps = 0;
-  LaneState L;
-  if (i < B.n && lane_load<MORSE>(sys, ip, sT, B, i, L, rhs)) {
-    while (L.status == QCAMS_LANE_RUNNING) lane_attempt<MORSE>(sys, shapes, ip, sT, L);
-    rhs += 6ull * L.calls;
-    steps += L.calls;
-    lane_store<MORSE>(sys, B, i, L);
-  }
-  flush_counters(rhs, steps, counters);
-}
-
 // Persistent refill-queue launch: each warp pops trajectory indices for all
-// of its idle lanes with one atomicAdd (ballot + popc + shuffle).
+// of its idle lanes with one atomicAdd (ballot + popc + shuffle).  With
+// q.keep > 0 the lanes that are left when the queue is empty are handed on
+// (StageQueue).
 template <bool MORSE, int BLOCK, int MINB>
 __global__ void __launch_bounds__(BLOCK, MINB) k_integrate_persistent(SysSet sys, const DevShape* shapes,
                                                               IntegParams ip, DevBatch B,
-                                                              unsigned long long* counters) {
-  __shared__ double sT[kExpTableSize];
-  load_exp_table(sT);
+                                                              unsigned long long* counters,
+                                                              StageQueue q) {
+  __shared__ double sT[kExpTableSize], sK[kOpRegs], sB[8];
+  op_reg_fill(sK);
+  if (threadIdx.x < 8) sB[threadIdx.x] = kT.b[threadIdx.x];
+  load_exp_table(sT);   // ends with a barrier
+  OpReg op;
+  op.load(sK);
   const unsigned lane = threadIdx.x & 31u;
   unsigned long long rhs = 0, steps = 0;
   LaneState L;
@@ -467,30 +468,74 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_integrate_persistent(SysSet sys
     if (want) {
       const int leader = __ffs(want) - 1;
       unsigned long long base = 0;
-      if ((int)lane == leader) base = atomicAdd(&counters[2], (unsigned long long)__popc(want));
+      if ((int)lane == leader) base = atomicAdd(q.head, (unsigned long long)__popc(want));
       base = __shfl_sync(FULL, base, leader);
+      bool skip = false;   // took a lane that does not run
       if (need) {
         const int64_t k = (int64_t)(base + __popc(want & ((1u << lane) - 1u)));
         if (k >= B.n) {
           exhausted = true;
         } else {
           idx = k;
-          have = lane_load<MORSE>(sys, ip, sT, B, idx, L, rhs);
+          have = lane_load<MORSE>(sys, ip, sT, B, idx, L, rhs, op);
+          skip = !have;
         }
       }
+      const unsigned gone = __ballot_sync(FULL, skip);
+      if (gone && lane == 0) atomicAdd(q.retired, (unsigned long long)__popc(gone));
     }
     if (__all_sync(FULL, exhausted && !have)) break;
-    if (have) {
-      lane_attempt<MORSE>(sys, shapes, ip, sT, L);
-      if (L.status != QCAMS_LANE_RUNNING) {
+    if (q.keep > 0 && stage_over(q, B.n, lane)) {
+      const unsigned pass = __ballot_sync(FULL, have);
+      unsigned long long at = 0;
+      if (lane == 0) at = atomicAdd(q.n_out, (unsigned long long)__popc(pass));
+      at = __shfl_sync(FULL, at, 0);
+      if (have) {
+        rhs += 6ull * L.calls;
+        steps += L.calls;
+        lane_store<MORSE>(sys, B, idx, L, true);
+        q.list_out[at + __popc(pass & ((1u << lane) - 1u))] = idx;
+      }
+      break;
+    }
+    if (have) lane_attempt<MORSE>(sys, shapes, ip, sT, L, op, sB);
+    const bool done = have && L.status != QCAMS_LANE_RUNNING;
+    const unsigned ended = __ballot_sync(FULL, done);
+    if (ended) {
+      if (done) {
         rhs += 6ull * L.calls;
         steps += L.calls;
         lane_store<MORSE>(sys, B, idx, L);
         have = false;
       }
+      if (lane == 0) atomicAdd(q.retired, (unsigned long long)__popc(ended));
     }
   }
   flush_counters(rhs, steps, counters);
+}
+
+// Starting step of every runnable lane that has none yet (h = 0), for the
+// lane-group stages: two right-hand sides a lane, once per trajectory.
+template <bool MORSE>
+__global__ void __launch_bounds__(128) k_start_step(SysSet sys, IntegParams ip, DevBatch B,
+                                                    unsigned long long* counters) {
+  __shared__ double sT[kExpTableSize], sK[kOpRegs], sB[8];
+  op_reg_fill(sK);
+  if (threadIdx.x < 8) sB[threadIdx.x] = kT.b[threadIdx.x];
+  load_exp_table(sT);   // ends with a barrier
+  OpReg op;
+  op.load(sK);
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  unsigned long long rhs = 0;
+  if (i < B.n && runnable(B.status[i]) && !(B.h[i] > 0.0)) {
+    LaneState L;
+    unsigned long long all = 0;
+    if (lane_load<MORSE>(sys, ip, sT, B, i, L, all, op)) {
+      B.h[i] = L.h;
+      rhs = 1;
+    }
+  }
+  flush_counters(rhs, 0, counters);
 }
 
 // Fixed-step mode: exactly max_steps steps of size h_fixed, no control and
@@ -498,8 +543,12 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_integrate_persistent(SysSet sys
 template <bool MORSE>
 __global__ void __launch_bounds__(128) k_integrate_fixed(SysSet sys, IntegParams ip, DevBatch B,
                                                          unsigned long long* counters) {
-  __shared__ double sT[kExpTableSize];
-  load_exp_table(sT);
+  __shared__ double sT[kExpTableSize], sK[kOpRegs], sB[8];
+  op_reg_fill(sK);
+  if (threadIdx.x < 8) sB[threadIdx.x] = kT.b[threadIdx.x];
+  load_exp_table(sT);   // ends with a barrier
+  OpReg op;
+  op.load(sK);
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   unsigned long long rhs = 0, steps = 0;
   if (i < B.n) {
@@ -518,13 +567,13 @@ __global__ void __launch_bounds__(128) k_integrate_fixed(SysSet sys, IntegParams
         L.vel[3 + k] = B.y[9 + k][i] * S.inv_mu123;
       }
       double s2[3];
-      accel<MORSE>(S, sT, L.rho, L.acc[0], s2);
+      accel<MORSE>(S, sT, L.rho, L.acc[0], s2, op);
       double t = B.t[i];
       const double h = ip.h_fixed;
       for (long long it = 0; it < ip.max_steps; ++it) {
         double xn[6], vn[6];
         float er[6], ev[6];
-        dp_step<MORSE>(S, sT, L.rho, L.vel, L.acc, h, xn, vn, er, ev, s2);
+        dp_step<MORSE>(S, sT, L.rho, L.vel, L.acc, h, xn, vn, er, ev, s2, op, sB);
 #pragma unroll
         for (int q = 0; q < 6; ++q) {
           L.rho[q] = xn[q];
@@ -622,41 +671,33 @@ int find_variant(int block, int minb) {
 
 template <bool MORSE, int BLOCK, int MINB>
 cudaError_t launch_shape(const SysSet& sys, const DevShape* shapes, const IntegParams& ip,
-                         const DevBatch& b, int persistent, Ctx& ctx, cudaStream_t st,
-                         int* blocks_per_sm_out) {
-  if (persistent) {
-    cudaError_t e = cudaMemsetAsync(ctx.counters + 2, 0, sizeof(unsigned long long), st);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, k_integrate_persistent<MORSE, BLOCK, MINB>, BLOCK, 0);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
-    if (blocks_per_sm_out) *blocks_per_sm_out = per_sm;
-    long long grid = (long long)per_sm * ctx.sm_count;
-    const long long need = (b.n + BLOCK - 1) / BLOCK;
-    if (grid > need) grid = need;
-    if (grid < 1) grid = 1;
-    k_integrate_persistent<MORSE, BLOCK, MINB><<<(unsigned)grid, BLOCK, 0, st>>>(
-        sys, shapes, ip, b, ctx.counters);
-    return cudaGetLastError();
-  }
-  const unsigned grid = (unsigned)((b.n + BLOCK - 1) / BLOCK);
-  k_integrate_plain<MORSE, BLOCK, MINB><<<grid, BLOCK, 0, st>>>(sys, shapes, ip, b, ctx.counters);
+                         const DevBatch& b, int sm_count, unsigned long long* counters,
+                         const StageQueue& q, cudaStream_t st) {
+  int per_sm = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      &per_sm, k_integrate_persistent<MORSE, BLOCK, MINB>, BLOCK, 0);
+  if (e != cudaSuccess) return e;
+  if (per_sm < 1) per_sm = 1;
+  long long grid = (long long)per_sm * sm_count;
+  const long long need = (b.n + BLOCK - 1) / BLOCK;
+  if (grid > need) grid = need;
+  if (grid < 1) grid = 1;
+  k_integrate_persistent<MORSE, BLOCK, MINB><<<(unsigned)grid, BLOCK, 0, st>>>(
+      sys, shapes, ip, b, counters, q);
   return cudaGetLastError();
 }
 
 template <bool MORSE>
 cudaError_t launch_variant(int v, const SysSet& sys, const DevShape* shapes,
-                           const IntegParams& ip, const DevBatch& b, int persistent, Ctx& ctx,
-                           cudaStream_t st, int* bps) {
+                           const IntegParams& ip, const DevBatch& b, int sm_count,
+                           unsigned long long* counters, const StageQueue& q, cudaStream_t st) {
   switch (v) {
-    case 0: return launch_shape<MORSE, 128, 1>(sys, shapes, ip, b, persistent, ctx, st, bps);
-    case 1: return launch_shape<MORSE, 64, 1>(sys, shapes, ip, b, persistent, ctx, st, bps);
-    case 2: return launch_shape<MORSE, 128, 3>(sys, shapes, ip, b, persistent, ctx, st, bps);
-    case 3: return launch_shape<MORSE, 64, 6>(sys, shapes, ip, b, persistent, ctx, st, bps);
-    case 4: return launch_shape<MORSE, 64, 7>(sys, shapes, ip, b, persistent, ctx, st, bps);
-    case 5: return launch_shape<MORSE, 256, 1>(sys, shapes, ip, b, persistent, ctx, st, bps);
+    case 0: return launch_shape<MORSE, 128, 1>(sys, shapes, ip, b, sm_count, counters, q, st);
+    case 1: return launch_shape<MORSE, 64, 1>(sys, shapes, ip, b, sm_count, counters, q, st);
+    case 2: return launch_shape<MORSE, 128, 3>(sys, shapes, ip, b, sm_count, counters, q, st);
+    case 3: return launch_shape<MORSE, 64, 6>(sys, shapes, ip, b, sm_count, counters, q, st);
+    case 4: return launch_shape<MORSE, 64, 7>(sys, shapes, ip, b, sm_count, counters, q, st);
+    case 5: return launch_shape<MORSE, 256, 1>(sys, shapes, ip, b, sm_count, counters, q, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -682,11 +723,119 @@ cudaError_t launch_ff_dot_check(const double* a, const double* w, int m, double*
   return cudaGetLastError();
 }
 
+cudaError_t launch_integrate_shape(const SysSet& sys, const DevShape* shapes,
+                                   const IntegParams& ip, const DevBatch& b, int block,
+                                   int blocks_per_sm, Ctx& ctx, cudaStream_t st) {
+  const int v = find_variant(block, blocks_per_sm);
+  if (v < 0) return cudaErrorInvalidValue;
+  cudaError_t e = cudaMemsetAsync(ctx.counters, 0, kCounters * sizeof(unsigned long long), st);
+  if (e != cudaSuccess) return e;
+  StageQueue q;
+  q.head = ctx.counters + 4;
+  q.retired = ctx.counters + 5;
+  return all_morse(sys)
+             ? launch_variant<true>(v, sys, shapes, ip, b, ctx.sm_count, ctx.counters, q, st)
+             : launch_variant<false>(v, sys, shapes, ip, b, ctx.sm_count, ctx.counters, q, st);
+}
+
+namespace {
+
+// FP64 adaptive run of modes 0 and 1 in stages.  A stage runs until its
+// source is used up and at most keep_per_sm trajectories per SM are
+// unfinished, then hands those on (StageQueue): near its end a batch has few
+// long trajectories scattered over its warps, each warp-wide FP64
+// instruction costs a sub-partition 64 cycles however many lanes it serves,
+// and packing the survivors into fewer warps, with more lanes each, shortens
+// their steps.  Every stage forms the same bits, so the path a trajectory
+// takes does not show in its results.  Where the lines lie (GB300, 152 SMs):
+//  * The one-thread kernel only for all-Morse batches of at least 512
+//    trajectories per SM (77,824), which fill it twice over: there it runs
+//    1.08 G attempts/s against 1.06 of the three-lane queue (200,000 sweep
+//    lanes); in the generic form the queue is ahead, 0.84 against 0.75, and
+//    below that size the one-thread kernel has idle sub-partitions (0.54
+//    against 0.97 at 12,096 lanes).  It hands on as soon as its source is
+//    empty: its own capacity is 256 per SM.
+//  * Three lanes per trajectory hold 120 trajectories per SM; at 80 and at 20
+//    per SM (2 warps and half a warp per sub-partition) the survivors are
+//    packed again, the last time with six lanes each (7.3 instead of 8.8 us a
+//    step when each sub-partition has one warp).
+// 12,288 sweep lanes take 472 ms this way, 572 ms with three lanes to the
+// end, 660 ms without packing and 1,250 ms in the one-thread kernel alone;
+// 200,000 mixed lanes 769 ms against 1,440 ms.
+struct Stage {
+  int lanes;         // lanes per trajectory (1: the persistent kernel)
+  int keep_per_sm;   // hands on at this many trajectories per SM (0: none)
+};
+constexpr Stage kStages[] = {{1, 256}, {3, 80}, {3, 20}, {6, 0}};
+constexpr int kNumStages = sizeof(kStages) / sizeof(kStages[0]);
+constexpr int kOneThreadMinPerSm = 512;
+static_assert(4 + 4 * kNumStages <= kCounters, "a counter block per stage");
+
+// The lists of handed-on lanes live in vprime and jprime, which the product
+// analysis writes for every lane after the run.  A caller may have pointed
+// several outputs at one buffer: then no stage hands on.
+bool lists_usable(const DevBatch& b) {
+  const uintptr_t v = (uintptr_t)b.vprime, j = (uintptr_t)b.jprime, len = 8 * (uintptr_t)b.n;
+  if (!v || !j || (v & 7) || (j & 7)) return false;
+  auto apart = [&](const void* p, size_t size) {
+    const uintptr_t a = (uintptr_t)p, e = a + size * (uintptr_t)b.n;
+    return !a || ((e <= v || a >= v + len) && (e <= j || a >= j + len));
+  };
+  for (int k = 0; k < 12; ++k)
+    if (!apart(b.y[k], 8)) return false;
+  return (v + len <= j || j + len <= v) && apart(b.t, 8) && apart(b.h, 8) &&
+         apart(b.t_scale, 8) && apart(b.E0, 8) && apart(b.Ecol, 8) && apart(b.status, 1) &&
+         apart(b.nsteps, 4) && apart(b.nrej, 4) && apart(b.sys_id, 4);
+}
+
+template <bool MORSE>
+cudaError_t launch_stages(const SysSet& sys, const DevShape* shapes, const IntegParams& ip,
+                          const DevBatch& b, int variant, Ctx& ctx, cudaStream_t st) {
+  const int64_t sms = ctx.sm_count;
+  const bool lists = lists_usable(b);
+  int64_t bound = b.n;   // the most trajectories the next stage can meet
+  bool started = false;
+  StageQueue q;
+  for (int s = 0; s < kNumStages; ++s) {
+    const Stage& g = kStages[s];
+    const int64_t keep = g.keep_per_sm * sms;
+    if (g.lanes == 1 ? !(MORSE && lists && b.n >= kOneThreadMinPerSm * sms) : bound <= keep)
+      continue;
+    unsigned long long* c = ctx.counters + 4 + 4 * s;
+    q.head = c;
+    q.retired = c + 1;
+    q.n_out = c + 2;
+    q.list_out = reinterpret_cast<long long*>(s & 1 ? b.jprime : b.vprime);
+    q.keep = lists ? keep : 0;
+    cudaError_t e = cudaSuccess;
+    if (g.lanes == 1) {
+      e = launch_variant<MORSE>(variant, sys, shapes, ip, b, ctx.sm_count, ctx.counters, q, st);
+    } else {
+      if (!started) {
+        k_start_step<MORSE>
+            <<<(unsigned)((b.n + 127) / 128), 128, 0, st>>>(sys, ip, b, ctx.counters);
+        e = cudaGetLastError();
+      }
+      if (e == cudaSuccess)
+        e = launch_integrate_queue(sys, shapes, ip, b, g.lanes, bound, ctx.sm_count,
+                                   ctx.counters, q, st, MORSE);
+    }
+    if (e != cudaSuccess || q.keep == 0) return e;
+    started = true;
+    q.list_in = q.list_out;
+    q.n_in = q.n_out;
+    bound = keep < bound ? keep : bound;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace
+
 cudaError_t launch_integrate(const SysSet& sys, const DevShape* shapes, const IntegParams& ip,
                              const DevBatch& b, int precision, int persistent, int block,
                              int blocks_per_sm, Ctx& ctx, cudaStream_t st) {
   if (b.n == 0) return cudaSuccess;
-  cudaError_t e = cudaMemsetAsync(ctx.counters, 0, 2 * sizeof(unsigned long long), st);
+  cudaError_t e = cudaMemsetAsync(ctx.counters, 0, kCounters * sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
   const bool morse = all_morse(sys);
   if (precision == 32) return launch_integrate32(sys, shapes, ip, b, persistent, ctx, st, morse);
@@ -701,8 +850,8 @@ cudaError_t launch_integrate(const SysSet& sys, const DevShape* shapes, const In
                                     morse);
   const int v = find_variant(block, blocks_per_sm);
   if (v < 0) return cudaErrorInvalidValue;
-  return morse ? launch_variant<true>(v, sys, shapes, ip, b, persistent, ctx, st, nullptr)
-               : launch_variant<false>(v, sys, shapes, ip, b, persistent, ctx, st, nullptr);
+  return morse ? launch_stages<true>(sys, shapes, ip, b, v, ctx, st)
+               : launch_stages<false>(sys, shapes, ip, b, v, ctx, st);
 }
 
 int integrate_variant_count() { return kNumVariants; }

@@ -22,10 +22,10 @@ namespace qcams {
 namespace {
 
 // Scratch layout: shape table for QCAMS_NOALLOC_MAX_SYS systems x 3 pairs,
-// then 8 counters (0: rhs, 1: steps, 2: refill-queue head).
+// then the work counters (0: rhs, 1: steps, then the queues).
 constexpr size_t kShapeBytes = sizeof(DevShape) * QCAMS_NOALLOC_MAX_SYS * 3;
 constexpr size_t kCounterOffset = (kShapeBytes + 255) / 256 * 256;
-static_assert(kCounterOffset + 8 * sizeof(unsigned long long) <= QCAMS_NOALLOC_SCRATCH_BYTES,
+static_assert(kCounterOffset + kCounters * sizeof(unsigned long long) <= QCAMS_NOALLOC_SCRATCH_BYTES,
               "no-alloc scratch too small");
 // SysSet holds QCAMS_MAX_SYS systems and the shape kernel writes n_sys * 3
 // records: the no-alloc limit may not exceed the library's.

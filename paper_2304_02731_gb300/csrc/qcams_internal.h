@@ -20,7 +20,7 @@ struct Ctx {
   // were solved for (levels depend on nothing else)
   double level_key[QCAMS_MAX_SYS][9] = {};
   bool level_key_set[QCAMS_MAX_SYS] = {};
-  unsigned long long* counters = nullptr;  // [8]: 0 rhs, 1 steps, 2 queue head
+  unsigned long long* counters = nullptr;  // [kCounters]: 0 rhs, 1 steps, then queues
   qcams_level* req_out = nullptr;      // [65536] qcams_levels output staging
   int32_t* req_in = nullptr;           // [3 * 65536] qcams_levels input staging
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};  // integrate / analyze timing
@@ -60,6 +60,11 @@ cudaError_t launch_analyze(const SysSet& ss, const DevShape* shapes, double gb_s
 cudaError_t launch_integrate(const SysSet& sys, const DevShape* shapes, const IntegParams& ip,
                              const DevBatch& b, int precision, int persistent, int block,
                              int blocks_per_sm, Ctx& ctx, cudaStream_t st);
+// The FP64 persistent kernel of one launch shape alone, from first to last
+// lane (the autotuner's measurement).
+cudaError_t launch_integrate_shape(const SysSet& sys, const DevShape* shapes,
+                                   const IntegParams& ip, const DevBatch& b, int block,
+                                   int blocks_per_sm, Ctx& ctx, cudaStream_t st);
 
 // FP64 integrator for small batches, `lanes` = 3 or 6 lanes per trajectory
 // (integrate_grp.cu).
@@ -67,6 +72,41 @@ cudaError_t launch_integrate_grouped(const SysSet& sys, const DevShape* shapes,
                                      const IntegParams& ip, const DevBatch& b, int lanes,
                                      unsigned long long* counters, cudaStream_t st,
                                      bool all_morse);
+
+// One stage of an FP64 run: its source of trajectories (all lanes of the
+// batch, or a list of lane indices that an earlier stage handed on), the
+// progress counters in device memory, and the list it hands on.  A stage
+// that has used up its source and has at most `keep` unfinished
+// trajectories (0: runs to the end) stores them between two attempts, with
+// P / mu in y[6..11] and kHandoff in the status, and ends.
+struct StageQueue {
+  const long long* list_in = nullptr;
+  const unsigned long long* n_in = nullptr;   // length of list_in
+  unsigned long long* head = nullptr;         // next source entry to take
+  unsigned long long* retired = nullptr;      // trajectories finished in this stage
+  long long* list_out = nullptr;
+  unsigned long long* n_out = nullptr;
+  long long keep = 0;
+};
+// Whether a stage with n source entries hands on now (same in all lanes).
+__device__ __forceinline__ bool stage_over(const StageQueue& q, long long n, int lane) {
+  int over = 0;
+  if (lane == 0)
+    over = (long long)*(volatile unsigned long long*)q.head >= n &&
+           n - (long long)*(volatile unsigned long long*)q.retired <= q.keep;
+  return __shfl_sync(0xffffffffu, over, 0) != 0;
+}
+// Lane status bits of a handed-on trajectory (never seen by a caller).
+constexpr int kHandoff = 0x40, kHandoffRejected = 0x80;
+constexpr int kCounters = 32;   // work counters of one run
+
+// `lanes` = 3 or 6 lanes per trajectory, bit for bit the one-thread kernels'
+// results (integrate_grp.cu); at most n_max trajectories in the source, all
+// with a starting step (b.h > 0).
+cudaError_t launch_integrate_queue(const SysSet& sys, const DevShape* shapes,
+                                   const IntegParams& ip, const DevBatch& b, int lanes,
+                                   int64_t n_max, int sm_count, unsigned long long* counters,
+                                   const StageQueue& q, cudaStream_t st, bool all_morse);
 
 // Registers per thread and resident blocks per SM of the lane-group kernel.
 cudaError_t grouped_func_info(int lanes, bool all_morse, int* regs, int* blocks_per_sm);
