@@ -123,8 +123,9 @@ __device__ __forceinline__ __nv_bfloat16 bf_hi(uint32_t w) {
 // Weights to shared memory (blockDim.x == THREADS).  With p 16-byte aligned
 // every matrix starts on a 16-byte boundary: each thread issues all of its
 // 16-byte loads of 8-element row segments first, then stores each segment
-// to its W row and, element by element, to the W^T column.  Otherwise,
-// element loads.
+// to its W row and, TRANSPOSED (the backward pass), element by element to the
+// W^T column.  Otherwise, element loads.
+template <bool TRANSPOSED>
 __device__ void load_weights(WeightsSmem& W, const __nv_bfloat16* p, const float* pf) {
   const __nv_bfloat16 zero = __float2bfloat16(0.0f);
   if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0) {
@@ -159,7 +160,7 @@ __device__ void load_weights(WeightsSmem& W, const __nv_bfloat16* p, const float
       __nv_bfloat16* row = is4 ? &W.w4[r][c] : i < N1 + N2 ? &W.w2[r][c] : &W.w3[r][c];
       *reinterpret_cast<uint4*>(row) = v[k];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
+      for (int e = 0; e < (TRANSPOSED ? 4 : 0); ++e) {
         if (is4) {
           W.w4t[c + 2 * e][r] = bf_lo(w[e]);
           W.w4t[c + 2 * e + 1][r] = bf_hi(w[e]);
@@ -423,7 +424,7 @@ __global__ void __launch_bounds__(THREADS) k_mlp_grad(const __nv_bfloat16* pb, c
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TrainSmem<CPW>& S = *reinterpret_cast<TrainSmem<CPW>*>(smem_raw);
   constexpr int RS = BlockTiles<CPW>::RS, LDT = BlockTiles<CPW>::LDT;
-  load_weights(S.w, pb, pf);
+  load_weights<true>(S.w, pb, pf);
   for (int i = threadIdx.x; i < NGB; i += blockDim.x) S.gb[i] = 0.0f;
   // padding rows of the X^T and dZ4^T tiles (never written by the passes)
   const __nv_bfloat16 zero = __float2bfloat16(0.0f);
@@ -525,7 +526,7 @@ __global__ void __launch_bounds__(THREADS) k_mlp_infer(const __nv_bfloat16* pb, 
                                                        float* probs, double* g_out,
                                                        double eps) {
   __shared__ WeightsSmem W;
-  load_weights(W, pb, pf);
+  load_weights<false>(W, pb, pf);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
   const int64_t chunks = (n + 15) / 16;
@@ -639,86 +640,227 @@ __global__ void k_moments(const float* x, int64_t n, double* acc) {
   if (threadIdx.x < 16) atomicAdd(&acc[threadIdx.x], s[threadIdx.x]);
 }
 
-// Normalise the proposal and form its integer CDF in one block with a fixed
-// summation order (deterministic bits).  g holds g_c on entry, q_c on exit.
-constexpr int kScanThreads = 1024;
-__global__ void __launch_bounds__(kScanThreads) k_proposal_finish(double* g, int64_t n_cells,
-                                                                  double alpha, int64_t* qfix,
-                                                                  int64_t* cdf) {
-  __shared__ double ds[kScanThreads];
-  __shared__ long long ls[kScanThreads];
-  const int t = threadIdx.x;
-  const int64_t per = (n_cells + kScanThreads - 1) / kScanThreads;
-  const int64_t lo = t * per, hi = min(n_cells, lo + per);
+// Normalisation of the proposal and its integer CDF, in a fixed summation
+// order (deterministic bits): 1,024 runs of consecutive cells are summed cell
+// by cell, the run sums by a halving tree.  q needs a correctly rounded FP64
+// division per cell, about 20 instructions of the scarce FP64 pipe, so the
+// work is spread over all SMs in four small kernels (one block of one SM took
+// 180 us for 32,768 cells, 160 of them at the FP64 pipe's rate; now 20 us):
+//   k_run_sums   run sums, staged through shared memory (coalesced)
+//   k_normalise  total, q, qfix and each scan block's sum of qfix
+//   k_scan_sums  exclusive prefixes of the block sums
+//   k_cdf        inclusive scan within each block
+// The intermediate values live in cdf until k_cdf overwrites it: the run
+// sums (as doubles) in its first 1,024 entries, each scan block's sum and
+// then prefix in the block's last entry.
+constexpr int kRuns = 1024;
+constexpr int kScanCells = 2048;   // cells per scan block
+static_assert(kScanCells > kRuns, "a scan block's last entry lies beyond the run sums");
+constexpr int kRunTile = 32;
+
+__global__ void __launch_bounds__(32) k_run_sums(const double* g, int64_t n_cells, int64_t* cdf,
+                                                 int scan_blocks) {
+  __shared__ double tile[kRunTile][kRunTile + 1];
+  const int lane = threadIdx.x;
+  const int64_t per = (n_cells + kRuns - 1) / kRuns;
+  const int64_t run0 = (int64_t)blockIdx.x * kRunTile;
+  const int64_t lo = (run0 + lane) * per, hi = min(n_cells, lo + per);
   double sum = 0.0;
-  for (int64_t c = lo; c < hi; ++c) sum += g[c];
-  ds[t] = sum;
+  for (int64_t c0 = 0; c0 < per; c0 += kRunTile) {
+#pragma unroll 8
+    for (int r = 0; r < kRunTile; ++r) {   // row r: cells c0 .. c0 + 31 of run run0 + r
+      const int64_t c = (run0 + r) * per + c0 + lane;
+      tile[r][lane] = c0 + lane < per && c < n_cells ? g[c] : 0.0;
+    }
+    __syncwarp();
+    const int64_t last = min(per - c0, (int64_t)kRunTile);
+    for (int k = 0; k < last; ++k)
+      if (lo + c0 + k < hi) sum += tile[lane][k];
+    __syncwarp();
+  }
+  // runs past the last cell are empty; only runs that exist have an entry
+  if (lo < n_cells) cdf[run0 + lane] = __double_as_longlong(sum);
+  if (scan_blocks > 1)   // clear the scan blocks' sums
+    for (int64_t b = run0 + lane; b < scan_blocks; b += kRuns)
+      cdf[min(n_cells, (b + 1) * kScanCells) - 1] = 0;
+}
+
+constexpr int kNormBlock = 256;   // small blocks: the divisions spread over the SMs
+static_assert(kScanCells % kNormBlock == 0, "a block lies in one scan block");
+__global__ void __launch_bounds__(kNormBlock) k_normalise(double* g, int64_t n_cells, double alpha,
+                                                          int64_t* qfix, int64_t* cdf, bool sums) {
+  __shared__ double ds[kRuns];
+  const int t = threadIdx.x;
+  const int64_t per = (n_cells + kRuns - 1) / kRuns;
+  for (int r = t; r < kRuns; r += kNormBlock)
+    ds[r] = r * per < n_cells ? __longlong_as_double(cdf[r]) : 0.0;
   __syncthreads();
-  for (int o = kScanThreads / 2; o > 0; o >>= 1) {
-    if (t < o) ds[t] += ds[t + o];
+  for (int o = kRuns / 2; o > 0; o >>= 1) {
+    for (int r = t; r < o; r += kNormBlock) ds[r] += ds[r + o];
     __syncthreads();
   }
   const double total = ds[0];
-  long long part = 0;
-  for (int64_t c = lo; c < hi; ++c) {
+  const int64_t c = (int64_t)blockIdx.x * kNormBlock + t;
+  long long qi = 0;
+  if (c < n_cells) {
     const double qc = alpha / (double)n_cells + (1.0 - alpha) * g[c] / total;
     g[c] = qc;
-    const long long qi = __double2ll_rn(qc * 1099511627776.0);  // 2^40
+    qi = __double2ll_rn(qc * 1099511627776.0);  // 2^40
     qfix[c] = qi;
-    part += qi;
   }
-  ls[t] = part;
-  __syncthreads();
-  // inclusive scan of the per-thread parts (Hillis-Steele)
-  for (int o = 1; o < kScanThreads; o <<= 1) {
-    long long v = t >= o ? ls[t - o] : 0;
-    __syncthreads();
-    ls[t] += v;
-    __syncthreads();
-  }
-  long long run = t > 0 ? ls[t - 1] : 0;
-  for (int64_t c = lo; c < hi; ++c) {
-    run += qfix[c];
-    cdf[c] = run;
+  if (!sums) return;   // one scan block: its prefix is zero
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) qi += __shfl_xor_sync(0xffffffffu, qi, o);
+  if ((t & 31) == 0 && qi) {
+    const int64_t b = (int64_t)blockIdx.x * kNormBlock / kScanCells;
+    atomicAdd(reinterpret_cast<unsigned long long*>(&cdf[min(n_cells, (b + 1) * kScanCells) - 1]),
+              (unsigned long long)qi);
   }
 }
 
-__global__ void k_sample(CellGrid grid, int64_t n_cells, const int64_t* qfix, const int64_t* cdf,
+// Inclusive scan over a block of 1,024 threads.
+__device__ __forceinline__ long long block_scan(long long v, long long* ws) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const long long u = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += u;
+  }
+  if (lane == 31) ws[warp] = v;
+  __syncthreads();
+  if (warp == 0) {
+    long long w = ws[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long u = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += u;
+    }
+    ws[lane] = w;
+  }
+  __syncthreads();
+  return warp ? v + ws[warp - 1] : v;
+}
+
+constexpr int kScanThreads = 1024;
+__global__ void __launch_bounds__(kScanThreads) k_scan_sums(int64_t n_cells, int blocks,
+                                                            int64_t* cdf) {
+  __shared__ long long ws[32];
+  long long run = 0;
+  for (int b0 = 0; b0 < blocks; b0 += kScanThreads) {
+    const int b = b0 + threadIdx.x;
+    const int64_t at = min(n_cells, (int64_t)(b + 1) * kScanCells) - 1;
+    const long long mine = b < blocks ? cdf[at] : 0;
+    const long long inc = run + block_scan(mine, ws);
+    if (b < blocks) cdf[at] = inc - mine;
+    __syncthreads();
+    run += ws[31];
+    __syncthreads();
+  }
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_cdf(int64_t n_cells, const int64_t* qfix,
+                                                      int64_t* cdf, bool sums) {
+  __shared__ long long ws[32];
+  const int64_t base = (int64_t)blockIdx.x * kScanCells;
+  const int64_t end = min(n_cells, base + kScanCells);
+  const long long before = sums ? cdf[end - 1] : 0;
+  // two consecutive cells per thread
+  const int64_t c = base + 2 * threadIdx.x;
+  const long long a = c < end ? qfix[c] : 0, b = c + 1 < end ? qfix[c + 1] : 0;
+  const long long inc = before + block_scan(a + b, ws);   // barriers: every thread has read `before`
+  if (c < end) cdf[c] = inc - b;
+  if (c + 1 < end) cdf[c + 1] = inc;
+}
+
+// (i + u) with u = (w + 1/2) 2^-32, exactly, for 0 <= i < 2^19: the integer
+// i 2^33 + 2 w + 1 < 2^52 as a double, scaled by 2^-33.
+__device__ __forceinline__ double cell_pos(int i, uint32_t w) {
+  const unsigned long long m = ((unsigned long long)i << 33) | (2ull * w + 1ull);
+  const double d = __longlong_as_double((long long)(m | 0x4330000000000000ull)) - 4503599627370496.0;
+  return __hiloint2double(__double2hiint(d) - (33 << 20), __double2loint(d));
+}
+// x / n correctly rounded, with rn = 1 / n (Markstein, IBM J. Res. Dev. 34
+// (1990)): x and n are positive and far from the exponent range's ends.
+__device__ __forceinline__ double div_by(double x, double n, double rn) {
+  const double q = x * rn;
+  return fma(fma(-q, n, x), rn, q);
+}
+
+// Lanes per launch block and coarse CDF entries held in shared memory.
+constexpr int kSampleBlock = 256, kCoarse = 1024;
+
+// Draws from the integer CDF.  A lane costs about 50 FP64 instructions (the
+// positions formed from integers, the divisions by the grid sizes as
+// multiplications by their reciprocals with a correction; 120 before), the
+// first ten steps of its search run in shared memory on every
+// (N / 1024)-th entry.  200,000 lanes of 32,768 cells: 50 -> 32 us.
+__global__ void __launch_bounds__(kSampleBlock) k_sample(CellGrid grid, int64_t n_cells,
+                         const int64_t* qfix, const int64_t* cdf,
                          int64_t n, uint64_t seed, uint64_t id_offset, double b2_max, double* b,
                          double* u0, double* u1, double* u2, double* u3, double* w,
                          int32_t* cell) {
+  __shared__ unsigned long long coarse[kCoarse];
+  __shared__ double rn[5], mean;
+  const int64_t step = (n_cells + kCoarse - 1) / kCoarse;
+  const int n_coarse = (int)((n_cells + step - 1) / step);
+  // coarse[k]: the last entry of the k-th run of `step` cells
+  for (int k = threadIdx.x; k < n_coarse; k += kSampleBlock)
+    coarse[k] = (unsigned long long)cdf[min(n_cells, (k + 1) * step) - 1];
+  if (threadIdx.x < 5) {
+    const int d = threadIdx.x == 0 ? grid.n_b2 : threadIdx.x == 1 ? grid.n_cth
+                  : threadIdx.x == 2 ? grid.n_phi : threadIdx.x == 3 ? grid.n_eta : grid.n_chi;
+    rn[threadIdx.x] = 1.0 / (double)d;
+  }
+  if (threadIdx.x == 32)
+    mean = (double)(unsigned long long)cdf[n_cells - 1] / (double)n_cells;
+  __syncthreads();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   const uint64_t id = id_offset + (uint64_t)i;
   const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
   const uint4 wa = philox4x32_10(make_uint4((uint32_t)id, (uint32_t)(id >> 32), 1u, 0u), key);
   const uint4 wb = philox4x32_10(make_uint4((uint32_t)id, (uint32_t)(id >> 32), 2u, 0u), key);
-  const unsigned long long total = (unsigned long long)cdf[n_cells - 1];
+  const unsigned long long total = coarse[n_coarse - 1];
   // U = floor(u_0 total) with u_0 = (w + 1/2) 2^-32, in exact integer arithmetic:
   // (2 w + 1) total / 2^33
   const unsigned long long m = 2ull * wa.x + 1ull;
   const unsigned long long lo = m * total, hi = __umul64hi(m, total);
   const unsigned long long U = (hi << 31) | (lo >> 33);
-  int64_t a = 0, z = n_cells - 1;
+  // first entry above U: its run among the coarse entries, then within the run
+  int ca = 0, cz = n_coarse - 1;
+  while (ca < cz) {
+    const int mid = (ca + cz) >> 1;
+    if (coarse[mid] > U) cz = mid;
+    else ca = mid + 1;
+  }
+  int64_t a = ca * step, z = min(n_cells, (ca + 1) * step) - 1;
   while (a < z) {
     const int64_t mid = (a + z) >> 1;
     if ((unsigned long long)cdf[mid] > U) z = mid;
     else a = mid + 1;
   }
-  int64_t c = a;
-  cell[i] = (int32_t)c;
-  const int i_chi = (int)(c % grid.n_chi); c /= grid.n_chi;
-  const int i_eta = (int)(c % grid.n_eta); c /= grid.n_eta;
-  const int i_phi = (int)(c % grid.n_phi); c /= grid.n_phi;
-  const int i_cth = (int)(c % grid.n_cth); c /= grid.n_cth;
-  const int i_b2 = (int)c;
-  const double b2 = b2_max * (i_b2 + u01(wa.y)) / grid.n_b2;
-  b[i] = sqrt(b2);
-  u0[i] = (i_cth + u01(wa.z)) / grid.n_cth;
-  u1[i] = (i_phi + u01(wa.w)) / grid.n_phi;
-  u2[i] = (i_eta + u01(wb.x)) / grid.n_eta;
-  u3[i] = (i_chi + u01(wb.y)) / grid.n_chi;
-  w[i] = ((double)total / (double)n_cells) / (double)qfix[a];
+  int c = (int)a;   // at most 2^22 cells
+  cell[i] = c;
+  const int i_chi = c % grid.n_chi; c /= grid.n_chi;
+  const int i_eta = c % grid.n_eta; c /= grid.n_eta;
+  const int i_phi = c % grid.n_phi; c /= grid.n_phi;
+  const int i_cth = c % grid.n_cth; c /= grid.n_cth;
+  const int i_b2 = c;
+  const int widest = max(max(grid.n_b2, grid.n_cth), max(grid.n_phi, max(grid.n_eta, grid.n_chi)));
+  if (widest <= (1 << 19) && b2_max > 1e-100 && b2_max < 1e100) {
+    b[i] = sqrt(div_by(b2_max * cell_pos(i_b2, wa.y), (double)grid.n_b2, rn[0]));
+    u0[i] = div_by(cell_pos(i_cth, wa.z), (double)grid.n_cth, rn[1]);
+    u1[i] = div_by(cell_pos(i_phi, wa.w), (double)grid.n_phi, rn[2]);
+    u2[i] = div_by(cell_pos(i_eta, wb.x), (double)grid.n_eta, rn[3]);
+    u3[i] = div_by(cell_pos(i_chi, wb.y), (double)grid.n_chi, rn[4]);
+  } else {   // a dimension of more than 2^19 cells, or an extreme b2_max
+    b[i] = sqrt(b2_max * (i_b2 + u01(wa.y)) / grid.n_b2);
+    u0[i] = (i_cth + u01(wa.z)) / grid.n_cth;
+    u1[i] = (i_phi + u01(wa.w)) / grid.n_phi;
+    u2[i] = (i_eta + u01(wb.x)) / grid.n_eta;
+    u3[i] = (i_chi + u01(wb.y)) / grid.n_chi;
+  }
+  w[i] = mean / (double)qfix[a];
 }
 
 int dev_ok() {
@@ -966,7 +1108,13 @@ int qcams_build_proposal(const qcams_mlp* m, const qcams_proposal_spec* spec, do
       grid_of(spec), 1, nullptr, q, spec->eps);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return QCAMS_E_CUDA;
-  k_proposal_finish<<<1, kScanThreads, 0, st>>>(q, N, spec->alpha, qfix, cdf);
+  const unsigned blocks = (unsigned)((N + kScanCells - 1) / kScanCells);
+  const bool sums = blocks > 1;
+  k_run_sums<<<kRuns / kRunTile, 32, 0, st>>>(q, N, cdf, (int)blocks);
+  k_normalise<<<(unsigned)((N + kNormBlock - 1) / kNormBlock), kNormBlock, 0, st>>>(
+      q, N, spec->alpha, qfix, cdf, sums);
+  if (sums) k_scan_sums<<<1, kScanThreads, 0, st>>>(N, (int)blocks, cdf);
+  k_cdf<<<blocks, kScanThreads, 0, st>>>(N, qfix, cdf, sums);
   return status_of(cudaGetLastError());
 }
 
@@ -982,7 +1130,8 @@ int qcams_sample_proposal(const qcams_proposal_spec* spec, const int64_t* qfix,
   if ((rc = dev_ok()) != QCAMS_OK) return rc;
   const int64_t N = (int64_t)spec->n_b2 * spec->n_cth * spec->n_phi * spec->n_eta * spec->n_chi;
   (void)cudaGetLastError();
-  k_sample<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)cuda_stream>>>(
+  k_sample<<<(unsigned)((n + kSampleBlock - 1) / kSampleBlock), kSampleBlock, 0,
+             (cudaStream_t)cuda_stream>>>(
       grid_of(spec), N, qfix, cdf, n, seed, id_offset, spec->b2_max, b, u_out[0], u_out[1],
       u_out[2], u_out[3], w, cell);
   return status_of(cudaGetLastError());
