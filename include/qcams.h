@@ -326,8 +326,8 @@ typedef struct {
  * the lanes' (cls, v_t, j_t, W, isw) per cell, flushed with int64 atomics
  * into hist_out (device, n_cells * QCAMS_H_STRIDE int64, zeroed by this
  * call).  Lanes with a cell outside [0, n_cells) are ignored.
- * If xsec_out (host) is non-NULL the call synchronises the stream, copies
- * the histograms back and writes, in doubles, with E = QCAMS_XSEC_ENTRIES
+ * If xsec_out (host) is non-NULL the call synchronises the stream, brings
+ * the counts and weight sums back and writes, in doubles, with E = QCAMS_XSEC_ENTRIES
  * entries per cell and per group (k = 0..5 the classes, k = 6 the reactive
  * total R_AC + R_BC):
  *   per cell c, entry k:  xsec_out[2E c + 2 k] = P_k = N_k / N,

@@ -244,62 +244,141 @@ DevBatch dev_batch(const qcams_batch* b) {
 
 // ---------------------------------------------------------------------------
 // Potential shapes (once per call): well bottom r_eq, Buckingham short-range
-// maximum r_b, and the maximum of g(r) = r^3 V'(r) beyond r_eq.
+// maximum r_b, and the maximum of g(r) = r^3 V'(r) beyond r_eq.  One block
+// per pair.  Its chains are short and latency-bound (an FP64 instruction
+// takes 64 cycles with one lane or 32), so what can be evaluated ahead is:
+// the Buckingham scan's 4,096 points all at once, its two roots in two
+// lanes, the bracket's points in one go, and the golden section five
+// iterations at a time, lane by lane over the 31 points its next five
+// comparisons can lead to.  Every value compared is the serial search's, so
+// the result is too.  H2 + Ca with Buckingham Ca-H: 4,834 -> 178 us, with
+// Morse 87 -> 50 us.
 // ---------------------------------------------------------------------------
-__device__ DevShape pair_shape(const DevPair& q) {
+constexpr int kShapeBlock = 512;
+constexpr int kScanPts = 4096;
+
+// First index k in [from, kScanPts] for which cond(k) holds, over the block.
+template <class C>
+__device__ int block_first(int from, int* best, C cond) {
+  if (threadIdx.x == 0) *best = kScanPts + 1;
+  __syncthreads();
+  for (int k = from + (int)threadIdx.x; k <= kScanPts; k += kShapeBlock)
+    if (cond(k)) {
+      atomicMin(best, k);
+      break;
+    }
+  __syncthreads();
+  const int r = *best;
+  __syncthreads();
+  return r;
+}
+
+// Golden-section state and one step of it with a known new function value.
+struct Golden {
+  double a, b, x1, x2;
+  // moves to the side the comparison chose; returns the point to evaluate
+  __device__ __forceinline__ double move(bool right) {
+    const double gr = 0.6180339887498949;
+    if (right) { a = x1; x1 = x2; x2 = a + gr * (b - a); return x2; }
+    b = x2; x2 = x1; x1 = b - gr * (b - a);
+    return x1;
+  }
+  __device__ __forceinline__ bool open() const { return (b - a) > 1e-12 * b; }
+};
+
+// Bracket and golden section by one warp, from the well bottom r_eq.
+__device__ void shape_peak(const DevPair& q, DevShape& sh) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  // bracket the maximum of g beyond r_eq by geometric steps, then golden
+  // section (g is unimodal on (r_eq, inf) for the three potential kinds)
+  Golden G;
+  double a = sh.r_eq, m = sh.r_eq * 1.5, b = m * 1.5;
+  {
+    double x = m;   // lane l: the point r_eq 1.5^(l + 1)
+    for (int k = 0; k < 31; ++k) x = k < lane ? x * 1.5 : x;
+    const double g = gfun(q, x), gn = __shfl_down_sync(full, g, 1);
+    const unsigned stop = __ballot_sync(full, lane < 31 && !(gn >= g));
+    const int k = stop ? __ffs(stop) - 1 : 30;   // the step that ends the search
+    const double xk = __shfl_sync(full, x, k), xp = __shfl_sync(full, x, k > 0 ? k - 1 : 0);
+    a = k > 0 ? xp : a;
+    m = xk;
+    b = __shfl_sync(full, x, k + 1);
+    if (!stop) {
+      double gm = __shfl_sync(full, g, 30), gb = __shfl_sync(full, g, 31);
+      for (int it = 30; it < 200 && gb >= gm; ++it) {
+        a = m; m = b; gm = gb;
+        b = m * 1.5;
+        gb = gfun(q, b);
+      }
+    }
+  }
+  const double gr = 0.6180339887498949;
+  G.a = a;
+  G.b = b;
+  G.x1 = b - gr * (b - a);
+  G.x2 = a + gr * (b - a);
+  const double fi = gfun(q, (lane & 1) ? G.x2 : G.x1);
+  double f1 = __shfl_sync(full, fi, 0), f2 = __shfl_sync(full, fi, 1);
+  // lane 2^d - 1 + p evaluates the point of step d + 1 that the comparisons
+  // p (first one in the highest of d bits) after the known first lead to
+  const int depth = 31 - __clz(lane + 1), path = lane + 1 - (1 << depth);
+  for (int it = 0; it < 200 && G.open();) {
+    Golden H = G;
+    double x = H.move(f1 < f2);
+    for (int d = 1; d <= depth; ++d)
+      if (lane < 31) x = H.move((path >> (depth - d)) & 1);
+    const double f = gfun(q, x);
+    int at = 0;   // lane holding the next value
+    for (int d = 0; d < 5 && it < 200 && G.open(); ++d, ++it) {
+      const double fn = __shfl_sync(full, f, at);
+      const bool right = f1 < f2;
+      G.move(right);
+      if (right) { f1 = f2; f2 = fn; }
+      else { f2 = f1; f1 = fn; }
+      at = 2 * at + 1 + (f1 < f2 ? 1 : 0);
+    }
+  }
+  sh.r_peak = 0.5 * (G.a + G.b);
+  sh.g_max = gfun(q, sh.r_peak);
+  sh.ok = (sh.g_max > 0.0 && sh.r_eq > 0.0) ? 1 : 0;
+}
+
+__global__ void __launch_bounds__(kShapeBlock) k_pair_shapes(SysSet sys, DevShape* out) {
+  __shared__ double dv[kScanPts + 1];
+  __shared__ int best;
+  const DevPair& q = sys.s[blockIdx.x / 3].pair[blockIdx.x % 3];
   DevShape sh{};
   sh.ok = 0;
+  bool found = true;
   if (q.kind == QCAMS_MORSE) {
     sh.r_eq = q.p[1];
   } else if (q.kind == QCAMS_LJ) {
-    sh.r_eq = pow(q.c2 / q.c3, 1.0 / (q.m - q.n));
+    if (threadIdx.x < 32) sh.r_eq = pow(q.c2 / q.c3, 1.0 / (q.m - q.n));
   } else {
     // Buckingham: V' > 0 at short range (collapse side), then the maximum
     // r_b (V' from + to -), then the well bottom r_eq (V' from - to +).
     // Scan a logarithmic grid over [0.02, 200] bohr for the two changes.
-    const int N = 4096;
-    const double lo = 0.02, hi = 200.0, dl = log(hi / lo) / N;
-    double pr = lo, pv = pot_dV(q, lo);
-    double rb_a = 0, rb_b = 0, re_a = 0, re_b = 0;
-    bool got_b = false, got_e = false;
-    for (int k = 1; k <= N && !got_e; ++k) {
-      double r = lo * exp(dl * k), dv = pot_dV(q, r);
-      if (!got_b && pv > 0 && dv <= 0) { got_b = true; rb_a = pr; rb_b = r; }
-      else if (got_b && pv < 0 && dv >= 0) { got_e = true; re_a = pr; re_b = r; }
-      pr = r; pv = dv;
+    const double lo = 0.02, hi = 200.0, dl = log(hi / lo) / kScanPts;
+    auto point = [&](int k) { return k == 0 ? lo : lo * exp(dl * k); };
+    for (int k = threadIdx.x; k <= kScanPts; k += kShapeBlock) dv[k] = pot_dV(q, point(k));
+    __syncthreads();
+    const int kb = block_first(1, &best, [&](int k) { return dv[k - 1] > 0 && dv[k] <= 0; });
+    const int ke = block_first(kb + 1, &best, [&](int k) { return dv[k - 1] < 0 && dv[k] >= 0; });
+    found = kb <= kScanPts && ke <= kScanPts;
+    if (found && threadIdx.x < 32) {
+      auto f = [&](double r) { return pot_dV(q, r); };
+      const int k = (threadIdx.x & 1) ? ke : kb;
+      const double ra = point(k - 1), rb = point(k);
+      const double root = illinois(f, ra, rb, f(ra), f(rb));
+      sh.r_b = __shfl_sync(0xffffffffu, root, 0);
+      sh.r_b2 = sh.r_b * sh.r_b;
+      sh.r_eq = __shfl_sync(0xffffffffu, root, 1);
     }
-    if (!got_b || !got_e) return sh;
-    auto f = [&](double r) { return pot_dV(q, r); };
-    sh.r_b = illinois(f, rb_a, rb_b, f(rb_a), f(rb_b));
-    sh.r_b2 = sh.r_b * sh.r_b;
-    sh.r_eq = illinois(f, re_a, re_b, f(re_a), f(re_b));
   }
-  // bracket the maximum of g beyond r_eq by geometric steps, then golden
-  // section (g is unimodal on (r_eq, inf) for the three potential kinds)
-  double a = sh.r_eq, m = sh.r_eq * 1.5, b = m * 1.5;
-  double gm = gfun(q, m), gb = gfun(q, b);
-  for (int it = 0; it < 200 && gb >= gm; ++it) {
-    a = m; m = b; gm = gb;
-    b = m * 1.5;
-    gb = gfun(q, b);
-  }
-  const double gr = 0.6180339887498949;
-  double x1 = b - gr * (b - a), x2 = a + gr * (b - a);
-  double f1 = gfun(q, x1), f2 = gfun(q, x2);
-  for (int it = 0; it < 200 && (b - a) > 1e-12 * b; ++it) {
-    if (f1 < f2) { a = x1; x1 = x2; f1 = f2; x2 = a + gr * (b - a); f2 = gfun(q, x2); }
-    else { b = x2; x2 = x1; f2 = f1; x1 = b - gr * (b - a); f1 = gfun(q, x1); }
-  }
-  sh.r_peak = 0.5 * (a + b);
-  sh.g_max = gfun(q, sh.r_peak);
-  sh.ok = (sh.g_max > 0.0 && sh.r_eq > 0.0) ? 1 : 0;
-  return sh;
-}
-
-__global__ void k_pair_shapes(SysSet sys, DevShape* out) {
-  int t = threadIdx.x;
-  if (t >= sys.n * 3) return;
-  out[t] = pair_shape(sys.s[t / 3].pair[t % 3]);
+  if (threadIdx.x >= 32) return;
+  if (found) shape_peak(q, sh);
+  if (threadIdx.x == 0) out[blockIdx.x] = sh;
 }
 
 // Bohr-Sommerfeld level: solve v(E) = -1/2 + sqrt(2 mu)/pi I_act(E) = v by a
@@ -349,6 +428,236 @@ __device__ DevLevel solve_level(const DevPair& q, const DevShape& sh, double mu,
   return L;
 }
 
+// ---------------------------------------------------------------------------
+// The levels a caller asks for by number (qcams_levels): the same equation,
+// one block of 128 threads per level.  The first warp iterates, its even and
+// odd lanes on the inner and the outer root of each pair of searches, and a
+// Newton iteration from the last energy's turning points takes 2-4
+// evaluations where the serial solver's bracketing takes about 15; each of the 128
+// quadrature points has a thread.  What bounds it is the first warp's chain
+// of FP64 instructions (64 cycles each).  Its levels equal the serial solver's to
+// rounding but not to the last bit, and a last bit of r_plus or tau would
+// change every chaotic trajectory that starts there: the table behind the
+// initial conditions, solved once per molecule, keeps solve_level.
+// 231 levels of one molecule, with the copies: 16.1 ms with one thread per
+// level, 3.5 ms with one block per level and bracketing, now 0.52 ms.
+constexpr int kLevelBlock = kGL128;
+struct LevelSmem {
+  double sum[kLevelBlock / 32][2];
+  double E, c, d;
+  int more;
+};
+
+// V and V' of a pair in one evaluation (Morse without the cancellation of
+// De (1 - x)^2 - De at large r, where high levels have their outer ends).
+__device__ __forceinline__ void pot_VdV(const DevPair& q, double r, double* V, double* dV) {
+  if (q.kind == QCAMS_MORSE) {
+    const double x = exp(q.c1 - q.c0 * r);
+    *V = q.c3 * (x * (x - 2.0));
+    *dV = q.c2 * x * (1.0 - x);
+    return;
+  }
+  const double ri = 1.0 / r;
+  if (q.kind == QCAMS_LJ) {
+    const double rm = ipow(ri, q.m), rn = ipow(ri, q.n);
+    *V = q.c0 * rm - q.c1 * rn;
+    *dV = (q.c3 * rn - q.c2 * rm) * ri;
+  } else {
+    const double ex = exp(-q.c1 * r), ri2 = ri * ri, ri6 = ri2 * ri2 * ri2;
+    *V = q.c0 * ex - q.c4 * ri6;
+    *dV = q.c3 * ri6 * ri - q.c2 * ex;
+  }
+}
+
+// The block's share of the action and period sums: one point per thread,
+// summed over each warp.
+__device__ __forceinline__ void level_points(const DevPair& q, double a, LevelSmem& S) {
+  const int k = threadIdx.x >> 1;
+  const double sn = kGL128S[k], w = kGL128WC[k], c = S.c, d = S.d;
+  const double r = (threadIdx.x & 1) ? fma(-d, sn, c) : fma(d, sn, c);
+  const double ri = rsqrt(r * r);   // 1/r and sqrt(g) from reciprocal square roots
+  double V, dV;
+  pot_VdV(q, r, &V, &dV);
+  const double g = S.E - (V + a * (ri * ri));
+  double sa = 0.0, sp = 0.0;
+  if (g > 0.0) {
+    const double rg = rsqrt(g);
+    sa = w * (g * rg);
+    sp = w * rg;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    sa += __shfl_xor_sync(0xffffffffu, sa, o);
+    sp += __shfl_xor_sync(0xffffffffu, sp, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    S.sum[threadIdx.x >> 5][0] = sa;
+    S.sum[threadIdx.x >> 5][1] = sp;
+  }
+}
+
+// Action and period integrals at E between rm and rp, for the first warp.
+__device__ __forceinline__ void level_integrals(const DevPair& q, double a, double E, double rm,
+                                                double rp, LevelSmem& S, double* act,
+                                                double* per) {
+  const double c = 0.5 * (rp + rm), d = 0.5 * (rp - rm);
+  if (threadIdx.x == 0) {
+    S.E = E;
+    S.c = c;
+    S.d = d;
+    S.more = 1;
+  }
+  __syncthreads();
+  level_points(q, a, S);
+  __syncthreads();
+  const int k = threadIdx.x & 1;
+  const double s = (S.sum[0][k] + S.sum[1][k]) + (S.sum[2][k] + S.sum[3][k]);
+  *act = 0.5 * kPi * d * __shfl_sync(0xffffffffu, s, 0);
+  *per = 0.5 * kPi * d * __shfl_sync(0xffffffffu, s, 1);
+}
+
+// Well of the effective potential by one warp (eff_well's searches, the
+// barrier's root in the even lanes and the bottom's in the odd ones).
+__device__ bool warp_well(const DevPair& q, const DevShape& sh, double mu, double L2,
+                          double* r_min, double* r_top, double* thr) {
+  *r_top = INFINITY;
+  *thr = 0.0;
+  *r_min = sh.r_eq;
+  if (L2 <= 0.0) return true;
+  const double c = L2 / mu;
+  if (!(c < sh.g_max)) return false;
+  auto G = [&](double r) { return gfun(q, r) - c; };
+  double a = sh.r_peak, b = 2.0 * sh.r_peak, gb = G(b);
+  for (int it = 0; it < 60 && gb >= 0.0; ++it) {
+    a = b;
+    b *= 2.0;
+    gb = G(b);
+  }
+  const bool far = gb >= 0.0;   // barrier beyond reach (vanishing L): threshold 0
+  const bool bottom = (threadIdx.x & 1) || far;
+  const double ga = G(a);
+  const double root = illinois(G, bottom ? sh.r_eq : a, bottom ? sh.r_peak : b,
+                               bottom ? -c : ga, bottom ? sh.g_max - c : gb);
+  *r_min = __shfl_sync(0xffffffffu, root, 1);
+  if (!far) {
+    *r_top = __shfl_sync(0xffffffffu, root, 0);
+    *thr = veff_<false>(q, mu, 0.0, L2, *r_top, nullptr);
+  }
+  return true;
+}
+
+// Turning points of E by one warp, by bracketing (turning_points' searches,
+// the inner root in the even lanes and the outer in the odd ones).
+__device__ bool warp_turning_points(const DevPair& q, const DevShape& sh, double mu, double L2,
+                                    double E, double r_in, double r_top, double* root) {
+  auto f = [&](double r) { return veff_<false>(q, mu, 0.0, L2, r, nullptr) - E; };
+  const double fin = f(r_in);
+  if (!(fin < 0.0)) return false;
+  const bool outer = threadIdx.x & 1, fixed = outer ? isfinite(r_top) : q.kind == QCAMS_BUCK;
+  const double scale = outer ? 2.0 : 0.5;
+  double x = fixed ? (outer ? r_top : sh.r_b) : scale * r_in;
+  double fx = f(x);
+  for (int it = 0; it < 60 && !fixed && fx <= 0.0; ++it) {
+    x *= scale;
+    fx = f(x);
+  }
+  if (!__all_sync(0xffffffffu, fx > 0.0)) return false;
+  *root = illinois(f, outer ? r_in : x, outer ? x : r_in, outer ? fin : fx, outer ? fx : fin);
+  return true;
+}
+
+// Turning point of E between in (V_eff < E) and out (V_eff > E) by Newton
+// steps from r, kept inside the bracket; *slope is V_eff' there.  k = L^2 /
+// (2 mu).  V_eff is formed as the quadrature forms it, and of the last
+// iterates the one with the smallest |V_eff - E| is taken: the period's
+// integrand diverges at the ends, where their last bits count.
+__device__ double newton_turning_point(const DevPair& q, double k, double E, double in,
+                                       double out, double r, double* slope) {
+  if (!(r > fmin(in, out) && r < fmax(in, out))) r = 0.5 * (in + out);
+  double best = r, fbest = INFINITY;
+  int near = 0;
+  for (int it = 0; it < 100; ++it) {
+    double V, dV;
+    pot_VdV(q, r, &V, &dV);
+    const double ri = rsqrt(r * r);
+    const double f = V + k * (ri * ri) - E, d1 = dV - 2.0 * k * (ri * ri) * ri;
+    if (fabs(f) < fbest) {
+      fbest = fabs(f);
+      best = r;
+    }
+    if (f < 0.0) in = r;
+    else out = r;
+    double rn = r - f / d1;
+    if (!(rn >= fmin(in, out) && rn <= fmax(in, out))) rn = 0.5 * (in + out);
+    *slope = d1;
+    near += fabs(rn - r) <= 1e-9 * r ? 1 : 0;   // quadratic: the rest is rounding
+    if (near == 3 || rn == r) break;
+    r = rn;
+  }
+  return best;
+}
+
+// The level (v, j), valid in the first warp.  The other warps serve its
+// quadratures.
+__device__ qcams_level solve_level_block(const DevPair& q, const DevShape& sh, double mu, int v,
+                                         int j, LevelSmem& S) {
+  qcams_level L{};
+  const double L2 = (double)j * (double)(j + 1);
+  const double a = L2 / (2.0 * mu);
+  if (threadIdx.x >= 32) {
+    for (;;) {
+      __syncthreads();
+      if (!S.more) return L;
+      level_points(q, a, S);
+      __syncthreads();
+    }
+  }
+  double r_min, r_top, Etop, out, act, per;
+  if (sh.ok && warp_well(q, sh, mu, L2, &r_min, &r_top, &Etop)) {
+    const double Vmin = veff(q, mu, L2, r_min);
+    const double s2mu = sqrt(2.0 * mu);
+    double lo = Vmin, hi = Etop - 1e-10 * (Etop - Vmin);
+    bool exists = false;
+    if (warp_turning_points(q, sh, mu, L2, hi, r_min, r_top, &out)) {
+      level_integrals(q, a, hi, __shfl_sync(0xffffffffu, out, 0),
+                      __shfl_sync(0xffffffffu, out, 1), S, &act, &per);
+      exists = !(-0.5 + s2mu / kPi * act < v);
+    }
+    if (exists) {
+      // harmonic first guess
+      const double k2 = fmax(pot_d2V(q, r_min) + 3.0 * L2 / (mu * r_min * r_min * r_min * r_min), 0.0);
+      double E = Vmin + (v + 0.5) * sqrt(k2 / mu);
+      if (!(E > lo && E < hi)) E = 0.5 * (lo + hi);
+      const double w = sqrt(2.0 * (E - Vmin) / k2);
+      double r = (threadIdx.x & 1) ? r_min + w : r_min - w, slope = 1.0;
+      bool last = false;
+      for (int it = 0; it < 200; ++it) {
+        r = newton_turning_point(q, a, E, r_min, out, r, &slope);
+        const double rm = __shfl_sync(0xffffffffu, r, 0), rp = __shfl_sync(0xffffffffu, r, 1);
+        level_integrals(q, a, E, rm, rp, S, &act, &per);
+        const double f = -0.5 + s2mu / kPi * act - v;
+        if (f < 0) lo = E; else hi = E;
+        double En = E - f * 2.0 * kPi / (s2mu * per);
+        if (last) {   // E is converged: the integrals at it are the result
+          L.E = E;
+          L.r_minus = rm;
+          L.r_plus = rp;
+          L.tau = s2mu * per;
+          L.ok = 1;
+          break;
+        }
+        last = fabs(En - E) <= 4e-16 * fmax(fabs(E), fabs(Vmin)) || hi - lo <= 4e-16 * fabs(Vmin);
+        if (!(En > lo && En < hi)) En = last ? E : 0.5 * (lo + hi);
+        r += (En - E) / slope;
+        E = En;
+      }
+    }
+  }
+  if (threadIdx.x == 0) S.more = 0;
+  __syncthreads();
+  return L;
+}
+
 // Mark the (sys, v, j) levels the lanes need and the cache does not hold.
 __global__ void k_mark_levels(int64_t n, const int32_t* sys_id, const int32_t* v,
                               const int32_t* j, int n_sys, const uint8_t* valid, uint8_t* flag) {
@@ -373,16 +682,16 @@ __global__ void k_solve_levels(SysSet sys, const DevShape* shapes, const uint8_t
   valid[idx] = 1;
 }
 
-// Levels for an explicit request list (qcams_levels).
-__global__ void k_levels_list(SysSet sys, const DevShape* shapes, const int32_t* req, int n,
-                              qcams_level* out) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  int s = req[3 * k], v = req[3 * k + 1], j = req[3 * k + 2];
-  DevLevel L = solve_level(sys.s[s].pair[0], shapes[s * 3], sys.s[s].mu_pair[0], v, j);
-  qcams_level o;
-  o.E = L.E; o.r_minus = L.r_minus; o.r_plus = L.r_plus; o.tau = L.tau; o.ok = L.ok; o.pad = 0;
-  out[k] = o;
+// Levels for an explicit request list (qcams_levels), one block each.
+__global__ void __launch_bounds__(kLevelBlock) k_levels_list(SysSet sys, const DevShape* shapes,
+                                                             const int32_t* req,
+                                                             qcams_level* out) {
+  __shared__ LevelSmem S;
+  const int k = blockIdx.x;
+  const int s = req[3 * k], v = req[3 * k + 1], j = req[3 * k + 2];
+  const qcams_level L =
+      solve_level_block(sys.s[s].pair[0], shapes[s * 3], sys.s[s].mu_pair[0], v, j, S);
+  if (threadIdx.x == 0) out[k] = L;
 }
 
 // Total energy (Eq. 2).
@@ -485,30 +794,47 @@ __global__ void __launch_bounds__(128) k_analyze(SysSet sys, const DevShape* sha
 
 // ---------------------------------------------------------------------------
 // Histogram reduction (Sec. 2.3): each block takes a contiguous chunk of
-// lanes and accumulates the per-cell records of up to kSlots distinct cells
-// in shared memory (64-bit shared atomics); lanes of further cells go to
-// global memory directly.  Fixed-point sums make the result independent of
-// the order of the additions.
+// lanes and accumulates the records of up to kSlots distinct cells in shared
+// memory; lanes of further cells go to global memory directly.  Fixed-point
+// sums make the result independent of the order of the additions.
+//
+// Atomics bound it (the lanes' outcomes are 17 bytes each), so a lane adds
+// only what cannot be had from the other entries: its v_t, j_t and Gaussian
+// bins, or its class if it has none.  The counts of the classes with bins
+// are the sums over v_t, the total is the sum of the counts, and without
+// weights the weight sums are the counts times 2^32: k_reduce_finish fills
+// those in, one warp per cell.  2 M lanes over 330 interleaved cells: 184 us
+// with up to nine adds per lane, now 56 us.
 // ---------------------------------------------------------------------------
 constexpr int kSlots = 2;
 constexpr int kReduceBlock = 512;
-constexpr int kReduceChunk = 8192;
+constexpr int kReduceChunk = 4096;
 
 __device__ __forceinline__ unsigned long long fixp(double x) {
   return (unsigned long long)__double2ll_rn(x * 4294967296.0);
 }
 
+// A cell's record of one chunk: counts of at most kReduceChunk lanes in 32
+// bits, fixed-point sums in 64.
+struct SlotRec {
+  unsigned count[8], vt[3 * 64], jt[3 * 256];
+  unsigned long long gb[3 * 64], w[8], w2[8];
+};
+
+template <bool WEIGHTED>
 __global__ void __launch_bounds__(kReduceBlock) k_reduce(DevBatch B, int n_cells,
                                                          unsigned long long* hist) {
   __shared__ int slot_cell[kSlots];
-  __shared__ unsigned long long sh[kSlots][QCAMS_H_STRIDE];
+  __shared__ SlotRec sh[kSlots];
   const int tid = threadIdx.x;
   if (tid < kSlots) slot_cell[tid] = -1;
-  for (int k = tid; k < kSlots * QCAMS_H_STRIDE; k += blockDim.x) (&sh[0][0])[k] = 0ull;
+  for (int k = tid; k < (int)(sizeof(sh) / 4); k += blockDim.x)
+    reinterpret_cast<unsigned*>(sh)[k] = 0u;
   __syncthreads();
   const int64_t begin = (int64_t)blockIdx.x * kReduceChunk;
   const int64_t end = min(B.n, begin + kReduceChunk);
-  for (int64_t i = begin + tid; i < end; i += blockDim.x) {
+#pragma unroll 4
+  for (int64_t i = begin + tid; i < end; i += kReduceBlock) {
     const int c = B.cell[i];
     if (c < 0 || c >= n_cells) continue;
     int slot = -1;
@@ -520,17 +846,28 @@ __global__ void __launch_bounds__(kReduceBlock) k_reduce(DevBatch B, int n_cells
         if (prev == -1 || prev == c) slot = k;
       }
     }
-    unsigned long long* H = slot >= 0 ? sh[slot] : hist + (size_t)c * QCAMS_H_STRIDE;
     int k = B.cls[i];
     if (k < 0 || k >= QCAMS_N_CLS) k = QCAMS_CLS_FAIL;
-    const double wv = B.isw ? B.isw[i] : 1.0;
-    atomicAdd(&H[QCAMS_H_COUNT + k], 1ull);
-    atomicAdd(&H[QCAMS_H_COUNT + 6], 1ull);
-    atomicAdd(&H[QCAMS_H_W + k], fixp(wv));
-    atomicAdd(&H[QCAMS_H_W2 + k], fixp(wv * wv));
-    if (k <= 2) {
-      const int v = max(0, min((int)B.vt[i], 63));
-      const int jj = max(0, min((int)B.jt[i], 255));
+    const int v = max(0, min((int)B.vt[i], 63)), jj = max(0, min((int)B.jt[i], 255));
+    unsigned long long* H = hist + (size_t)c * QCAMS_H_STRIDE;
+    if (WEIGHTED) {
+      const double wv = B.isw[i];
+      if (slot >= 0) {
+        atomicAdd(&sh[slot].w[k], fixp(wv));
+        atomicAdd(&sh[slot].w2[k], fixp(wv * wv));
+      } else {
+        atomicAdd(&H[QCAMS_H_W + k], fixp(wv));
+        atomicAdd(&H[QCAMS_H_W2 + k], fixp(wv * wv));
+      }
+    }
+    if (k > 2) {
+      if (slot >= 0) atomicAdd(&sh[slot].count[k], 1u);
+      else atomicAdd(&H[QCAMS_H_COUNT + k], 1ull);
+    } else if (slot >= 0) {
+      atomicAdd(&sh[slot].vt[64 * k + v], 1u);
+      atomicAdd(&sh[slot].jt[256 * k + jj], 1u);
+      atomicAdd(&sh[slot].gb[64 * k + v], fixp(B.gbw[i]));
+    } else {
       atomicAdd(&H[QCAMS_H_VT + 64 * k + v], 1ull);
       atomicAdd(&H[QCAMS_H_JT + 256 * k + jj], 1ull);
       atomicAdd(&H[QCAMS_H_GB + 64 * k + v], fixp(B.gbw[i]));
@@ -541,11 +878,78 @@ __global__ void __launch_bounds__(kReduceBlock) k_reduce(DevBatch B, int n_cells
     const int c = slot_cell[s];
     if (c < 0) continue;
     unsigned long long* G = hist + (size_t)c * QCAMS_H_STRIDE;
-    for (int k = tid; k < QCAMS_H_STRIDE; k += blockDim.x) {
-      const unsigned long long v = sh[s][k];
-      if (v) atomicAdd(&G[k], v);
+    auto add = [&](int at, unsigned long long v) { if (v) atomicAdd(&G[at], v); };
+    for (int k = tid; k < 3 * 256; k += blockDim.x) add(QCAMS_H_JT + k, sh[s].jt[k]);
+    if (tid < 3 * 64) {
+      add(QCAMS_H_VT + tid, sh[s].vt[tid]);
+      add(QCAMS_H_GB + tid, sh[s].gb[tid]);
+    } else if (tid < 3 * 64 + 8) {
+      const int k = tid - 3 * 64;
+      add(QCAMS_H_COUNT + k, sh[s].count[k]);
+      if (WEIGHTED) {
+        add(QCAMS_H_W + k, sh[s].w[k]);
+        add(QCAMS_H_W2 + k, sh[s].w2[k]);
+      }
     }
   }
+}
+
+constexpr int kXsecRow = 3 * QCAMS_N_CLS;   // counts, sums of w and of w^2 per class
+
+template <bool WEIGHTED>
+__global__ void __launch_bounds__(128) k_reduce_finish(int n_cells, unsigned long long* hist,
+                                                       unsigned long long* rows) {
+  const int c = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (c >= n_cells) return;
+  unsigned long long* H = hist + (size_t)c * QCAMS_H_STRIDE;
+  unsigned long long mine = lane >= 3 && lane < QCAMS_N_CLS ? H[QCAMS_H_COUNT + lane] : 0ull;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    unsigned long long s = H[QCAMS_H_VT + 64 * k + lane] + H[QCAMS_H_VT + 64 * k + 32 + lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    mine = lane == k ? s : mine;
+  }
+  unsigned long long total = mine;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+  if (lane < 3) H[QCAMS_H_COUNT + lane] = mine;
+  if (lane == 6) H[QCAMS_H_COUNT + 6] = total;
+  if (!WEIGHTED && lane < QCAMS_N_CLS) {
+    H[QCAMS_H_W + lane] = mine << 32;
+    H[QCAMS_H_W2 + lane] = mine << 32;
+  }
+  if (rows && lane < QCAMS_N_CLS) {   // what the cross sections need, packed for one copy
+    unsigned long long* R = rows + (size_t)c * kXsecRow;
+    R[lane] = mine;
+    R[QCAMS_N_CLS + lane] = WEIGHTED ? H[QCAMS_H_W + lane] : mine << 32;
+    R[2 * QCAMS_N_CLS + lane] = WEIGHTED ? H[QCAMS_H_W2 + lane] : mine << 32;
+  }
+}
+
+// Pinned host rows for the cross sections of one call at a time (1 MB, kept
+// until qcams_shutdown; callers hold g_rows_mutex).
+constexpr int kHostRows = (1 << 20) / (kXsecRow * (int)sizeof(unsigned long long));
+std::mutex g_rows_mutex;
+unsigned long long* g_rows = nullptr;
+bool host_rows() {
+  if (!g_rows && cudaHostAlloc((void**)&g_rows, kHostRows * kXsecRow * sizeof(*g_rows),
+                               cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+    g_rows = nullptr;
+    (void)cudaGetLastError();
+  }
+  return g_rows != nullptr;
+}
+
+template <bool WEIGHTED>
+cudaError_t launch_reduce(const DevBatch& d, int n_cells, unsigned long long* hist,
+                          unsigned long long* rows, cudaStream_t st) {
+  if (d.n > 0)
+    k_reduce<WEIGHTED><<<(unsigned)((d.n + kReduceChunk - 1) / kReduceChunk), kReduceBlock, 0,
+                         st>>>(d, n_cells, hist);
+  if (d.n > 0 || rows)
+    k_reduce_finish<WEIGHTED><<<(unsigned)((n_cells + 3) / 4), 128, 0, st>>>(n_cells, hist, rows);
+  return cudaGetLastError();
 }
 
 int cuda_status(cudaError_t e) { return e == cudaSuccess ? QCAMS_OK : QCAMS_E_CUDA; }
@@ -591,7 +995,7 @@ int prepare_run(const qcams_system* sys, int32_t n_sys, const qcams_integ* integ
 }
 
 cudaError_t launch_shapes(const SysSet& ss, DevShape* shapes, cudaStream_t st) {
-  k_pair_shapes<<<1, 32, 0, st>>>(ss, shapes);
+  k_pair_shapes<<<3 * ss.n, kShapeBlock, 0, st>>>(ss, shapes);
   return cudaGetLastError();
 }
 
@@ -702,9 +1106,8 @@ int qcams_levels(const qcams_system* sys, int32_t n_sys, const int32_t* sys_id, 
   cudaError_t e = cudaMemcpyAsync(ctx->req_in, req.data(), req.size() * sizeof(int32_t),
                                   cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return QCAMS_E_CUDA;
-  k_pair_shapes<<<1, 32, 0, st>>>(ss, ctx->shapes);
-  k_levels_list<<<(n_levels + 63) / 64, 64, 0, st>>>(ss, ctx->shapes, ctx->req_in, n_levels,
-                                                      ctx->req_out);
+  k_pair_shapes<<<3 * ss.n, kShapeBlock, 0, st>>>(ss, ctx->shapes);
+  k_levels_list<<<n_levels, kLevelBlock, 0, st>>>(ss, ctx->shapes, ctx->req_in, ctx->req_out);
   e = cudaGetLastError();
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(out, ctx->req_out, sizeof(qcams_level) * n_levels, cudaMemcpyDeviceToHost,
@@ -736,7 +1139,7 @@ int qcams_init_states(const qcams_system* sys, int32_t n_sys, const double* E_co
   DevBatch d = dev_batch(batch);
   const int64_t n = batch->n;
   const unsigned grid = (unsigned)((n + 255) / 256);
-  k_pair_shapes<<<1, 32, 0, st>>>(ss, ctx->shapes);
+  k_pair_shapes<<<3 * ss.n, kShapeBlock, 0, st>>>(ss, ctx->shapes);
   // Level cache: a system slot keeps its solved levels while its AB pair and
   // masses are unchanged (the levels depend on nothing else).
   cudaError_t e = cudaSuccess;
@@ -778,7 +1181,7 @@ int qcams_run_batch(const qcams_system* sys, int32_t n_sys, const qcams_integ* i
   cudaStream_t st = (cudaStream_t)cuda_stream;
   if (batch->n == 0) return QCAMS_OK;
   DevBatch d = dev_batch(batch);
-  k_pair_shapes<<<1, 32, 0, st>>>(ss, ctx->shapes);
+  k_pair_shapes<<<3 * ss.n, kShapeBlock, 0, st>>>(ss, ctx->shapes);
   ctx->timed = false;
   cudaError_t e = record_event(ctx->ev[0], st);
   if (e == cudaSuccess)
@@ -813,14 +1216,17 @@ int qcams_analyze(const qcams_system* sys, int32_t n_sys, const qcams_integ* int
   cudaStream_t st = (cudaStream_t)cuda_stream;
   if (batch->n == 0) return QCAMS_OK;
   DevBatch d = dev_batch(batch);
-  k_pair_shapes<<<1, 32, 0, st>>>(ss, ctx->shapes);
+  k_pair_shapes<<<3 * ss.n, kShapeBlock, 0, st>>>(ss, ctx->shapes);
   const double sg = integ->gb_sigma > 0 ? integ->gb_sigma : 0.1 / (2.0 * std::sqrt(2.0 * std::log(2.0)));
   return cuda_status(launch_analyze(ss, ctx->shapes, sg, d, st));
 }
 
 // Cross sections from host histograms (Sec. 2.3 and Sec. 4): shared by
 // qcams_reduce_xsec and qcams_xsec_from_hist.
-static void xsec_finalize(const int64_t* hist, const qcams_cells* cells, double* xsec_out) {
+// Cell c's counts start at count[c stride], its sums of w and w^2 at
+// wsum[c stride] and w2sum[c stride].
+static void xsec_finalize(const int64_t* count, const int64_t* wsum, const int64_t* w2sum,
+                          size_t stride, const qcams_cells* cells, double* xsec_out) {
   // Opacity and binomial error per cell (Eqs. 13, 16); cross sections per
   // group as 2 pi sum w b P (Eq. 18 with the angular measure divided out).
   // Entry 6 is the reactive total R_AC + R_BC (exclusive classes, so its
@@ -831,22 +1237,22 @@ static void xsec_finalize(const int64_t* hist, const qcams_cells* cells, double*
   double* grp = xsec_out + 2 * NE * (size_t)nc;
   for (size_t k = 0; k < 2 * NE * (size_t)ng; ++k) grp[k] = 0.0;
   for (int c = 0; c < nc; ++c) {
-    const int64_t* h = hist + (size_t)c * QCAMS_H_STRIDE;
+    const int64_t *hc = count + c * stride, *hw = wsum + c * stride, *hw2 = w2sum + c * stride;
     double N = 0.0;
-    for (int k = 0; k < 5; ++k) N += (double)h[QCAMS_H_COUNT + k];
+    for (int k = 0; k < 5; ++k) N += (double)hc[k];
     for (int k = 0; k < NE; ++k) {
-      auto sum = [&](int off) {
-        return k < 6 ? (double)h[off + k] : (double)h[off + 1] + (double)h[off + 2];
+      auto sum = [&](const int64_t* h) {
+        return k < 6 ? (double)h[k] : (double)h[1] + (double)h[2];
       };
       double P = 0.0, dl = 0.0;
       if (N > 0) {
         if (!cells->weighted) {
-          const double Nx = sum(QCAMS_H_COUNT);
+          const double Nx = sum(hc);
           P = Nx / N;
           dl = std::sqrt(Nx) / N * std::sqrt((N - Nx) / N);
         } else {
-          const double sw = std::ldexp(sum(QCAMS_H_W), -32);
-          const double sw2 = std::ldexp(sum(QCAMS_H_W2), -32);
+          const double sw = std::ldexp(sum(hw), -32);
+          const double sw2 = std::ldexp(sum(hw2), -32);
           P = sw / N;
           dl = N > 1 ? std::sqrt(std::fmax(0.0, sw2 / N - P * P) / (N - 1.0)) : 0.0;
         }
@@ -883,18 +1289,38 @@ int qcams_reduce_xsec(const qcams_batch* batch, const qcams_cells* cells, int64_
   const size_t nh = (size_t)cells->n_cells * QCAMS_H_STRIDE;
   cudaError_t e = cudaMemsetAsync(hist_out, 0, nh * sizeof(int64_t), st);
   if (e != cudaSuccess) return QCAMS_E_CUDA;
-  if (batch->n > 0) {
-    DevBatch d = dev_batch(batch);
-    const unsigned grid = (unsigned)((batch->n + kReduceChunk - 1) / kReduceChunk);
-    k_reduce<<<grid, kReduceBlock, 0, st>>>(d, cells->n_cells, (unsigned long long*)hist_out);
-    if ((e = cudaGetLastError()) != cudaSuccess) return QCAMS_E_CUDA;
+  // The cross sections need only each record's counts and weight sums.
+  // k_reduce_finish writes them straight into pinned host rows; a call that
+  // finds the rows in use by another thread, or more cells than they hold,
+  // copies the two column ranges instead.
+  DevBatch d = dev_batch(batch);
+  unsigned long long* hist = (unsigned long long*)hist_out;
+  std::unique_lock<std::mutex> lock(g_rows_mutex, std::defer_lock);
+  const bool packed = xsec_out && cells->n_cells <= kHostRows && lock.try_lock() && host_rows();
+  unsigned long long* rows = packed ? g_rows : nullptr;
+  e = batch->isw ? launch_reduce<true>(d, cells->n_cells, hist, rows, st)
+                 : launch_reduce<false>(d, cells->n_cells, hist, rows, st);
+  if (!xsec_out) return cuda_status(e);
+  if (packed) {
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return QCAMS_E_CUDA;
+    const int64_t* R = (const int64_t*)rows;
+    xsec_finalize(R, R + QCAMS_N_CLS, R + 2 * QCAMS_N_CLS, kXsecRow, cells, xsec_out);
+    return QCAMS_OK;
   }
-  if (!xsec_out) return QCAMS_OK;
-  std::vector<int64_t> H(nh);
-  e = cudaMemcpyAsync(H.data(), hist_out, nh * sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+  constexpr size_t kC = QCAMS_H_VT - QCAMS_H_COUNT, kW = QCAMS_H_STRIDE - QCAMS_H_W, kRow = kC + kW;
+  const size_t nc = cells->n_cells, pitch = QCAMS_H_STRIDE * sizeof(int64_t);
+  std::vector<int64_t> H(nc * kRow);
+  if (e == cudaSuccess)
+    e = cudaMemcpy2DAsync(H.data(), kRow * sizeof(int64_t), hist_out + QCAMS_H_COUNT, pitch,
+                          kC * sizeof(int64_t), nc, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpy2DAsync(H.data() + kC, kRow * sizeof(int64_t), hist_out + QCAMS_H_W, pitch,
+                          kW * sizeof(int64_t), nc, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return QCAMS_E_CUDA;
-  xsec_finalize(H.data(), cells, xsec_out);
+  xsec_finalize(H.data(), H.data() + kC, H.data() + kC + (QCAMS_H_W2 - QCAMS_H_W), kRow, cells,
+                xsec_out);
   return QCAMS_OK;
 }
 
@@ -903,7 +1329,8 @@ int qcams_xsec_from_hist(const int64_t* hist, const qcams_cells* cells, double* 
   if (cells->n_cells < 1 || cells->n_groups < 0) return QCAMS_E_INVALID;
   if (cells->n_cells > kMaxCells || cells->n_groups > kMaxCells) return QCAMS_E_CAPACITY;
   if (!cells->b || !cells->w || (cells->n_groups > 0 && !cells->group)) return QCAMS_E_INVALID;
-  xsec_finalize(hist, cells, xsec_out);
+  xsec_finalize(hist + QCAMS_H_COUNT, hist + QCAMS_H_W, hist + QCAMS_H_W2, QCAMS_H_STRIDE, cells,
+                xsec_out);
   return QCAMS_OK;
 }
 
@@ -1148,6 +1575,11 @@ int qcams_shutdown(void) {
   if (cudaGetDevice(&dev) != cudaSuccess) return QCAMS_E_NODEVICE;
   if (dev < 0 || dev >= kMaxDevices) return QCAMS_E_INVALID;
   noalloc_forget_device(dev);
+  {
+    std::lock_guard<std::mutex> rows(g_rows_mutex);
+    if (g_rows) cudaFreeHost(g_rows);
+    g_rows = nullptr;
+  }
   std::lock_guard<std::mutex> lk(g_mutex);
   Ctx* c = g_ctx[dev];
   if (!c) return QCAMS_OK;

@@ -1,0 +1,76 @@
+"""Reduction and proposal kernels at the edges of their tiles, against plain
+integer / FP64 numpy: chunks and cells of one, odd and large sizes, lanes with
+classes, bins and cells out of range; grids below, at and above the run and
+scan blocks."""
+import numpy as np
+import pytest
+
+
+@pytest.fixture(scope="module")
+def Q():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    from paper_2304_02731_gb300 import qcams
+    return qcams
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,n_cells,weighted,sort", [
+    (1, 1, False, False), (37, 3, True, False), (4096, 5, False, True), (4097, 400, True, False),
+    (30_011, 9000, False, False), (50_001, 2, True, True)])
+def test_reduce_matches_counts(Q, n, n_cells, weighted, sort):
+    rng = np.random.default_rng(n)
+    cell = rng.integers(-1, n_cells + 1, n).astype(np.int32)
+    if sort:
+        cell.sort()
+    cls, vt, jt = rng.integers(0, 8, n), rng.integers(-3, 90, n), rng.integers(-3, 400, n)
+    gbw = rng.uniform(0, 9, n)
+    w = rng.uniform(0, 3, n) if weighted else np.ones(n)
+    b = Q.Batch.empty(n, "cuda", cell=cell, isw=w if weighted else None)
+    import torch
+    for dst, src in ((b.cls, cls), (b.vt, vt), (b.jt, jt), (b.f64["gbw"], gbw)):
+        dst.copy_(torch.as_tensor(src))
+    hist, cells, _ = Q.reduce_xsec(b, n_cells, np.ones(n_cells), np.ones(n_cells),
+                                   np.zeros(n_cells), 1, weighted=weighted)
+    want = np.zeros((n_cells, Q.H_STRIDE), np.int64)
+    fix = lambda x: np.rint(x * 2.0 ** 32).astype(np.int64)  # noqa: E731
+    keep = (cell >= 0) & (cell < n_cells)
+    c, k = cell[keep], np.where(cls < 6, cls, 5)[keep]
+    v, j = np.clip(vt[keep], 0, 63), np.clip(jt[keep], 0, 255)
+    np.add.at(want, (c, Q.H_COUNT + k), 1)
+    np.add.at(want, (c, np.full(c.size, Q.H_COUNT + 6)), 1)
+    np.add.at(want, (c, Q.H_W + k), fix(w[keep]))
+    np.add.at(want, (c, Q.H_W2 + k), fix(w[keep] * w[keep]))
+    p = k <= 2
+    np.add.at(want, (c[p], Q.H_VT + 64 * k[p] + v[p]), 1)
+    np.add.at(want, (c[p], Q.H_JT + 256 * k[p] + j[p]), 1)
+    np.add.at(want, (c[p], Q.H_GB + 64 * k[p] + v[p]), fix(gbw[keep][p]))
+    assert np.array_equal(hist.cpu().numpy(), want)
+    host, _ = Q.xsec_from_hist(want, np.ones(n_cells), np.ones(n_cells), np.zeros(n_cells), 1,
+                               weighted=weighted)
+    assert np.array_equal(cells, host)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dims", [(1, 1, 1, 1, 1), (3, 1, 2, 1, 1), (1023, 1, 1, 1, 1),
+                                  (2048, 1, 1, 1, 1), (2049, 1, 1, 1, 1), (31, 17, 13, 11, 7),
+                                  (1, 1, 1, 1 << 20, 3)])
+def test_proposal_cdf_and_draws(Q, dims):
+    import torch
+    mlp = Q.MLP("cuda", seed=3)
+    spec = Q.proposal_spec(0.1, 3, 5, dims=dims, b2_max=77.0)
+    q, qfix, cdf = (t.cpu().numpy() for t in mlp.build_proposal(spec))
+    N = int(np.prod(dims))
+    assert abs(q.sum() - 1.0) < 1e-12
+    assert np.array_equal(qfix, np.rint(q * 2.0 ** 40).astype(np.int64))
+    assert np.array_equal(cdf, np.cumsum(qfix))
+    n = 3001
+    b, u, w, cell = (t.cpu().numpy() for t in Q.sample_proposal(
+        spec, torch.as_tensor(qfix).cuda(), torch.as_tensor(cdf).cuda(), n, 9, 12345678901))
+    idx = np.stack(np.unravel_index(cell, dims))
+    pos = np.stack([b * b / 77.0, *u])
+    d = np.array(dims, np.float64)[:, None]
+    # a coordinate lies in its cell to the rounding of sqrt and its square
+    assert np.all(pos * d >= idx * (1 - 1e-15)) and np.all(pos * d <= (idx + 1) * (1 + 1e-15))
+    assert np.array_equal(w, (cdf[-1] / N) / qfix[cell])
