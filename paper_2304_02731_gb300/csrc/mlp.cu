@@ -33,8 +33,8 @@ constexpr int IN = 8, H = 64, OUT = 4, NP = QCAMS_MLP_NPARAMS;
 constexpr int OW1 = 0, OB1 = OW1 + H * IN, OW2 = OB1 + H, OB2 = OW2 + H * H, OW3 = OB2 + H,
               OB3 = OW3 + H * H, OW4 = OB3 + H, OB4 = OW4 + OUT * H;
 static_assert(OB4 + OUT == NP, "parameter layout");
-static_assert(OW1 % 2 == 0 && OW2 % 2 == 0 && OW3 % 2 == 0 && OW4 % 2 == 0 && IN % 2 == 0,
-              "weight-gradient pairs are 8-byte aligned");
+static_assert(OW1 % 4 == 0 && OW2 % 4 == 0 && OW3 % 4 == 0 && OW4 % 4 == 0 && IN % 4 == 0,
+              "weight-gradient quads are 16-byte aligned");
 constexpr int WARPS = 4, THREADS = WARPS * 32;
 constexpr double kPi = 3.14159265358979323846;
 
@@ -124,7 +124,8 @@ __device__ __forceinline__ __nv_bfloat16 bf_hi(uint32_t w) {
 // every matrix starts on a 16-byte boundary: each thread issues all of its
 // 16-byte loads of 8-element row segments first, then stores each segment
 // to its W row and, TRANSPOSED (the backward pass), element by element to the
-// W^T column.  Otherwise, element loads.
+// W^T column.  Otherwise, element loads.  All loads go to L2: the training
+// kernel's other blocks rewrite the parameters between its steps.
 template <bool TRANSPOSED>
 __device__ void load_weights(WeightsSmem& W, const __nv_bfloat16* p, const float* pf) {
   const __nv_bfloat16 zero = __float2bfloat16(0.0f);
@@ -142,7 +143,7 @@ __device__ void load_weights(WeightsSmem& W, const __nv_bfloat16* p, const float
       else if (i < N1 + N2) off = OW2 + 8 * (i - N1);
       else if (i < N1 + 2 * N2) off = OW3 + 8 * (i - N1 - N2);
       else if (i < NSEG) off = OW4 + 8 * (i - N1 - 2 * N2);
-      if (i < NSEG) v[k] = *reinterpret_cast<const uint4*>(p + off);
+      if (i < NSEG) v[k] = __ldcg(reinterpret_cast<const uint4*>(p + off));
     }
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
@@ -177,32 +178,35 @@ __device__ void load_weights(WeightsSmem& W, const __nv_bfloat16* p, const float
     for (int i = threadIdx.x; i < H * (16 - OUT); i += blockDim.x)
       W.w4t[i / (16 - OUT)][OUT + i % (16 - OUT)] = zero;
   } else {
+    auto ld = [&](int k) {
+      return __ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short*>(p) + k));
+    };
     for (int i = threadIdx.x; i < H * 16; i += blockDim.x) {
       const int r = i / 16, c = i % 16;
-      W.w1[r][c] = c < IN ? p[OW1 + r * IN + c] : zero;
+      W.w1[r][c] = c < IN ? ld(OW1 + r * IN + c) : zero;
     }
     for (int i = threadIdx.x; i < H * H; i += blockDim.x) {
       const int r = i / H, c = i % H;
-      W.w2[r][c] = p[OW2 + i];
-      W.w3[r][c] = p[OW3 + i];
-      W.w2t[c][r] = p[OW2 + i];
-      W.w3t[c][r] = p[OW3 + i];
+      W.w2[r][c] = ld(OW2 + i);
+      W.w3[r][c] = ld(OW3 + i);
+      W.w2t[c][r] = ld(OW2 + i);
+      W.w3t[c][r] = ld(OW3 + i);
     }
     for (int i = threadIdx.x; i < 8 * H; i += blockDim.x) {
       const int r = i / H, c = i % H;
-      W.w4[r][c] = r < OUT ? p[OW4 + r * H + c] : zero;
+      W.w4[r][c] = r < OUT ? ld(OW4 + r * H + c) : zero;
     }
     for (int i = threadIdx.x; i < H * 16; i += blockDim.x) {
       const int r = i / 16, c = i % 16;
-      W.w4t[r][c] = c < OUT ? p[OW4 + c * H + r] : zero;
+      W.w4t[r][c] = c < OUT ? ld(OW4 + c * H + r) : zero;
     }
   }
   for (int i = threadIdx.x; i < H; i += blockDim.x) {
-    W.b1[i] = pf[OB1 + i];
-    W.b2[i] = pf[OB2 + i];
-    W.b3[i] = pf[OB3 + i];
+    W.b1[i] = __ldcg(pf + OB1 + i);
+    W.b2[i] = __ldcg(pf + OB2 + i);
+    W.b3[i] = __ldcg(pf + OB3 + i);
   }
-  if (threadIdx.x < 8) W.b4[threadIdx.x] = threadIdx.x < OUT ? pf[OB4 + threadIdx.x] : 0.0f;
+  if (threadIdx.x < 8) W.b4[threadIdx.x] = threadIdx.x < OUT ? __ldcg(pf + OB4 + threadIdx.x) : 0.0f;
 }
 
 // Features of the 16 rows handled by this lane's fragment rows: either from
@@ -211,15 +215,30 @@ struct CellGrid {
   int n_b2, n_cth, n_phi, n_eta, n_chi;
   float E, v, j, b2_max;
 };
-__device__ __forceinline__ void features(const float* x, const int64_t* idx, int64_t n,
+// Minibatch rows: row i is sample i, or (draw) a uniform one of `n`, from
+// Philox4x32-10 with key = seed and counter (i, step_lo, step_hi, 4); the
+// 64-bit word w1:w0 is mapped by the high half of w * n (bias <= n / 2^64).
+struct RowSrc {
+  bool draw;
+  int64_t n;
+  uint64_t seed, step;
+  __device__ __forceinline__ int64_t at(int64_t i) const {
+    if (!draw) return i;
+    const uint4 w = philox4x32_10(
+        make_uint4((uint32_t)i, (uint32_t)step, (uint32_t)(step >> 32), 4u),
+        make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
+    const unsigned long long u = ((unsigned long long)w.y << 32) | w.x;
+    return (int64_t)__umul64hi(u, (unsigned long long)n);
+  }
+};
+__device__ __forceinline__ void features(const float* x, int64_t src, int64_t n,
                                          int64_t row, const CellGrid* grid, float* f) {
   if (row >= n) {
     for (int k = 0; k < IN; ++k) f[k] = 0.0f;
     return;
   }
   if (!grid) {
-    const int64_t r = idx ? idx[row] : row;   // minibatch rows gathered through idx
-    for (int k = 0; k < IN; ++k) f[k] = x[r * IN + k];
+    for (int k = 0; k < IN; ++k) f[k] = x[src * IN + k];
     return;
   }
   int64_t c = row;
@@ -238,19 +257,20 @@ __device__ __forceinline__ void features(const float* x, const int64_t* idx, int
   f[7] = 2.0f * (float)kPi * (i_eta + 0.5f) / grid->n_eta;
 }
 
-// Forward pass of 16 samples (rows base .. base+15) by one warp.  Returns the
+// Forward pass of 16 samples (rows base .. base+15) by one warp; this lane's
+// rows base + g and base + g + 8 are samples src0 and src1.  Returns the
 // logits fragment (rows g and g+8, columns 2q, 2q+1 of the padded 16x8 tile).
 // With TRAIN, pre-activations go to the warp's z tiles and the transposed
 // inputs and activations to the block tiles T, at sample columns col ..
 // col + 15, for the backward pass.
 template <bool TRAIN, int CPW>
 __device__ void forward16(const WeightsSmem& W, WarpZ* wz, BlockTiles<CPW>* T, int col, const float* x,
-                          const int64_t* idx, int64_t n, int64_t base, const CellGrid* grid,
-                          const Std& sd, float* logit) {
+                          int64_t src0, int64_t src1, int64_t n, int64_t base,
+                          const CellGrid* grid, const Std& sd, float* logit) {
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
   float f0[IN], f1[IN];
-  features(x, idx, n, base + g, grid, f0);
-  features(x, idx, n, base + g + 8, grid, f1);
+  features(x, src0, n, base + g, grid, f0);
+  features(x, src1, n, base + g + 8, grid, f1);
   for (int k = 0; k < IN; ++k) {
     f0[k] = (f0[k] - sd.mean[k]) * sd.inv_std[k];
     f1[k] = (f1[k] - sd.mean[k]) * sd.inv_std[k];
@@ -344,6 +364,7 @@ template <int LDT>
 __device__ void block_dw(const __nv_bfloat16 (*dzt)[LDT], const __nv_bfloat16 (*at)[LDT], int m0,
                          int n0, int n_tiles, int n_out, int n_in, float* gW) {
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+  const bool vec4 = (reinterpret_cast<uintptr_t>(gW) & 15u) == 0;
   float d[8][4];
 #pragma unroll
   for (int t = 0; t < 8; ++t) d[t][0] = d[t][1] = d[t][2] = d[t][3] = 0.0f;
@@ -362,15 +383,29 @@ __device__ void block_dw(const __nv_bfloat16 (*dzt)[LDT], const __nv_bfloat16 (*
       }
     }
   }
+  // Lanes q and q ^ 1 hold columns 2q, 2q + 1 of rows g and g + 8: the even
+  // one takes both lanes' share of row g, the odd one of row g + 8, four
+  // consecutive columns each (vector atomics, sm_90 and later; n_in is a
+  // multiple of 4 and the parameter offsets are too).
 #pragma unroll
   for (int t = 0; t < 8; ++t) {
     if (t >= n_tiles) continue;
-    const int r0 = m0 + g, r1 = r0 + 8, c = n0 + 8 * t + 2 * q;
-    // c and n_in are even and the parameter offsets are even: 8-byte
-    // aligned pairs (vector atomics, sm_90 and later)
-    if (c < n_in) {
-      if (r0 < n_out) atomicAdd(reinterpret_cast<float2*>(&gW[r0 * n_in + c]), make_float2(d[t][0], d[t][1]));
-      if (r1 < n_out) atomicAdd(reinterpret_cast<float2*>(&gW[r1 * n_in + c]), make_float2(d[t][2], d[t][3]));
+    const bool odd = q & 1;
+    const float s0 = odd ? d[t][0] : d[t][2], s1 = odd ? d[t][1] : d[t][3];
+    const float o0 = __shfl_xor_sync(0xffffffffu, s0, 1), o1 = __shfl_xor_sync(0xffffffffu, s1, 1);
+    const float4 v = odd ? make_float4(o0, o1, d[t][2], d[t][3])
+                         : make_float4(d[t][0], d[t][1], o0, o1);
+    const int r = m0 + g + (odd ? 8 : 0), c = n0 + 8 * t + 2 * (q & 2);
+    if (c < n_in && r < n_out) {
+      float* at = &gW[r * n_in + c];
+      if (vec4) {
+        atomicAdd(reinterpret_cast<float4*>(at), v);
+      } else {   // a gradient buffer that is not 16-byte aligned
+        atomicAdd(at, v.x);
+        atomicAdd(at + 1, v.y);
+        atomicAdd(at + 2, v.z);
+        atomicAdd(at + 3, v.w);
+      }
     }
   }
 }
@@ -409,27 +444,35 @@ __device__ __forceinline__ void accumulate_db(const float (*dz)[4], int tiles, i
   }
 }
 
-// Gradient of the mean cross-entropy over n rows; with idx, row r of the
-// minibatch is sample idx[r] of (x, label).  Block rounds of RS samples: each
+// Shared state of a gradient block before its first round (ends without a
+// barrier).
+template <int CPW>
+__device__ void grad_begin(TrainSmem<CPW>& S, const __nv_bfloat16* pb, const float* pf) {
+  load_weights<true>(S.w, pb, pf);
+  for (int i = threadIdx.x; i < NGB; i += blockDim.x) S.gb[i] = 0.0f;
+}
+// Padding rows of the X^T and dZ4^T tiles (never written by the passes).
+template <int CPW>
+__device__ void grad_pad(TrainSmem<CPW>& S) {
+  constexpr int LDT = BlockTiles<CPW>::LDT;
+  const __nv_bfloat16 zero = __float2bfloat16(0.0f);
+  for (int i = threadIdx.x; i < (16 - IN) * LDT; i += blockDim.x) S.t.xt[IN + i / LDT][i % LDT] = zero;
+  for (int i = threadIdx.x; i < (16 - 8) * LDT; i += blockDim.x) S.t.dz4t[8 + i / LDT][i % LDT] = zero;
+}
+
+// This block's share of the gradient of the mean cross-entropy over n rows
+// (rows.at(r) the sample behind row r).  Block rounds of RS samples: each
 // warp carries its chunks of 16 through the forward and backward passes
 // (activations and errors to the block tiles, bias gradients to shared FP32
 // sums), then the four weight gradients of the round are formed as block
 // GEMMs (warp w: rows 16w .. 16w+15 of dW1..dW3, columns 16w .. 16w+15 of
 // dW4) and added to the global gradient.
 template <int CPW>
-__global__ void __launch_bounds__(THREADS) k_mlp_grad(const __nv_bfloat16* pb, const float* pf,
-                                                      Std sd, const float* x,
-                                                      const uint8_t* label, const int64_t* idx,
-                                                      int64_t n, float* grad, float* loss) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  TrainSmem<CPW>& S = *reinterpret_cast<TrainSmem<CPW>*>(smem_raw);
-  constexpr int RS = BlockTiles<CPW>::RS, LDT = BlockTiles<CPW>::LDT;
-  load_weights<true>(S.w, pb, pf);
-  for (int i = threadIdx.x; i < NGB; i += blockDim.x) S.gb[i] = 0.0f;
-  // padding rows of the X^T and dZ4^T tiles (never written by the passes)
-  const __nv_bfloat16 zero = __float2bfloat16(0.0f);
-  for (int i = threadIdx.x; i < (16 - IN) * LDT; i += blockDim.x) S.t.xt[IN + i / LDT][i % LDT] = zero;
-  for (int i = threadIdx.x; i < (16 - 8) * LDT; i += blockDim.x) S.t.dz4t[8 + i / LDT][i % LDT] = zero;
+__device__ void grad_rounds(TrainSmem<CPW>& S, const Std& sd, const float* x,
+                            const uint8_t* label, const RowSrc& rows, int64_t n, float* grad,
+                            float* loss) {
+  constexpr int RS = BlockTiles<CPW>::RS;
+  if ((int64_t)blockIdx.x * RS >= n) return;   // no round for this block
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
   WarpZ* wz = &S.wz[warp];
@@ -441,7 +484,9 @@ __global__ void __launch_bounds__(THREADS) k_mlp_grad(const __nv_bfloat16* pb, c
       const int col = 16 * (WARPS * c + warp);
       const int64_t base = rnd * RS + col;
       float lg[4];
-      forward16<true, CPW>(S.w, wz, &S.t, col, x, idx, n, base, nullptr, sd, lg);
+      const int64_t r0 = base + g, r1 = base + g + 8;
+      const int64_t s0 = rows.at(r0), s1 = rows.at(r1);
+      forward16<true, CPW>(S.w, wz, &S.t, col, x, s0, s1, n, base, nullptr, sd, lg);
       // softmax cross-entropy and dZ4 = (p - onehot) / n; rows past n and
       // rows without a target have dZ4 = 0 and so add nothing below
       float dz4[1][4] = {{0.f, 0.f, 0.f, 0.f}};
@@ -449,9 +494,8 @@ __global__ void __launch_bounds__(THREADS) k_mlp_grad(const __nv_bfloat16* pb, c
       softmax_pair(lg[0], lg[1], &p[0], &p[1]);
       softmax_pair(lg[2], lg[3], &p[2], &p[3]);
       if (q < 2) {
-        const int64_t r0 = base + g, r1 = base + g + 8;
-        int l0 = r0 < n ? (int)label[idx ? idx[r0] : r0] : -1;
-        int l1 = r1 < n ? (int)label[idx ? idx[r1] : r1] : -1;
+        int l0 = r0 < n ? (int)label[s0] : -1;
+        int l1 = r1 < n ? (int)label[s1] : -1;
         if (l0 >= OUT) l0 = -1;   // AMBIG / FAIL lanes carry no target
         if (l1 >= OUT) l1 = -1;
         for (int e = 0; e < 2; ++e) {
@@ -520,6 +564,18 @@ __global__ void __launch_bounds__(THREADS) k_mlp_grad(const __nv_bfloat16* pb, c
   }
 }
 
+template <int CPW>
+__global__ void __launch_bounds__(THREADS) k_mlp_grad(const __nv_bfloat16* pb, const float* pf,
+                                                      Std sd, const float* x,
+                                                      const uint8_t* label, int64_t n,
+                                                      float* grad, float* loss) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  TrainSmem<CPW>& S = *reinterpret_cast<TrainSmem<CPW>*>(smem_raw);
+  grad_pad<CPW>(S);
+  grad_begin<CPW>(S, pb, pf);
+  grad_rounds<CPW>(S, sd, x, label, RowSrc{false, n, 0, 0}, n, grad, loss);
+}
+
 __global__ void __launch_bounds__(THREADS) k_mlp_infer(const __nv_bfloat16* pb, const float* pf,
                                                        Std sd, const float* x, int64_t n,
                                                        CellGrid grid, int use_grid,
@@ -534,8 +590,8 @@ __global__ void __launch_bounds__(THREADS) k_mlp_infer(const __nv_bfloat16* pb, 
        ch += (int64_t)gridDim.x * WARPS) {
     const int64_t base = ch * 16;
     float lg[4], p[4];
-    forward16<false, 1>(W, nullptr, nullptr, 0, x, nullptr, n, base, use_grid ? &grid : nullptr, sd,
-                     lg);
+    forward16<false, 1>(W, nullptr, nullptr, 0, x, base + g, base + g + 8, n, base,
+                        use_grid ? &grid : nullptr, sd, lg);
     softmax_pair(lg[0], lg[1], &p[0], &p[1]);
     softmax_pair(lg[2], lg[3], &p[2], &p[3]);
     const int64_t r0 = base + g, r1 = base + g + 8;
@@ -556,30 +612,103 @@ __global__ void __launch_bounds__(THREADS) k_mlp_infer(const __nv_bfloat16* pb, 
   }
 }
 
+// One parameter's Adam step (beta1 0.9, beta2 0.999, eps 1e-8; c1, c2 the
+// bias corrections).
+__device__ __forceinline__ void adam_one(int i, float gr, float* p, float* m, float* v,
+                                         __nv_bfloat16* pb, float lr, float c1, float c2) {
+  const float mi = 0.9f * m[i] + 0.1f * gr;
+  const float vi = 0.999f * v[i] + 0.001f * gr * gr;
+  m[i] = mi;
+  v[i] = vi;
+  const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+  p[i] = pi;
+  pb[i] = __float2bfloat16(pi);
+}
+
 __global__ void k_adam(float* p, float* m, float* v, const float* grad, __nv_bfloat16* pb,
                        float lr, float c1, float c2) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < NP; i += gridDim.x * blockDim.x) {
-    const float gr = grad[i];
-    const float mi = 0.9f * m[i] + 0.1f * gr;
-    const float vi = 0.999f * v[i] + 0.001f * gr * gr;
-    m[i] = mi;
-    v[i] = vi;
-    const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
-    p[i] = pi;
-    pb[i] = __float2bfloat16(pi);
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < NP; i += gridDim.x * blockDim.x)
+    adam_one(i, grad[i], p, m, v, pb, lr, c1, c2);
+}
+
+// All steps of one training call in one cooperative launch, one block per
+// SM.  Separate launches took 36 us a step (index draw 2.4, memsets, gradient
+// 22, Adam 3.4 and the gaps between them) for work that needs a fraction of
+// a microsecond at the tensor cores' rate: the step is a chain of latencies,
+// and this kernel shortens it to 21 us.  Each step a block draws its own
+// rows, adds its share of the gradient and, after a grid barrier, takes the
+// Adam step of its own slice of the parameters; a second barrier publishes
+// them.  Gradient, loss and Adam arithmetic are those of the separate kernels.
+struct GridBarrier {
+  unsigned* count;      // zero at launch
+  unsigned target;
+  // Bounded: a barrier that is not complete after about ten seconds gives up.
+  __device__ bool wait() {
+    __shared__ int ok;
+    __syncthreads();
+    target += gridDim.x;
+    if (threadIdx.x == 0) {
+      __threadfence();
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+      unsigned seen = 0;
+      int left = 1 << 25;
+      do {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
+      } while ((int)(seen - target) < 0 && --left > 0);
+      ok = left > 0;
+    }
+    __syncthreads();
+    return ok != 0;
+  }
+};
+
+template <int CPW>
+__global__ void __launch_bounds__(THREADS) k_mlp_train(float* p, float* m, float* v, float* grad,
+                                                       __nv_bfloat16* pb, Std sd, const float* x,
+                                                       const uint8_t* label, RowSrc rows,
+                                                       int64_t steps, int64_t batch, float lr,
+                                                       double b1, double b2, float* losses,
+                                                       unsigned* barrier) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  TrainSmem<CPW>& S = *reinterpret_cast<TrainSmem<CPW>*>(smem_raw);
+  GridBarrier bar{barrier, 0u};
+  const int per = (NP + gridDim.x - 1) / gridDim.x;
+  const int lo = blockIdx.x * per, hi = min(NP, lo + per);
+  grad_pad<CPW>(S);
+  for (int64_t s = 0; s < steps; ++s, ++rows.step) {
+    grad_begin<CPW>(S, pb, p);
+    grad_rounds<CPW>(S, sd, x, label, rows, batch, grad, losses ? losses + s : nullptr);
+    b1 *= 0.9;
+    b2 *= 0.999;
+    const float c1 = (float)(1.0 - b1), c2 = (float)(1.0 - b2);
+    bool ok = bar.wait();   // the gradient is complete
+    // the next step's first rows towards L2 while the barriers pass
+    if (s + 1 < steps) {
+      RowSrc next = rows;
+      ++next.step;
+      const int64_t r = (int64_t)blockIdx.x * BlockTiles<CPW>::RS + threadIdx.x;
+      if (threadIdx.x < BlockTiles<CPW>::RS && r < batch) {
+        const int64_t src = next.at(r);
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(x + src * IN));
+        asm volatile("prefetch.global.L1 [%0];" ::"l"(label + src));
+      }
+    }
+    for (int i = lo + threadIdx.x; i < hi; i += THREADS) {
+      adam_one(i, __ldcg(grad + i), p, m, v, pb, lr, c1, c2);
+      if (s + 1 < steps) grad[i] = 0.0f;
+    }
+    ok = ok && bar.wait();  // the parameters are
+    if (!ok) {
+      if (losses && threadIdx.x == 0) losses[s] = __int_as_float(0x7fc00000);
+      return;
+    }
   }
 }
 
-// Minibatch indices for training step `step`: idx[i] uniform on [0, n) from
-// Philox4x32-10 with key = seed and counter (i, step_lo, step_hi, 4); the
-// 64-bit word w1:w0 is mapped by the high half of w * n (bias <= n / 2^64).
-__global__ void k_draw_idx(int64_t* idx, int batch, int64_t n, uint64_t seed, uint64_t step) {
+// The rows of training step `step` (RowSrc).
+__global__ void k_draw_idx(int64_t* idx, int batch, RowSrc rows) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= batch) return;
-  const uint4 w = philox4x32_10(make_uint4((uint32_t)i, (uint32_t)step, (uint32_t)(step >> 32), 4u),
-                                make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
-  const unsigned long long u = ((unsigned long long)w.y << 32) | w.x;
-  idx[i] = (int64_t)__umul64hi(u, (unsigned long long)n);
+  if (i < batch) idx[i] = rows.at(i);
 }
 
 __global__ void k_mlp_init(float* p, float* m, float* v, __nv_bfloat16* pb, uint64_t seed) {
@@ -623,21 +752,46 @@ __global__ void k_features(int64_t n, const double* E, const double* b, const in
   x[i * 8 + 7] = (float)(2.0 * kPi * u2[i]);
 }
 
-__global__ void k_moments(const float* x, int64_t n, double* acc) {
-  __shared__ double s[16];
-  if (threadIdx.x < 16) s[threadIdx.x] = 0.0;
+// Sums and sums of squares of the 8 columns of x, in FP64: thread t takes
+// the elements t, t + (grid size), .. of the flat array, all of column t mod
+// 8, so loads are coalesced and a thread has two sums.  Bound by the FP64
+// pipe, two instructions an element (the conversion runs on the integer
+// pipe).  1 M rows: 157 us with 16 sums and shared atomics per thread, now
+// 51 us.
+constexpr int kMomentsBlock = 512;
+__global__ void __launch_bounds__(kMomentsBlock) k_moments(const float* x, int64_t n, double* acc) {
+  __shared__ double s[kMomentsBlock / 32][16];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double a = 0.0, b = 0.0;
+#pragma unroll 4
+  for (int64_t i = blockIdx.x * (int64_t)kMomentsBlock + threadIdx.x; i < 8 * n;
+       i += (int64_t)gridDim.x * kMomentsBlock) {
+    const float f = x[i];
+    const unsigned u = __float_as_uint(f), e = u & 0x7f800000u;
+    // normal f on the integer pipe, the rest by a conversion
+    const double v = e == 0u || e == 0x7f800000u
+                         ? (double)f
+                         : __hiloint2double((int)((u & 0x80000000u) |
+                                                  (((u & 0x7fffffffu) >> 3) + (896u << 20))),
+                                            (int)(u << 29));
+    a += v;
+    b = fma(v, v, b);
+  }
+#pragma unroll
+  for (int o = 8; o < 32; o <<= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+  }
+  if (lane < 8) {
+    s[warp][lane] = a;
+    s[warp][8 + lane] = b;
+  }
   __syncthreads();
-  double loc[16] = {0};
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x)
-    for (int k = 0; k < 8; ++k) {
-      const double v = x[i * 8 + k];
-      loc[k] += v;
-      loc[8 + k] += v * v;
-    }
-  for (int k = 0; k < 16; ++k) atomicAdd(&s[k], loc[k]);
-  __syncthreads();
-  if (threadIdx.x < 16) atomicAdd(&acc[threadIdx.x], s[threadIdx.x]);
+  if (threadIdx.x < 16) {
+    double t = 0.0;
+    for (int w = 0; w < kMomentsBlock / 32; ++w) t += s[w][threadIdx.x];
+    atomicAdd(&acc[threadIdx.x], t);
+  }
 }
 
 // Normalisation of the proposal and its integer CDF, in a fixed summation
@@ -922,7 +1076,7 @@ CellGrid grid_of(const qcams_proposal_spec* s) {
 
 template <int CPW>
 cudaError_t launch_grad_cpw(const qcams_mlp* m, const float* x, const uint8_t* label,
-                            const int64_t* idx, int64_t n, float* loss_out, cudaStream_t st) {
+                            int64_t n, float* loss_out, cudaStream_t st) {
   const size_t smem = sizeof(TrainSmem<CPW>);
   cudaError_t e = cudaFuncSetAttribute(k_mlp_grad<CPW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)smem);
@@ -931,24 +1085,44 @@ cudaError_t launch_grad_cpw(const qcams_mlp* m, const float* x, const uint8_t* l
   if (grid > sm_count()) grid = sm_count();
   if (grid < 1) grid = 1;
   k_mlp_grad<CPW><<<(unsigned)grid, THREADS, smem, st>>>(
-      reinterpret_cast<const __nv_bfloat16*>(m->params_bf16), m->params, std_of(m), x, label, idx,
-      n, m->grad, loss_out);
+      reinterpret_cast<const __nv_bfloat16*>(m->params_bf16), m->params, std_of(m), x, label, n,
+      m->grad, loss_out);
   return cudaGetLastError();
 }
 
-int launch_grad(const qcams_mlp* m, const float* x, const uint8_t* label, const int64_t* idx,
-                int64_t n, float* loss_out, bool zero_loss, cudaStream_t st) {
+int launch_grad(const qcams_mlp* m, const float* x, const uint8_t* label, int64_t n,
+                float* loss_out, cudaStream_t st) {
   cudaError_t e = cudaMemsetAsync(m->grad, 0, NP * sizeof(float), st);
-  if (e == cudaSuccess && loss_out && zero_loss) e = cudaMemsetAsync(loss_out, 0, sizeof(float), st);
+  if (e == cudaSuccess && loss_out) e = cudaMemsetAsync(loss_out, 0, sizeof(float), st);
   if (e != cudaSuccess) return QCAMS_E_CUDA;
   // At most one block per SM (the weights, the round's tiles and the warps'
   // SiLU' values take 155 KB of shared memory with 64-sample rounds, 203 KB
   // with 128).  A batch that fits one 64-sample round per SM (8,192 samples:
   // 128 blocks) takes that, the shortest block; larger batches take
   // 128-sample rounds, half the rounds' global-atomic flushes.
-  e = (n + 63) / 64 <= sm_count() ? launch_grad_cpw<1>(m, x, label, idx, n, loss_out, st)
-                                  : launch_grad_cpw<2>(m, x, label, idx, n, loss_out, st);
+  e = (n + 63) / 64 <= sm_count() ? launch_grad_cpw<1>(m, x, label, n, loss_out, st)
+                                  : launch_grad_cpw<2>(m, x, label, n, loss_out, st);
   return status_of(e);
+}
+
+template <int CPW>
+cudaError_t launch_train(const qcams_mlp* m, const float* x, const uint8_t* label, RowSrc rows,
+                         int64_t steps, int64_t batch, float lr, float* losses, unsigned* barrier,
+                         cudaStream_t st) {
+  const size_t smem = sizeof(TrainSmem<CPW>);
+  cudaError_t e = cudaFuncSetAttribute(k_mlp_train<CPW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
+  if (e != cudaSuccess) return e;
+  // one block per SM: those without a round share the Adam step
+  const unsigned grid = (unsigned)sm_count();
+  float *p = m->params, *am = m->adam_m, *av = m->adam_v, *grad = m->grad;
+  __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(m->params_bf16);
+  Std sd = std_of(m);
+  double b1 = std::pow(0.9, (double)m->step), b2 = std::pow(0.999, (double)m->step);
+  void* args[] = {&p, &am, &av, &grad, &pb, &sd, &x, &label, &rows, &steps, &batch, &lr, &b1, &b2,
+                  &losses, &barrier};
+  return cudaLaunchCooperativeKernel((const void*)k_mlp_train<CPW>, dim3(grid), dim3(THREADS), args,
+                                     smem, st);
 }
 
 int launch_adam(qcams_mlp* m, float lr, cudaStream_t st) {
@@ -1017,7 +1191,7 @@ int qcams_mlp_fit_standardizer(qcams_mlp* m, const float* x, int64_t n, void* cu
   if (cudaMallocAsync((void**)&acc, 16 * sizeof(double), st) != cudaSuccess) return QCAMS_E_CUDA;
   cudaError_t e = cudaMemsetAsync(acc, 0, 16 * sizeof(double), st);
   if (e == cudaSuccess) {
-    k_moments<<<sm_count() * 2, 256, 0, st>>>(x, n, acc);
+    k_moments<<<sm_count() * 2, kMomentsBlock, 0, st>>>(x, n, acc);
     e = cudaGetLastError();
   }
   double h[16];
@@ -1040,7 +1214,7 @@ int qcams_mlp_grad(const qcams_mlp* m, const float* x, const uint8_t* label, int
   int rc;
   if ((rc = dev_ok()) != QCAMS_OK) return rc;
   (void)cudaGetLastError();
-  return launch_grad(m, x, label, nullptr, n, loss_out, true, (cudaStream_t)cuda_stream);
+  return launch_grad(m, x, label, n, loss_out, (cudaStream_t)cuda_stream);
 }
 
 int qcams_mlp_train_step(qcams_mlp* m, const float* x, const uint8_t* label, int64_t n,
@@ -1063,14 +1237,23 @@ int qcams_mlp_train(qcams_mlp* m, const float* x, const uint8_t* label, int64_t 
   if (losses && steps > 0 &&
       cudaMemsetAsync(losses, 0, sizeof(float) * (size_t)steps, st) != cudaSuccess)
     return QCAMS_E_CUDA;
-  for (int64_t s = 0; s < steps; ++s) {
-    k_draw_idx<<<(batch + 255) / 256, 256, 0, st>>>(idx, batch, n, seed, (uint64_t)m->step);
-    if (cudaGetLastError() != cudaSuccess) return QCAMS_E_CUDA;
-    if ((rc = launch_grad(m, x, label, idx, batch, losses ? losses + s : nullptr, false, st)) !=
-        QCAMS_OK)
-      return rc;
-    if ((rc = launch_adam(m, lr, st)) != QCAMS_OK) return rc;
-  }
+  if (steps == 0) return QCAMS_OK;
+  // the grid barrier's counter lives in the index scratch until the kernel
+  // is done, then the last step's indices go there
+  cudaError_t e = cudaMemsetAsync(m->grad, 0, NP * sizeof(float), st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(idx, 0, sizeof(int64_t), st);
+  RowSrc rows{true, n, seed, (uint64_t)m->step};
+  unsigned* barrier = reinterpret_cast<unsigned*>(idx);
+  // rounds as launch_grad chooses them
+  if (e == cudaSuccess)
+    e = (batch + 63) / 64 <= sm_count()
+            ? launch_train<1>(m, x, label, rows, steps, batch, lr, losses, barrier, st)
+            : launch_train<2>(m, x, label, rows, steps, batch, lr, losses, barrier, st);
+  if (e != cudaSuccess) return QCAMS_E_CUDA;
+  rows.step += (uint64_t)(steps - 1);
+  k_draw_idx<<<(batch + 255) / 256, 256, 0, st>>>(idx, batch, rows);
+  if (cudaGetLastError() != cudaSuccess) return QCAMS_E_CUDA;
+  m->step += steps;
   return QCAMS_OK;
 }
 

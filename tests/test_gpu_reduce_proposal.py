@@ -49,7 +49,8 @@ def test_reduce_matches_counts(Q, n, n_cells, weighted, sort):
     assert np.array_equal(hist.cpu().numpy(), want)
     host, _ = Q.xsec_from_hist(want, np.ones(n_cells), np.ones(n_cells), np.zeros(n_cells), 1,
                                weighted=weighted)
-    assert np.array_equal(cells, host)
+    # a cell with more failures than outcomes has no error estimate (NaN) in class 5
+    assert np.array_equal(cells, host, equal_nan=True)
 
 
 @pytest.mark.gpu
