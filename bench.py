@@ -50,12 +50,13 @@ if ROOT not in sys.path:
 #   fraction of the FP64 pipe's instruction rate the kernel uses.
 FP64_FLOP_PER_STEP = 858
 FP64_INSTR_PER_STEP = 516
-#   FP32: 393 FFMA + 178 FMUL + 39 FADD = 1,004 FLOP and one DADD (the
-#   time) in 787 thread instructions per step (all pipes); the kernel is
-#   bound by instruction issue, so issue_frac below is the fraction of the
-#   SMs' issue rate (4 warp instructions per SM per cycle) it uses.
+#   FP32: 393 multiply-adds, 178 products and 39 sums = 1,004 FLOP and one
+#   DADD (the time), most of them two to a packed instruction, in 628
+#   thread instructions per step (all pipes, 400,000 sweep lanes capped at
+#   200 attempts); issue_frac below is the fraction of the SMs' issue rate
+#   (4 warp instructions per SM per cycle) they use.
 FP32_FLOP_PER_STEP = 1004
-FP32_THREAD_INSTR_PER_STEP = 787
+FP32_THREAD_INSTR_PER_STEP = 628
 KERNEL_SOURCES = {
     64: ["integrate.cu", "elem64.cuh", "ff.cuh", "texp.cuh", "exp2_table.inc",
          "dp5_tableau.cuh", "step_ctrl.cuh", "pair_force.cuh", "regop.cuh"],
@@ -63,7 +64,7 @@ KERNEL_SOURCES = {
 }
 COUNTS_SOURCE_SHA256 = {
     64: "d5c569ad3189817afd99549d55eb8ecb1a26b4d4691dcbe3ce9f99dc33bb0e57",
-    32: "70e2932855a88f714f4f7b48b180d82a8b03cd6726c5035bdfd2c9d94b9bb1c1",
+    32: "d9cbe3757a6014589cdc38132e600b44ad5e99066d6bdb99841805d6197d8421",
 }
 # DRAM bytes per trajectory of the integrator: ncu dram__bytes_read.sum +
 # dram__bytes_write.sum of the same FP64 profile case (1,110,784 B read,

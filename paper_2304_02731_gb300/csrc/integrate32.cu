@@ -20,6 +20,8 @@
 //    loads the FP64 state as (float, compensation) and stores y - c in FP64.
 #include <cuda_runtime.h>
 
+#include <cstring>
+
 #include "dp5_tableau.cuh"
 #include "qcams_device.cuh"
 #include "qcams_internal.h"
@@ -41,7 +43,6 @@ __host__ __device__ constexpr RknTabF make_rkn_tab_f() {
   }
   return f;
 }
-__constant__ RknTabF kTf = make_rkn_tab_f();
 
 constexpr unsigned FULL = 0xffffffffu;
 
@@ -82,6 +83,100 @@ __device__ __forceinline__ float pow_m01(float x) {
   return r;
 }
 
+// Two FP32 values in one aligned register pair, with the packed multiply-add,
+// multiply and add of sm_100: one instruction for two IEEE operations (each
+// half rounds as the scalar instruction does).
+struct F2 {
+  unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float lo, float hi) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float lo_of(F2 a) {
+  float l, h;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(l), "=f"(h) : "l"(a.v));
+  return l;
+}
+__device__ __forceinline__ float hi_of(F2 a) {
+  float l, h;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(l), "=f"(h) : "l"(a.v));
+  return h;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 dup(float a) { return f2(a, a); }
+// a - b: b's sign flips inside the (exact) product with -1
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) { return fma2(b, F2{0xbf800000bf800000ull}, a); }
+// The six components of a pair of Jacobi vectors are held as (0, 1), (3, 4)
+// and (2, 5): the pair vectors rho2 - cB rho1 and rho2 + cA rho1 then take
+// one packed and one scalar multiply-add each.
+struct V6 {
+  F2 a, b, c;
+};
+__device__ __forceinline__ void get6(const V6& v, float* x) {
+  x[0] = lo_of(v.a);
+  x[1] = hi_of(v.a);
+  x[2] = lo_of(v.c);
+  x[3] = lo_of(v.b);
+  x[4] = hi_of(v.b);
+  x[5] = hi_of(v.c);
+}
+__device__ __forceinline__ V6 put6(const float* x) {
+  return V6{f2(x[0], x[1]), f2(x[3], x[4]), f2(x[2], x[5])};
+}
+__device__ __forceinline__ V6 fma6(F2 w, const V6& x, const V6& y) {
+  return V6{fma2(w, x.a, y.a), fma2(w, x.b, y.b), fma2(w, x.c, y.c)};
+}
+__device__ __forceinline__ V6 mul6(F2 w, const V6& x) {
+  return V6{mul2(w, x.a), mul2(w, x.b), mul2(w, x.c)};
+}
+__device__ __forceinline__ V6 add6(const V6& x, const V6& y) {
+  return V6{add2(x.a, y.a), add2(x.b, y.b), add2(x.c, y.c)};
+}
+__device__ __forceinline__ V6 sub6(const V6& x, const V6& y) {
+  return V6{sub2(x.a, y.a), sub2(x.b, y.b), sub2(x.c, y.c)};
+}
+__device__ __forceinline__ F2 sel2(bool p, F2 a, F2 b) { return F2{p ? a.v : b.v}; }
+__device__ __forceinline__ V6 sel6(bool p, const V6& x, const V6& y) {
+  return V6{sel2(p, x.a, y.a), sel2(p, x.b, y.b), sel2(p, x.c, y.c)};
+}
+
+// The Runge-Kutta-Nystrom coefficients, each in both halves of a pair.
+struct RknTab2 {
+  F2 a2[8][8], b[8], e[8], ea[8];
+};
+constexpr F2 both(float x) {
+  const unsigned long long u = __builtin_bit_cast(unsigned, x);
+  return F2{u << 32 | u};
+}
+constexpr RknTab2 make_rkn_tab2() {
+  RknTab2 t{};
+  const RknTabF f = make_rkn_tab_f();
+  for (int s = 1; s <= 7; ++s) {
+    t.b[s] = both(f.b[s]);
+    t.e[s] = both(f.e[s]);
+    t.ea[s] = both(f.ea[s]);
+    for (int q = 1; q <= 7; ++q) t.a2[s][q] = both(f.a2[s][q]);
+  }
+  return t;
+}
+__constant__ RknTab2 kT2 = make_rkn_tab2();
+
 // FP32 copies of the per-system constants (built on the host, so the kernel
 // never converts doubles in its inner loop).
 struct PairF {
@@ -95,6 +190,9 @@ struct SysF {
   float kf[5], kf_morse[5];
   double mu12d, mu123d;
   PairF pair[3];
+  // packed operands: (-cB, -cB), (cA, cA); of the pairs BC and CA the Morse
+  // exponent's -l0 and l1 and the force coefficients (f1, f2) and (h1, h2)
+  F2 ncB, cA2, nl0, l1, f12, h12;
 };
 struct SysSetF {
   SysF s[QCAMS_MAX_SYS];
@@ -140,34 +238,45 @@ __device__ __forceinline__ float pair_u(const PairF& q, float s) {
 }
 
 template <bool MORSE>
-__device__ __forceinline__ void accel(const SysF& S, const float* x, float* a, float* s2) {
-  const float rbc0 = fmaf(-S.cB, x[0], x[3]), rbc1 = fmaf(-S.cB, x[1], x[4]),
-              rbc2 = fmaf(-S.cB, x[2], x[5]);
-  const float rca0 = fmaf(S.cA, x[0], x[3]), rca1 = fmaf(S.cA, x[1], x[4]),
-              rca2 = fmaf(S.cA, x[2], x[5]);
-  s2[0] = fmaf(x[0], x[0], fmaf(x[1], x[1], x[2] * x[2]));
+__device__ __forceinline__ void accel(const SysF& S, const V6& x, V6& a, float* s2) {
+  const F2 bc = fma2(S.ncB, x.a, x.b), ca = fma2(S.cA2, x.a, x.b);
+  const float x0 = lo_of(x.a), x1 = hi_of(x.a), x2 = lo_of(x.c);
+  const float rbc0 = lo_of(bc), rbc1 = hi_of(bc), rbc2 = fmaf(-S.cB, x2, hi_of(x.c));
+  const float rca0 = lo_of(ca), rca1 = hi_of(ca), rca2 = fmaf(S.cA, x2, hi_of(x.c));
+  s2[0] = fmaf(x0, x0, fmaf(x1, x1, x2 * x2));
   s2[1] = fmaf(rbc0, rbc0, fmaf(rbc1, rbc1, rbc2 * rbc2));
   s2[2] = fmaf(rca0, rca0, fmaf(rca1, rca1, rca2 * rca2));
+  float f0, f1, f2_, h1, h2;
   const float u0 = pair_u<MORSE>(S.pair[0], s2[0]);
-  const float u1 = pair_u<MORSE>(S.pair[1], s2[1]);
-  const float u2 = pair_u<MORSE>(S.pair[2], s2[2]);
-  const float f0 = (MORSE ? S.kf_morse[0] : S.kf[0]) * u0;
-  const float f1 = (MORSE ? S.kf_morse[1] : S.kf[1]) * u1;
-  const float f2 = (MORSE ? S.kf_morse[2] : S.kf[2]) * u2;
-  const float h1 = (MORSE ? S.kf_morse[3] : S.kf[3]) * u1;
-  const float h2 = (MORSE ? S.kf_morse[4] : S.kf[4]) * u2;
-  a[0] = fmaf(f0, x[0], fmaf(f1, rbc0, f2 * rca0));
-  a[1] = fmaf(f0, x[1], fmaf(f1, rbc1, f2 * rca1));
-  a[2] = fmaf(f0, x[2], fmaf(f1, rbc2, f2 * rca2));
-  a[3] = fmaf(h1, rbc0, h2 * rca0);
-  a[4] = fmaf(h1, rbc1, h2 * rca1);
-  a[5] = fmaf(h1, rbc2, h2 * rca2);
+  if (MORSE) {
+    f0 = S.kf_morse[0] * u0;
+    // pairs BC and CA packed (pair_u's operations)
+    const float i1 = rsqrt_approx(s2[1]), i2 = rsqrt_approx(s2[2]);
+    const F2 ri = f2(i1, i2), arg = fma2(S.nl0, mul2(f2(s2[1], s2[2]), ri), S.l1);
+    const float e1 = ex2_approx(lo_of(arg)), e2 = ex2_approx(hi_of(arg));
+    const F2 u = mul2(f2(fmaf(-e1, e1, e1), fmaf(-e2, e2, e2)), ri);
+    const F2 f = mul2(S.f12, u), h = mul2(S.h12, u);
+    f1 = lo_of(f);
+    f2_ = hi_of(f);
+    h1 = lo_of(h);
+    h2 = hi_of(h);
+  } else {
+    const float u1 = pair_u<MORSE>(S.pair[1], s2[1]), u2 = pair_u<MORSE>(S.pair[2], s2[2]);
+    f0 = S.kf[0] * u0;
+    f1 = S.kf[1] * u1;
+    f2_ = S.kf[2] * u2;
+    h1 = S.kf[3] * u1;
+    h2 = S.kf[4] * u2;
+  }
+  a.a = f2(fmaf(f0, x0, fmaf(f1, rbc0, f2_ * rca0)), fmaf(f0, x1, fmaf(f1, rbc1, f2_ * rca1)));
+  a.b = f2(fmaf(h1, rbc0, h2 * rca0), fmaf(h1, rbc1, h2 * rca1));
+  a.c = f2(fmaf(f0, x2, fmaf(f1, rbc2, f2_ * rca2)), fmaf(h1, rbc2, h2 * rca2));
 }
 
 struct Lane32 {
-  float rho[6], vel[6];   // state (true value = state - compensation)
-  float crho[6], cvel[6]; // Kahan compensations
-  float acc[7][6];
+  V6 rho, vel;       // state (true value = state - compensation)
+  V6 ncrho, ncvel;   // Kahan compensations, negated
+  V6 acc[7];
   double t, tmax;
   float h;
   float atv[2];
@@ -176,10 +285,22 @@ struct Lane32 {
   bool rejected;
 };
 
+// atol + rtol max(|a|, |b|), halves apart.
+__device__ __forceinline__ F2 scale2(F2 rt, F2 at, F2 a, F2 b) {
+  return fma2(rt, f2(fmaxf(fabsf(lo_of(a)), fabsf(lo_of(b))), fmaxf(fabsf(hi_of(a)), fabsf(hi_of(b)))),
+              at);
+}
+__device__ __forceinline__ F2 rcp2(F2 a) { return f2(rcp_approx(lo_of(a)), rcp_approx(hi_of(a))); }
+
 // One adaptive attempt (SciPy RK45 rules, as in the FP64 integrator), all
 // stages in FP32; the accepted increments are added with compensation.
 // ONE: the batch has a single system, so its constants are read with a
 // compile-time index (constant-bank operands, no per-lane indexed loads).
+// Every linear combination of 6-vectors runs in packed instructions: 628
+// instructions a step instead of 787, which bound the kernel by issue (79 %
+// of the rate); it now waits on the FMA pipes' bursts and on latency with 16
+// warps per SM (issue 69 %, FMA pipes 68 %).  The full sweep: 117.6 -> 110.7
+// ms.
 template <bool MORSE, bool ONE>
 __device__ __forceinline__ void attempt(const SysSetF& sys, const IntegParams& ip, Lane32& L) {
   const SysF& S = sys.s[ONE ? 0 : L.sid];
@@ -192,27 +313,17 @@ __device__ __forceinline__ void attempt(const SysSetF& sys, const IntegParams& i
     }
   }
   const float h = L.h, hh = h * h;
-  float x[6], s2[3];
+  const F2 h2 = dup(h), hh2 = dup(hh);
+  V6 x;
+  float s2[3];
 #define QCAMS_STAGE(sIdx)                                                            \
   {                                                                                  \
-    const float hc = h * (float)dpC(sIdx); /* folded: c_6 = 1 */                     \
-    float w[(sIdx) - 2];                                                             \
+    x = fma6(dup(h * (float)dpC(sIdx)), L.vel, L.rho); /* folded: c_6 = 1 */         \
     _Pragma("unroll") for (int q = 1; q <= (sIdx) - 2; ++q)                          \
-        w[q - 1] = hh * kTf.a2[sIdx][q];                                             \
-    _Pragma("unroll") for (int i = 0; i < 6; ++i) {                                  \
-      float xi = fmaf(hc, L.vel[i], L.rho[i]);                                       \
-      _Pragma("unroll") for (int q = 1; q <= (sIdx) - 2; ++q)                        \
-          if (!dpA2Zero(sIdx, q)) xi = fmaf(w[q - 1], L.acc[q - 1][i], xi);          \
-      x[i] = xi;                                                                     \
-    }                                                                                \
+        if (!dpA2Zero(sIdx, q)) x = fma6(mul2(hh2, kT2.a2[sIdx][q]), L.acc[q - 1], x); \
     accel<MORSE>(S, x, L.acc[(sIdx) - 1], s2);                                       \
   }
-  {  // stage 2: (A^2)_{2q} = 0, no acceleration term
-    const float hc = h * (float)dpC(2);
-#pragma unroll
-    for (int i = 0; i < 6; ++i) x[i] = fmaf(hc, L.vel[i], L.rho[i]);
-    accel<MORSE>(S, x, L.acc[1], s2);
-  }
+  QCAMS_STAGE(2)   // (A^2)_{2q} = 0, no acceleration term
   QCAMS_STAGE(3)
   QCAMS_STAGE(4)
   QCAMS_STAGE(5)
@@ -220,48 +331,40 @@ __device__ __forceinline__ void attempt(const SysSetF& sys, const IntegParams& i
 #undef QCAMS_STAGE
   // stage 7 = the new state: increment d = h v + h^2 sum (b^T A)_q a_q,
   // compensated sum x7 = rho + (d - c)
-  float yr[6];
+  V6 sum{F2{0}, F2{0}, F2{0}};
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    float sum = 0.0f;
-#pragma unroll
-    for (int q = 1; q <= 5; ++q)
-      if (!dpA2Zero(7, q)) sum = fmaf(kTf.a2[7][q], L.acc[q - 1][i], sum);
-    const float d = fmaf(hh, sum, h * L.vel[i]);
-    yr[i] = d - L.crho[i];
-    x[i] = L.rho[i] + yr[i];
-  }
+  for (int q = 1; q <= 5; ++q)
+    if (!dpA2Zero(7, q)) sum = fma6(kT2.a2[7][q], L.acc[q - 1], sum);
+  const V6 yr = add6(fma6(hh2, sum, mul6(h2, L.vel)), L.ncrho);
+  x = add6(L.rho, yr);
   accel<MORSE>(S, x, L.acc[6], s2);
-  float dv[6], er[6], ev[6];
+  V6 vb = mul6(kT2.b[1], L.acc[0]);
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    float vb = kTf.b[1] * L.acc[0][i];
+  for (int q = 3; q <= 6; ++q) vb = fma6(kT2.b[q], L.acc[q - 1], vb);
+  V6 ev = mul6(kT2.e[1], L.acc[0]);     // velocity error / h
 #pragma unroll
-    for (int q = 3; q <= 6; ++q) vb = fmaf(kTf.b[q], L.acc[q - 1][i], vb);
-    dv[i] = h * vb;
-    float e = kTf.e[1] * L.acc[0][i];
+  for (int q = 3; q <= 7; ++q) ev = fma6(kT2.e[q], L.acc[q - 1], ev);
+  V6 er = mul6(kT2.ea[1], L.acc[0]);    // position error / h^2
 #pragma unroll
-    for (int q = 3; q <= 7; ++q) e = fmaf(kTf.e[q], L.acc[q - 1][i], e);
-    ev[i] = e;   // velocity error / h
-    float ea = kTf.ea[1] * L.acc[0][i];
-#pragma unroll
-    for (int q = 2; q <= 6; ++q)
-      if (!dpEAZero(q)) ea = fmaf(kTf.ea[q], L.acc[q - 1][i], ea);
-    er[i] = ea;  // position error / h^2
-  }
+  for (int q = 2; q <= 6; ++q)
+    if (!dpEAZero(q)) er = fma6(kT2.ea[q], L.acc[q - 1], er);
+  const V6 yv = fma6(h2, vb, L.ncvel);  // h vb - c
+  const V6 vn = add6(L.vel, yv);
   // the factors h and h^2 multiply the two partial sums of squares once
-  float sum_r = 0.0f, sum_v = 0.0f;
-  float vn[6], yv[6];
+  const F2 rt = dup(ip.rtol_f), at = dup(ip.atol_f);
+  const V6 qr{mul2(er.a, rcp2(scale2(rt, at, L.rho.a, x.a))),
+              mul2(er.b, rcp2(scale2(rt, at, L.rho.b, x.b))),
+              mul2(er.c, rcp2(scale2(rt, at, L.rho.c, x.c)))};
+  const V6 qv{mul2(ev.a, rcp2(scale2(rt, dup(L.atv[0]), L.vel.a, vn.a))),
+              mul2(ev.b, rcp2(scale2(rt, dup(L.atv[1]), L.vel.b, vn.b))),
+              mul2(ev.c, rcp2(scale2(rt, f2(L.atv[0], L.atv[1]), L.vel.c, vn.c)))};
+  float sum_r = 0.0f, sum_v = 0.0f, tr[6], tv[6];
+  get6(qr, tr);
+  get6(qv, tv);
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
-    yv[i] = dv[i] - L.cvel[i];
-    vn[i] = L.vel[i] + yv[i];
-    const float scr = fmaf(ip.rtol_f, fmaxf(fabsf(L.rho[i]), fabsf(x[i])), ip.atol_f);
-    const float qr = er[i] * rcp_approx(scr);
-    const float scv = fmaf(ip.rtol_f, fmaxf(fabsf(L.vel[i]), fabsf(vn[i])), L.atv[i / 3]);
-    const float qv = ev[i] * rcp_approx(scv);
-    sum_r = fmaf(qr, qr, sum_r);
-    sum_v = fmaf(qv, qv, sum_v);
+    sum_r = fmaf(tr[i], tr[i], sum_r);
+    sum_v = fmaf(tv[i], tv[i], sum_v);
   }
   const float en2 = fmaf(hh, sum_v, (hh * hh) * sum_r) * (1.0f / 12.0f);
   L.calls += 1;
@@ -277,21 +380,18 @@ __device__ __forceinline__ void attempt(const SysSetF& sys, const IntegParams& i
   const double tn = L.t + (double)L.h;
   L.t = accept ? tn : L.t;
   L.h = L.h * f;
-#pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const float cr = (x[i] - L.rho[i]) - yr[i];
-    const float cv = (vn[i] - L.vel[i]) - yv[i];
-    L.crho[i] = accept ? cr : L.crho[i];
-    L.cvel[i] = accept ? cv : L.cvel[i];
-    L.rho[i] = accept ? x[i] : L.rho[i];
-    L.vel[i] = accept ? vn[i] : L.vel[i];
-    L.acc[0][i] = accept ? L.acc[6][i] : L.acc[0][i];
-  }
+  // new compensation (x - rho) - y, negated
+  L.ncrho = sel6(accept, sub6(yr, sub6(x, L.rho)), L.ncrho);
+  L.ncvel = sel6(accept, sub6(yv, sub6(vn, L.vel)), L.ncvel);
+  L.rho = sel6(accept, x, L.rho);
+  L.vel = sel6(accept, vn, L.vel);
+  L.acc[0] = sel6(accept, L.acc[6], L.acc[0]);
   L.nacc += accept ? 1 : 0;
   L.nrej += accept ? 0 : 1;
   L.rejected = !accept;
   const float smax = fmaxf(s2[0], fmaxf(s2[1], s2[2]));
-  const float radial = fmaf(L.rho[3], L.vel[3], fmaf(L.rho[4], L.vel[4], L.rho[5] * L.vel[5]));
+  const float radial = fmaf(lo_of(L.rho.b), lo_of(L.vel.b),
+                            fmaf(hi_of(L.rho.b), hi_of(L.vel.b), hi_of(L.rho.c) * hi_of(L.vel.c)));
   bool collapse = false;
   if (!MORSE) {
 #pragma unroll
@@ -308,33 +408,42 @@ __device__ __forceinline__ void attempt(const SysSetF& sys, const IntegParams& i
   L.status = st;
 }
 
-// Starting step (Hairer, Norsett & Wanner), in FP32.
+// Starting step (Hairer, Norsett & Wanner), in FP32.  The multiply-adds are
+// written out, so that the sums round the same in every kernel.
+__device__ __forceinline__ float add_squares(float s, float a, float b) {
+  return __fadd_rn(s, fmaf(a, a, __fmul_rn(b, b)));
+}
 template <bool MORSE>
 __device__ float initial_step(const SysF& S, const Lane32& L, float rtol, float atol) {
-  float d0 = 0.f, d1 = 0.f;
+  float d0 = 0.f, d1 = 0.f, rho[6], vel[6], acc0[6];
+  get6(L.rho, rho);
+  get6(L.vel, vel);
+  get6(L.acc[0], acc0);
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
-    const float scr = atol + fabsf(L.rho[i]) * rtol;
-    const float scv = L.atv[i / 3] + fabsf(L.vel[i]) * rtol;
-    const float q0 = L.rho[i] / scr, q1 = L.vel[i] / scv;
-    d0 += q0 * q0 + q1 * q1;
-    const float p0 = L.vel[i] / scr, p1 = L.acc[0][i] / scv;
-    d1 += p0 * p0 + p1 * p1;
+    const float scr = fmaf(fabsf(rho[i]), rtol, atol);
+    const float scv = fmaf(fabsf(vel[i]), rtol, L.atv[i / 3]);
+    const float q0 = rho[i] / scr, q1 = vel[i] / scv;
+    d0 = add_squares(d0, q0, q1);
+    const float p0 = vel[i] / scr, p1 = acc0[i] / scv;
+    d1 = add_squares(d1, p0, p1);
   }
   d0 = sqrtf(d0 / 12.f);
   d1 = sqrtf(d1 / 12.f);
   const float h0 = (d0 < 1e-5f || d1 < 1e-5f) ? 1e-6f : 0.01f * d0 / d1;
   float x1[6], a1[6], s2[3];
 #pragma unroll
-  for (int i = 0; i < 6; ++i) x1[i] = fmaf(h0, L.vel[i], L.rho[i]);
-  accel<MORSE>(S, x1, a1, s2);
+  for (int i = 0; i < 6; ++i) x1[i] = fmaf(h0, vel[i], rho[i]);
+  V6 av;
+  accel<MORSE>(S, put6(x1), av, s2);
+  get6(av, a1);
   float d2 = 0.f;
 #pragma unroll
   for (int i = 0; i < 6; ++i) {
-    const float scr = atol + fabsf(L.rho[i]) * rtol;
-    const float scv = L.atv[i / 3] + fabsf(L.vel[i]) * rtol;
-    const float p0 = h0 * L.acc[0][i] / scr, p1 = (a1[i] - L.acc[0][i]) / scv;
-    d2 += p0 * p0 + p1 * p1;
+    const float scr = fmaf(fabsf(rho[i]), rtol, atol);
+    const float scv = fmaf(fabsf(vel[i]), rtol, L.atv[i / 3]);
+    const float p0 = h0 * acc0[i] / scr, p1 = (a1[i] - acc0[i]) / scv;
+    d2 = add_squares(d2, p0, p1);
   }
   d2 = sqrtf(d2 / 12.f) / h0;
   const float h1 = (d1 <= 1e-15f && d2 <= 1e-15f) ? fmaxf(1e-6f, h0 * 1e-3f)
@@ -357,15 +466,20 @@ __device__ bool load(const SysSetF& sys, const DevShape* shapes, const IntegPara
     return false;
   }
   const SysF& S = sys.s[ONE ? 0 : L.sid];
+  float rho[6], vel[6], nr[6], nv[6];
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     const double r = B.y[k][i];
     const double v = B.y[6 + k][i] * (k < 3 ? 1.0 / S.mu12d : 1.0 / S.mu123d);
-    L.rho[k] = (float)r;
-    L.crho[k] = (float)((double)L.rho[k] - r);
-    L.vel[k] = (float)v;
-    L.cvel[k] = (float)((double)L.vel[k] - v);
+    rho[k] = (float)r;
+    nr[k] = -(float)((double)rho[k] - r);
+    vel[k] = (float)v;
+    nv[k] = -(float)((double)vel[k] - v);
   }
+  L.rho = put6(rho);
+  L.vel = put6(vel);
+  L.ncrho = put6(nr);
+  L.ncvel = put6(nv);
   L.t = B.t[i];
   L.h = (float)B.h[i];
   L.tmax = ip.t_stop * B.t_scale[i];
@@ -392,10 +506,15 @@ __device__ bool load(const SysSetF& sys, const DevShape* shapes, const IntegPara
 template <bool ONE>
 __device__ void store(const SysSetF& sys, const DevBatch& B, int64_t i, const Lane32& L) {
   const SysF& S = sys.s[ONE ? 0 : L.sid];
+  float rho[6], vel[6], nr[6], nv[6];
+  get6(L.rho, rho);
+  get6(L.vel, vel);
+  get6(L.ncrho, nr);
+  get6(L.ncvel, nv);
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
-    B.y[k][i] = (double)L.rho[k] - (double)L.crho[k];
-    B.y[6 + k][i] = ((double)L.vel[k] - (double)L.cvel[k]) * (k < 3 ? S.mu12d : S.mu123d);
+    B.y[k][i] = (double)rho[k] + (double)nr[k];
+    B.y[6 + k][i] = ((double)vel[k] + (double)nv[k]) * (k < 3 ? S.mu12d : S.mu123d);
   }
   B.t[i] = L.t;
   B.h[i] = (double)L.h;
@@ -433,8 +552,14 @@ __global__ void __launch_bounds__(128) k_integrate32_plain(SysSetF sys, const De
   flush(rhs, steps, counters);
 }
 
-template <bool MORSE, bool ONE>
-__global__ void __launch_bounds__(128) k_integrate32_persistent(SysSetF sys,
+// MINB resident blocks per SM cap the registers: the all-Morse kernel takes
+// 121, four blocks of 128 threads (five, at 96 registers, spill and run the
+// sweep in 115.8 ms against 110.7); the generic one 120 or, with five blocks
+// and 100 bytes of spills, 96: 35.8 against 37.9 ms for 1 M lanes, but 8.4
+// against 8.3 ms for 9,999, which four blocks per SM hold at once and whose
+// longest lanes set the time.
+template <bool MORSE, bool ONE, int MINB>
+__global__ void __launch_bounds__(128, MINB) k_integrate32_persistent(SysSetF sys,
                                                                 const DevShape* shapes,
                                                                 IntegParams ip, DevBatch B,
                                                                 unsigned long long* counters) {
@@ -507,31 +632,50 @@ SysSetF to_float(const SysSet& in) {
       g.l0 = (float)((q.kind == QCAMS_BUCK ? q.lc2 : q.c0) * log2e);
       g.l1 = (float)(q.c1 * log2e);
     }
+    auto pack = [](float lo, float hi) {
+      unsigned a, b;
+      std::memcpy(&a, &lo, 4);
+      std::memcpy(&b, &hi, 4);
+      return F2{(unsigned long long)b << 32 | a};
+    };
+    f.ncB = pack(-f.cB, -f.cB);
+    f.cA2 = pack(f.cA, f.cA);
+    f.nl0 = pack(-f.pair[1].l0, -f.pair[2].l0);
+    f.l1 = pack(f.pair[1].l1, f.pair[2].l1);
+    f.f12 = pack(f.kf_morse[1], f.kf_morse[2]);
+    f.h12 = pack(f.kf_morse[3], f.kf_morse[4]);
   }
   return o;
+}
+
+template <bool MORSE, bool ONE, int MINB>
+cudaError_t launch32_persistent(const SysSetF& sf, const DevShape* shapes, const IntegParams& ip,
+                                const DevBatch& b, Ctx& ctx, cudaStream_t st) {
+  const int block = 128;
+  cudaError_t e = cudaMemsetAsync(ctx.counters + 2, 0, sizeof(unsigned long long), st);
+  if (e != cudaSuccess) return e;
+  int per_sm = 0;
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      &per_sm, k_integrate32_persistent<MORSE, ONE, MINB>, block, 0);
+  if (e != cudaSuccess) return e;
+  long long grid = (long long)(per_sm < 1 ? 1 : per_sm) * ctx.sm_count;
+  const long long need_blocks = (b.n + block - 1) / block;
+  if (grid > need_blocks) grid = need_blocks;
+  if (grid < 1) grid = 1;
+  k_integrate32_persistent<MORSE, ONE, MINB><<<(unsigned)grid, block, 0, st>>>(sf, shapes, ip, b,
+                                                                              ctx.counters);
+  return cudaGetLastError();
 }
 
 template <bool MORSE, bool ONE>
 cudaError_t launch32(const SysSetF& sf, const DevShape* shapes, const IntegParams& ip,
                      const DevBatch& b, int persistent, Ctx& ctx, cudaStream_t st) {
-  const int block = 128;
-  if (persistent) {
-    cudaError_t e = cudaMemsetAsync(ctx.counters + 2, 0, sizeof(unsigned long long), st);
-    if (e != cudaSuccess) return e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm,
-                                                      k_integrate32_persistent<MORSE, ONE>, block, 0);
-    if (e != cudaSuccess) return e;
-    long long grid = (long long)(per_sm < 1 ? 1 : per_sm) * ctx.sm_count;
-    const long long need_blocks = (b.n + block - 1) / block;
-    if (grid > need_blocks) grid = need_blocks;
-    if (grid < 1) grid = 1;
-    k_integrate32_persistent<MORSE, ONE><<<(unsigned)grid, block, 0, st>>>(sf, shapes, ip, b,
-                                                                          ctx.counters);
-    return cudaGetLastError();
-  }
-  const unsigned grid = (unsigned)((b.n + block - 1) / block);
-  k_integrate32_plain<MORSE, ONE><<<grid, block, 0, st>>>(sf, shapes, ip, b, ctx.counters);
+  if (persistent)
+    return !MORSE && b.n > 4 * 128 * (int64_t)ctx.sm_count
+               ? launch32_persistent<MORSE, ONE, MORSE ? 4 : 5>(sf, shapes, ip, b, ctx, st)
+               : launch32_persistent<MORSE, ONE, 4>(sf, shapes, ip, b, ctx, st);
+  const unsigned grid = (unsigned)((b.n + 127) / 128);
+  k_integrate32_plain<MORSE, ONE><<<grid, 128, 0, st>>>(sf, shapes, ip, b, ctx.counters);
   return cudaGetLastError();
 }
 
