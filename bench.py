@@ -63,7 +63,7 @@ KERNEL_SOURCES = {
     32: ["integrate32.cu", "dp5_tableau.cuh"],
 }
 COUNTS_SOURCE_SHA256 = {
-    64: "d5c569ad3189817afd99549d55eb8ecb1a26b4d4691dcbe3ce9f99dc33bb0e57",
+    64: "cf67eb8adb5624b72744b7ef0d6d4d0e2fea000478fff561090cccdf7322210e",
     32: "d9cbe3757a6014589cdc38132e600b44ad5e99066d6bdb99841805d6197d8421",
 }
 # DRAM bytes per trajectory of the integrator: ncu dram__bytes_read.sum +

@@ -90,7 +90,8 @@ __device__ __forceinline__ double texp_hint(double x, float xa, const double* __
   const float P = __fmul_rn(rh, rh);
   const float Pl = fmaf(2.0f * rh, rl, fmaf(rh, rh, -P));   // r^2 = P + Pl to 2^-46
   const float cub = (P * rh) * (1.0f / 6.0f);
-  const double p = op.add(r, ff_to_double(0.5f * P, fmaf(0.5f, Pl, cub)));
+  // |Pl/2 + cub| is below 2^-11 P/2
+  const double p = op.add(r, ff_to_double<true>(0.5f * P, fmaf(0.5f, Pl, cub)));
   const double Tj = T[k & (kExpTableSize - 1)];
   const double y = fma(Tj, p, Tj);
   const double ex = __hiloint2double(__double2hiint(y) + ((k >> 11) << 20), __double2loint(y));

@@ -62,11 +62,14 @@ __device__ __forceinline__ void ff_dot_first(float& s, float& c, float wh, float
 // t + r = s + c, then r's significand is shifted into the 53-bit
 // significand of t (truncated below t's last double bit).  t = 0 (exact
 // cancellation) or a subnormal t gives 0; a subnormal r is dropped; an
-// infinite or NaN t gives NaN.
+// infinite or NaN t gives NaN.  ORDERED: |s| >= |c| or s = 0, where the
+// three-operation two-sum is error-free too (Dekker, Numer. Math. 18 (1971)).
+template <bool ORDERED = false>
 __device__ __forceinline__ double ff_to_double(float s, float c) {
   const float t = __fadd_rn(s, c);
   const float bb = __fsub_rn(t, s);
-  const float r = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(c, bb));
+  const float r = ORDERED ? __fsub_rn(c, bb)
+                          : __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(c, bb));
   const unsigned tb = __float_as_uint(t), rb = __float_as_uint(r);
   const unsigned et = (tb >> 23) & 0xffu, er = (rb >> 23) & 0xffu;
   const unsigned long long B = (unsigned long long)((tb & 0x7fffffu) | 0x800000u) << 29;

@@ -757,11 +757,11 @@ namespace {
 //    empty: its own capacity is 256 per SM.
 //  * Three lanes per trajectory hold 120 trajectories per SM; at 80 and at 20
 //    per SM (2 warps and half a warp per sub-partition) the survivors are
-//    packed again, the last time with six lanes each (7.3 instead of 8.8 us a
+//    packed again, the last time with six lanes each (6.7 instead of 8.8 us a
 //    step when each sub-partition has one warp).
-// 12,288 sweep lanes take 472 ms this way, 572 ms with three lanes to the
+// 12,288 sweep lanes take 460 ms this way, 572 ms with three lanes to the
 // end, 660 ms without packing and 1,250 ms in the one-thread kernel alone;
-// 200,000 mixed lanes 769 ms against 1,440 ms.
+// 200,000 mixed lanes 763 ms against 1,440 ms.
 struct Stage {
   int lanes;         // lanes per trajectory (1: the persistent kernel)
   int keep_per_sm;   // hands on at this many trajectories per SM (0: none)

@@ -13,7 +13,7 @@
 //   G = 3: lane j holds component j of both Jacobi vectors; a step takes
 //          177 warp-wide FP64 instructions (Morse), 10 trajectories a warp.
 //   G = 6: lane c holds one component (c < 3: rho1, else rho2), the two
-//          halves of the group evaluate the three pair forces twice; 146
+//          halves of the group evaluate the three pair forces twice; 140
 //          instructions a step, 5 trajectories a warp.
 // The group exchanges pair-vector components, the pair force factors, the
 // step's scalar coefficients (each lane forms every G-th) and the error
@@ -78,7 +78,8 @@ struct Grp {
   DevPair q;    // pair j of the trajectory's system
   double kf;    // dP1-force factor of pair j (f_j = kf u_j)
   double cA, cB;   // the system's Jacobi coefficients
-  double kh;    // dP2-force factor of pair j (h_1, h_2; pair AB: unused, not 0)
+  double kh;    // dP2-force factor of pair j (h_1, h_2; pair AB: unused); with
+                // G = 6 the upper half holds it in kf
   const double* coef;   // the step's nine tableau entries, in shared memory
   // global position component (0-2: rho1, 3-5: rho2) of local component k
   __device__ __forceinline__ int comp(int k) const { return G == 3 ? (k == 0 ? j : 3 + j) : c; }
@@ -199,16 +200,19 @@ __device__ __forceinline__ void accel_grp(const Grp<G>& L,
   const double s = fma(c0, c0, fma(c1, c1, op.mul(c2, c2)));
   s_own = s;
   const double u = pair_u_grp<MORSE>(L.q, s, T, op);
-  const double f = op.mul(L.kf, u), h = op.mul(L.kh, u);
-  const double f0 = __shfl_sync(FULL, f, L.base), f1 = __shfl_sync(FULL, f, L.base + 1),
-               f2 = __shfl_sync(FULL, f, L.base + 2);
-  const double h1 = __shfl_sync(FULL, h, L.base + 1), h2 = __shfl_sync(FULL, h, L.base + 2);
   if (G == 3) {
+    const double f = op.mul(L.kf, u), h = op.mul(L.kh, u);
+    const double f0 = __shfl_sync(FULL, f, L.base), f1 = __shfl_sync(FULL, f, L.base + 1),
+                 f2 = __shfl_sync(FULL, f, L.base + 2);
+    const double h1 = __shfl_sync(FULL, h, L.base + 1), h2 = __shfl_sync(FULL, h, L.base + 2);
     a[0] = fma(f0, rab, fma(f1, rbc, op.mul(f2, rca)));
     a[1] = fma(h1, rbc, op.mul(h2, rca));
   } else {
-    const bool first = L.c < 3;
-    a[0] = fma(first ? f0 : 0.0, rab, fma(first ? f1 : h1, rbc, op.mul(first ? f2 : h2, rca)));
+    // the lower half forms the f_j, the upper one the h_j: each half needs its own
+    const double f = op.mul(L.kf, u);
+    const double f0 = __shfl_sync(FULL, f, half), f1 = __shfl_sync(FULL, f, half + 1),
+                 f2 = __shfl_sync(FULL, f, half + 2);
+    a[0] = fma(L.c < 3 ? f0 : 0.0, rab, fma(f1, rbc, op.mul(f2, rca)));
   }
 }
 
@@ -516,6 +520,7 @@ __global__ void __launch_bounds__(kGrpBlock) k_integrate_grp(SysSet sys, const D
             L.cB = S.cB;
   L.kf = MORSE ? S.kf_morse[L.j] : S.kf[L.j];
   L.kh = L.j == 0 ? L.kf : (MORSE ? S.kf_morse[2 + L.j] : S.kf[2 + L.j]);
+  if (G == 6 && L.c >= 3) L.kf = L.kh;
 
   GrpLane<K> X;
   double inv_mu[K];
@@ -587,6 +592,7 @@ __device__ __forceinline__ void group_load(const SysSet& sys, const IntegParams&
   L.cB = S.cB;
   L.kf = MORSE ? S.kf_morse[L.j] : S.kf[L.j];
   L.kh = L.j == 0 ? L.kf : (MORSE ? S.kf_morse[2 + L.j] : S.kf[2 + L.j]);
+  if (G == 6 && L.c >= 3) L.kf = L.kh;
 #pragma unroll
   for (int k = 0; k < Grp<G>::K; ++k) {
     const int cg = L.comp(k);
