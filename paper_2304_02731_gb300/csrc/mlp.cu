@@ -42,20 +42,17 @@ struct Std {
   float mean[8], inv_std[8];
 };
 
-// Shared-memory weight tiles (BF16).  Forward B operands use W as [N][K];
-// backward dA = dZ W needs W^T as [K][N].  Padding: W1 K 8 -> 16, W4 N 4 -> 8
-// (forward) and W4^T N 4 -> 16.  Every row is padded by 8 elements (16 B):
-// a fragment load touches rows g = 0..7 at words 2q / 2 + const, and the
-// 16-byte row skew puts the 8 rows x 4 words on 32 distinct banks.
+// Shared-memory weight tiles (BF16), W as [N][K]: the forward pass takes its
+// B operands from rows of W (ldmatrix), the backward pass dA = dZ W the same
+// tiles transposed (ldmatrix.trans).  Padding: W1 K 8 -> 16, W4 N 4 -> 8.
+// Every row is padded by 8 elements (16 B): the 8 row segments of 16 bytes
+// that a matrix load touches lie on 32 distinct banks.
 constexpr int PK = 8;   // row padding (BF16 elements)
 struct alignas(16) WeightsSmem {   // 16-byte row-segment stores
   __nv_bfloat16 w1[H][16 + PK];
   __nv_bfloat16 w2[H][H + PK];
   __nv_bfloat16 w3[H][H + PK];
   __nv_bfloat16 w4[8][H + PK];
-  __nv_bfloat16 w2t[H][H + PK];
-  __nv_bfloat16 w3t[H][H + PK];
-  __nv_bfloat16 w4t[H][16 + PK];
   float b1[H], b2[H], b3[H], b4[8];
 };
 // Training works in block rounds of RS = 64 CPW samples (4 warps x CPW
@@ -64,22 +61,16 @@ struct alignas(16) WeightsSmem {   // 16-byte row-segment stores
 // back-propagated errors of its 16 samples (BF16, [unit][sample]); after the
 // round each warp forms 16 rows of every weight gradient dW = dZ^T A as an
 // MMA product over the round's samples, accumulated in registers and added
-// to the global gradient once.  Rows are padded by 8 elements: a fragment
-// load touches rows g = 0..7 at words q + const, and a row stride of
-// 32 CPW + 4 words puts them on 32 distinct banks.
+// to the global gradient once.  Rows are padded by 8 elements for the
+// matrix loads and stores, as the weights' are.
 template <int CPW>
-struct BlockTiles {
+struct alignas(16) BlockTiles {
   static constexpr int RS = 16 * WARPS * CPW;   // samples per block round
   static constexpr int LDT = RS + PK;           // row stride (BF16 elements)
   __nv_bfloat16 xt[16][LDT];         // X^T  [feature (padded to 16)][sample]
   __nv_bfloat16 at[3][H][LDT];       // A1^T, A2^T, A3^T [unit][sample]
   __nv_bfloat16 dzt[3][H][LDT];      // dZ1^T, dZ2^T, dZ3^T [unit][sample]
   __nv_bfloat16 dz4t[16][LDT];       // dZ4^T [output (padded to 16)][sample]
-};
-// SiLU'(Z) of the warp's current chunk (layers 1-3), fragment order
-// [i][lane], computed in the forward pass for the backward pass.
-struct WarpZ {
-  float ds[3][32][32];
 };
 // Bias gradients of the block (b1, b2, b3, b4), FP32 sums of the FP32 dZ
 // fragments.
@@ -89,44 +80,71 @@ struct TrainSmem {
   WeightsSmem w;
   float gb[NGB];
   BlockTiles<CPW> t;
-  WarpZ wz[WARPS];
 };
 
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
 }
-__device__ __forceinline__ uint32_t ld2(const __nv_bfloat16* p) {
-  return *reinterpret_cast<const uint32_t*>(p);
-}
-
 // D += A B for one m16n8k16 tile (BF16 in, FP32 accumulate).
 __device__ __forceinline__ void mma(float* d, const uint32_t* a, uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
       "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// Four 8 x 8 BF16 matrices from shared memory, lane l giving the address of
+// row l mod 8 of matrix l / 8 (16 bytes, 16-byte aligned); TRANS: each one
+// transposed.  Lane (g, q) receives elements (g, 2q), (g, 2q + 1).
+template <bool TRANS>
+__device__ __forceinline__ void ldsm4(uint32_t* r, const __nv_bfloat16* row) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(row);
+  if (TRANS)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
+}
+// The reverse, transposed: four (two) fragments to rows of their columns.
+__device__ __forceinline__ void stsm4t(__nv_bfloat16* row, const uint32_t* r) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(row)),
+               "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+}
+__device__ __forceinline__ void stsm2t(__nv_bfloat16* row, uint32_t r0, uint32_t r1) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x2.trans.shared.b16 [%0], {%1,%2};" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(row)),
+               "r"(r0), "r"(r1) : "memory");
+}
+// A 16-sample, 64-unit tile in A-fragment order (a[s]: units 16 s ..) to the
+// rows of dst ([unit][sample]) at sample columns col .. col + 15.
+template <int LDT>
+__device__ __forceinline__ void store_units(__nv_bfloat16 (*dst)[LDT], int col,
+                                            const uint32_t (*a)[4]) {
+  const int l = threadIdx.x & 31;
+#pragma unroll
+  for (int s = 0; s < 4; ++s)
+    stsm4t(&dst[16 * s + 8 * (l >> 4) + (l & 7)][col + 8 * ((l >> 3) & 1)], a[s]);
+}
+// An 8-unit tile (fragments of samples 0-7 and 8-15) likewise.
+template <int LDT>
+__device__ __forceinline__ void store_tile8(__nv_bfloat16 (*dst)[LDT], int col, uint32_t r0,
+                                            uint32_t r1) {
+  const int l = threadIdx.x & 15;
+  stsm2t(&dst[l & 7][col + 8 * (l >> 3)], r0, r1);
 }
 
 // Logistic function: __expf and the fast divide (a few ulp; the products it
 // feeds are rounded to BF16).  For z below about -87 the quotient is 0.
 __device__ __forceinline__ float sigm(float z) { return __fdividef(1.0f, 1.0f + __expf(-z)); }
 
-__device__ __forceinline__ __nv_bfloat16 bf_lo(uint32_t w) {
-  return __ushort_as_bfloat16((unsigned short)(w & 0xffffu));
-}
-__device__ __forceinline__ __nv_bfloat16 bf_hi(uint32_t w) {
-  return __ushort_as_bfloat16((unsigned short)(w >> 16));
-}
-
 // Weights to shared memory (blockDim.x == THREADS).  With p 16-byte aligned
 // every matrix starts on a 16-byte boundary: each thread issues all of its
 // 16-byte loads of 8-element row segments first, then stores each segment
-// to its W row and, TRANSPOSED (the backward pass), element by element to the
-// W^T column.  Otherwise, element loads.  All loads go to L2: the training
+// to its row.  Otherwise, element loads.  All loads go to L2: the training
 // kernel's other blocks rewrite the parameters between its steps.
-template <bool TRANSPOSED>
 __device__ void load_weights(WeightsSmem& W, const __nv_bfloat16* p, const float* pf) {
   const __nv_bfloat16 zero = __float2bfloat16(0.0f);
   if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0) {
@@ -149,7 +167,6 @@ __device__ void load_weights(WeightsSmem& W, const __nv_bfloat16* p, const float
     for (int k = 0; k < PER; ++k) {
       const int i = threadIdx.x + k * THREADS;
       if (i >= NSEG) continue;
-      const uint32_t w[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
       if (i < N1) {
         *reinterpret_cast<uint4*>(&W.w1[i][0]) = v[k];
         *reinterpret_cast<uint4*>(&W.w1[i][8]) = make_uint4(0u, 0u, 0u, 0u);
@@ -160,23 +177,8 @@ __device__ void load_weights(WeightsSmem& W, const __nv_bfloat16* p, const float
       const int r = j / (H / 8), c = 8 * (j % (H / 8));
       __nv_bfloat16* row = is4 ? &W.w4[r][c] : i < N1 + N2 ? &W.w2[r][c] : &W.w3[r][c];
       *reinterpret_cast<uint4*>(row) = v[k];
-#pragma unroll
-      for (int e = 0; e < (TRANSPOSED ? 4 : 0); ++e) {
-        if (is4) {
-          W.w4t[c + 2 * e][r] = bf_lo(w[e]);
-          W.w4t[c + 2 * e + 1][r] = bf_hi(w[e]);
-        } else if (i < N1 + N2) {
-          W.w2t[c + 2 * e][r] = bf_lo(w[e]);
-          W.w2t[c + 2 * e + 1][r] = bf_hi(w[e]);
-        } else {
-          W.w3t[c + 2 * e][r] = bf_lo(w[e]);
-          W.w3t[c + 2 * e + 1][r] = bf_hi(w[e]);
-        }
-      }
     }
     for (int i = threadIdx.x; i < (8 - OUT) * H; i += blockDim.x) W.w4[OUT + i / H][i % H] = zero;
-    for (int i = threadIdx.x; i < H * (16 - OUT); i += blockDim.x)
-      W.w4t[i / (16 - OUT)][OUT + i % (16 - OUT)] = zero;
   } else {
     auto ld = [&](int k) {
       return __ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short*>(p) + k));
@@ -189,16 +191,10 @@ __device__ void load_weights(WeightsSmem& W, const __nv_bfloat16* p, const float
       const int r = i / H, c = i % H;
       W.w2[r][c] = ld(OW2 + i);
       W.w3[r][c] = ld(OW3 + i);
-      W.w2t[c][r] = ld(OW2 + i);
-      W.w3t[c][r] = ld(OW3 + i);
     }
     for (int i = threadIdx.x; i < 8 * H; i += blockDim.x) {
       const int r = i / H, c = i % H;
       W.w4[r][c] = r < OUT ? ld(OW4 + r * H + c) : zero;
-    }
-    for (int i = threadIdx.x; i < H * 16; i += blockDim.x) {
-      const int r = i / 16, c = i % 16;
-      W.w4t[r][c] = c < OUT ? ld(OW4 + c * H + r) : zero;
     }
   }
   for (int i = threadIdx.x; i < H; i += blockDim.x) {
@@ -234,10 +230,12 @@ struct RowSrc {
 __device__ __forceinline__ void features(const float* x, int64_t src, int64_t n,
                                          int64_t row, const CellGrid* grid, float* f) {
   if (row >= n) {
+#pragma unroll
     for (int k = 0; k < IN; ++k) f[k] = 0.0f;
     return;
   }
   if (!grid) {
+#pragma unroll
     for (int k = 0; k < IN; ++k) f[k] = x[src * IN + k];
     return;
   }
@@ -260,47 +258,58 @@ __device__ __forceinline__ void features(const float* x, int64_t src, int64_t n,
 // Forward pass of 16 samples (rows base .. base+15) by one warp; this lane's
 // rows base + g and base + g + 8 are samples src0 and src1.  Returns the
 // logits fragment (rows g and g+8, columns 2q, 2q+1 of the padded 16x8 tile).
-// With TRAIN, pre-activations go to the warp's z tiles and the transposed
-// inputs and activations to the block tiles T, at sample columns col ..
-// col + 15, for the backward pass.
+// With TRAIN, ds receives SiLU'(Z) of layers 1-3 (accumulator order) and the
+// transposed inputs and activations go to the block tiles T, at sample
+// columns col .. col + 15, for the backward pass.
 template <bool TRAIN, int CPW>
-__device__ void forward16(const WeightsSmem& W, WarpZ* wz, BlockTiles<CPW>* T, int col, const float* x,
-                          int64_t src0, int64_t src1, int64_t n, int64_t base,
-                          const CellGrid* grid, const Std& sd, float* logit) {
+__device__ __forceinline__ void forward16(const WeightsSmem& W, float (*ds)[32], BlockTiles<CPW>* T,
+                                          int col, const float* x, int64_t src0, int64_t src1,
+                                          int64_t n, int64_t base, const CellGrid* grid,
+                                          const Std& sd, float* logit) {
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+  // this lane's row of two adjacent 8-unit tiles in a matrix load
+  const int wrow = 8 * (lane >> 4) + (lane & 7), wcol = 8 * ((lane >> 3) & 1);
   float f0[IN], f1[IN];
   features(x, src0, n, base + g, grid, f0);
   features(x, src1, n, base + g + 8, grid, f1);
+#pragma unroll
   for (int k = 0; k < IN; ++k) {
     f0[k] = (f0[k] - sd.mean[k]) * sd.inv_std[k];
     f1[k] = (f1[k] - sd.mean[k]) * sd.inv_std[k];
     if (base + g >= n) f0[k] = 0.0f;
     if (base + g + 8 >= n) f1[k] = 0.0f;
   }
+  // features 2q, 2q + 1 by selects (no dynamic register indexing)
+  auto pick = [&](const float* f, int e) {
+    return q == 0 ? f[e] : q == 1 ? f[2 + e] : q == 2 ? f[4 + e] : f[6 + e];
+  };
   uint32_t a[4][4];  // A fragments of the current layer input (up to 4 k-slices)
-  a[0][0] = pack2(f0[2 * q], f0[2 * q + 1]);
-  a[0][1] = pack2(f1[2 * q], f1[2 * q + 1]);
+  a[0][0] = pack2(pick(f0, 0), pick(f0, 1));
+  a[0][1] = pack2(pick(f1, 0), pick(f1, 1));
   a[0][2] = 0u;
   a[0][3] = 0u;
-  if (TRAIN) {
-    T->xt[2 * q][col + g] = __float2bfloat16(f0[2 * q]);
-    T->xt[2 * q + 1][col + g] = __float2bfloat16(f0[2 * q + 1]);
-    T->xt[2 * q][col + g + 8] = __float2bfloat16(f1[2 * q]);
-    T->xt[2 * q + 1][col + g + 8] = __float2bfloat16(f1[2 * q + 1]);
-  }
-  float c[8][4];
+  if (TRAIN) store_tile8(T->xt, col, a[0][0], a[0][1]);
+#pragma unroll
   for (int layer = 0; layer < 3; ++layer) {
     const float* bias = layer == 0 ? W.b1 : layer == 1 ? W.b2 : W.b3;
-    const int ks = layer == 0 ? 1 : 4;
+    float c[8][4];
 #pragma unroll
     for (int t = 0; t < 8; ++t) {
-      c[t][0] = c[t][2] = bias[8 * t + 2 * q];
-      c[t][1] = c[t][3] = bias[8 * t + 2 * q + 1];
-      for (int s = 0; s < ks; ++s) {
-        const __nv_bfloat16* wr = layer == 0 ? &W.w1[8 * t + g][0]
-                                  : layer == 1 ? &W.w2[8 * t + g][16 * s]
-                                               : &W.w3[8 * t + g][16 * s];
-        mma(c[t], a[s], ld2(wr + 2 * q), ld2(wr + 8 + 2 * q));
+      const float2 b = *reinterpret_cast<const float2*>(&bias[8 * t + 2 * q]);
+      c[t][0] = c[t][2] = b.x;
+      c[t][1] = c[t][3] = b.y;
+    }
+    // k-slices outside: eight independent accumulators in flight
+#pragma unroll
+    for (int s = 0; s < (layer == 0 ? 1 : 4); ++s) {
+#pragma unroll
+      for (int t = 0; t < 8; t += 2) {
+        uint32_t b[4];
+        ldsm4<false>(b, layer == 0   ? &W.w1[8 * t + wrow][wcol]
+                        : layer == 1 ? &W.w2[8 * t + wrow][16 * s + wcol]
+                                     : &W.w3[8 * t + wrow][16 * s + wcol]);
+        mma(c[t], a[s], b[0], b[1]);
+        mma(c[t + 1], a[s], b[2], b[3]);
       }
     }
 #pragma unroll
@@ -314,31 +323,23 @@ __device__ void forward16(const WeightsSmem& W, WarpZ* wz, BlockTiles<CPW>* T, i
         for (int e = 0; e < 4; ++e) {
           const float z = c[2 * s + h][e], sg = sigm(z);
           v[4 * h + e] = z * sg;
-          if (TRAIN) wz->ds[layer][4 * (2 * s + h) + e][lane] = sg * (1.0f + z * (1.0f - sg));
+          if (TRAIN) ds[layer][4 * (2 * s + h) + e] = sg * (1.0f + z * (1.0f - sg));
         }
       a[s][0] = pack2(v[0], v[1]);
       a[s][1] = pack2(v[2], v[3]);
       a[s][2] = pack2(v[4], v[5]);
       a[s][3] = pack2(v[6], v[7]);
-      if (TRAIN) {
-        __nv_bfloat16 (*at)[BlockTiles<CPW>::LDT] = T->at[layer];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int u = 16 * s + 8 * h + 2 * q;
-          at[u][col + g] = __float2bfloat16(v[4 * h]);
-          at[u + 1][col + g] = __float2bfloat16(v[4 * h + 1]);
-          at[u][col + g + 8] = __float2bfloat16(v[4 * h + 2]);
-          at[u + 1][col + g + 8] = __float2bfloat16(v[4 * h + 3]);
-        }
-      }
     }
+    if (TRAIN) store_units(T->at[layer], col, a);
   }
   logit[0] = logit[2] = W.b4[2 * q];
   logit[1] = logit[3] = W.b4[2 * q + 1];
 #pragma unroll
-  for (int s = 0; s < 4; ++s) {
-    const __nv_bfloat16* wr = &W.w4[g][16 * s];
-    mma(logit, a[s], ld2(wr + 2 * q), ld2(wr + 8 + 2 * q));
+  for (int s = 0; s < 4; s += 2) {
+    uint32_t b[4];   // W4's one tile: k-slices s and s + 1
+    ldsm4<false>(b, &W.w4[lane & 7][16 * s + 8 * (lane >> 3)]);
+    mma(logit, a[s], b[0], b[1]);
+    mma(logit, a[s + 1], b[2], b[3]);
   }
 }
 
@@ -355,32 +356,31 @@ __device__ __forceinline__ void softmax_pair(float z0, float z1, float* p0, floa
 }
 
 // One warp's 16 rows m0 .. m0+15 of dW = dZ^T A over the round's RS samples,
-// for the n_tiles 8-column tiles from column n0: A operand from dZ^T (rows
+// for the NT 8-column tiles from column n0: A operand from dZ^T (rows
 // = output units, samples contiguous), B operand from A^T (rows = input
 // units, samples contiguous: the col layout of B), FP32 accumulation in
 // registers; added once to the global gradient gW (row-major, n_in columns)
 // for rows < n_out and columns < n_in.
-template <int LDT>
-__device__ void block_dw(const __nv_bfloat16 (*dzt)[LDT], const __nv_bfloat16 (*at)[LDT], int m0,
-                         int n0, int n_tiles, int n_out, int n_in, float* gW) {
+template <int NT, int LDT>
+__device__ __forceinline__ void block_dw(const __nv_bfloat16 (*dzt)[LDT],
+                                         const __nv_bfloat16 (*at)[LDT], int m0, int n0, int n_out,
+                                         int n_in, float* gW) {
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
   const bool vec4 = (reinterpret_cast<uintptr_t>(gW) & 15u) == 0;
-  float d[8][4];
+  float d[NT][4];
 #pragma unroll
-  for (int t = 0; t < 8; ++t) d[t][0] = d[t][1] = d[t][2] = d[t][3] = 0.0f;
-#pragma unroll 2
+  for (int t = 0; t < NT; ++t) d[t][0] = d[t][1] = d[t][2] = d[t][3] = 0.0f;
+#pragma unroll
   for (int ks = 0; ks < (LDT - PK) / 16; ++ks) {
     uint32_t a[4];
-    a[0] = ld2(&dzt[m0 + g][16 * ks + 2 * q]);
-    a[1] = ld2(&dzt[m0 + g + 8][16 * ks + 2 * q]);
-    a[2] = ld2(&dzt[m0 + g][16 * ks + 8 + 2 * q]);
-    a[3] = ld2(&dzt[m0 + g + 8][16 * ks + 8 + 2 * q]);
+    ldsm4<false>(a, &dzt[m0 + 8 * ((lane >> 3) & 1) + (lane & 7)][16 * ks + 8 * (lane >> 4)]);
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      if (t < n_tiles) {
-        const __nv_bfloat16* br = &at[n0 + 8 * t + g][16 * ks];
-        mma(d[t], a, ld2(br + 2 * q), ld2(br + 8 + 2 * q));
-      }
+    for (int t = 0; t < NT; t += 2) {   // (one tile: the second is the tile's zero padding)
+      uint32_t b[4];
+      ldsm4<false>(b, &at[n0 + 8 * t + 8 * (lane >> 4) + (lane & 7)]
+                         [16 * ks + 8 * ((lane >> 3) & 1)]);
+      mma(d[t], a, b[0], b[1]);
+      if (t + 1 < NT) mma(d[t + 1], a, b[2], b[3]);
     }
   }
   // Lanes q and q ^ 1 hold columns 2q, 2q + 1 of rows g and g + 8: the even
@@ -388,8 +388,7 @@ __device__ void block_dw(const __nv_bfloat16 (*dzt)[LDT], const __nv_bfloat16 (*
   // consecutive columns each (vector atomics, sm_90 and later; n_in is a
   // multiple of 4 and the parameter offsets are too).
 #pragma unroll
-  for (int t = 0; t < 8; ++t) {
-    if (t >= n_tiles) continue;
+  for (int t = 0; t < NT; ++t) {
     const bool odd = q & 1;
     const float s0 = odd ? d[t][0] : d[t][2], s1 = odd ? d[t][1] : d[t][3];
     const float o0 = __shfl_xor_sync(0xffffffffu, s0, 1), o1 = __shfl_xor_sync(0xffffffffu, s1, 1);
@@ -410,37 +409,44 @@ __device__ void block_dw(const __nv_bfloat16 (*dzt)[LDT], const __nv_bfloat16 (*
   }
 }
 
-// Write dZ (fragment layout: 16 samples x `tiles` 8-unit tiles) transposed
-// into the block tile dst at sample columns col .. col + 15.
-template <int LDT>
-__device__ __forceinline__ void store_dz(__nv_bfloat16 (*dst)[LDT], int col, const float (*dz)[4],
-                                         int tiles) {
+// Bias gradients of a 64-unit layer: the sums over the 16 samples of dZ's
+// columns, added to gb.  The 16 columns of a lane quad are reduced over its
+// eight row lanes by halving (14 shuffles), which leaves lane (g, q) with
+// columns 8 g + 2 q and + 1.
+__device__ __forceinline__ void accumulate_db(const float (*dz)[4], float* gb) {
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
-  for (int t = 0; t < tiles; ++t) {
-    const int c0 = 8 * t + 2 * q;
-    dst[c0][col + g] = __float2bfloat16(dz[t][0]);
-    dst[c0 + 1][col + g] = __float2bfloat16(dz[t][1]);
-    dst[c0][col + g + 8] = __float2bfloat16(dz[t][2]);
-    dst[c0 + 1][col + g + 8] = __float2bfloat16(dz[t][3]);
-  }
-}
-
-// Bias gradient: sum over the 16 samples of dZ columns.
-__device__ __forceinline__ void accumulate_db(const float (*dz)[4], int tiles, int n_valid,
-                                              float* gb) {
-  const int lane = threadIdx.x & 31, q = lane & 3;
-  for (int t = 0; t < tiles; ++t) {
-    float s0 = dz[t][0] + dz[t][2], s1 = dz[t][1] + dz[t][3];
+  float s[8][2];
 #pragma unroll
-    for (int o = 4; o < 32; o <<= 1) {
-      s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-    }
-    const int col = 8 * t + 2 * q;
-    if (lane < 4 && col < n_valid) {
-      atomicAdd(&gb[col], s0);
-      if (col + 1 < n_valid) atomicAdd(&gb[col + 1], s1);
-    }
+  for (int t = 0; t < 8; ++t) {
+    s[t][0] = dz[t][0] + dz[t][2];
+    s[t][1] = dz[t][1] + dz[t][3];
+  }
+#pragma unroll
+  for (int half = 4; half > 0; half >>= 1) {
+    const bool up = g & half;
+#pragma unroll
+    for (int t = 0; t < half; ++t)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float send = up ? s[t][e] : s[t + half][e], keep = up ? s[t + half][e] : s[t][e];
+        s[t][e] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * half);
+      }
+  }
+  atomicAdd(&gb[8 * g + 2 * q], s[0][0]);
+  atomicAdd(&gb[8 * g + 2 * q + 1], s[0][1]);
+}
+// The same for the 4 outputs (columns 0-3 of one tile).
+__device__ __forceinline__ void accumulate_db4(const float* dz, float* gb) {
+  const int lane = threadIdx.x & 31;
+  float s0 = dz[0] + dz[2], s1 = dz[1] + dz[3];
+#pragma unroll
+  for (int o = 4; o < 32; o <<= 1) {
+    s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+    s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+  }
+  if (lane < 2) {
+    atomicAdd(&gb[2 * lane], s0);
+    atomicAdd(&gb[2 * lane + 1], s1);
   }
 }
 
@@ -448,7 +454,7 @@ __device__ __forceinline__ void accumulate_db(const float (*dz)[4], int tiles, i
 // barrier).
 template <int CPW>
 __device__ void grad_begin(TrainSmem<CPW>& S, const __nv_bfloat16* pb, const float* pf) {
-  load_weights<true>(S.w, pb, pf);
+  load_weights(S.w, pb, pf);
   for (int i = threadIdx.x; i < NGB; i += blockDim.x) S.gb[i] = 0.0f;
 }
 // Padding rows of the X^T and dZ4^T tiles (never written by the passes).
@@ -475,7 +481,6 @@ __device__ void grad_rounds(TrainSmem<CPW>& S, const Std& sd, const float* x,
   if ((int64_t)blockIdx.x * RS >= n) return;   // no round for this block
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
-  WarpZ* wz = &S.wz[warp];
   const float inv_n = 1.0f / (float)n;
   float loss_acc = 0.0f;
   const int64_t rounds = (n + RS - 1) / RS;
@@ -483,10 +488,10 @@ __device__ void grad_rounds(TrainSmem<CPW>& S, const Std& sd, const float* x,
     for (int c = 0; c < CPW; ++c) {
       const int col = 16 * (WARPS * c + warp);
       const int64_t base = rnd * RS + col;
-      float lg[4];
+      float lg[4], ds[3][32];
       const int64_t r0 = base + g, r1 = base + g + 8;
       const int64_t s0 = rows.at(r0), s1 = rows.at(r1);
-      forward16<true, CPW>(S.w, wz, &S.t, col, x, s0, s1, n, base, nullptr, sd, lg);
+      forward16<true, CPW>(S.w, ds, &S.t, col, x, s0, s1, n, base, nullptr, sd, lg);
       // softmax cross-entropy and dZ4 = (p - onehot) / n; rows past n and
       // rows without a target have dZ4 = 0 and so add nothing below
       float dz4[1][4] = {{0.f, 0.f, 0.f, 0.f}};
@@ -510,49 +515,61 @@ __device__ void grad_rounds(TrainSmem<CPW>& S, const Std& sd, const float* x,
           }
         }
       }
-      store_dz(S.t.dz4t, col, dz4, 1);
-      accumulate_db(dz4, 1, OUT, &S.gb[3 * H]);
+      accumulate_db4(dz4[0], &S.gb[3 * H]);
       // dA3 = dZ4 W4: A operand from the dZ4 fragment (K padded 8 -> 16)
       uint32_t a[4][4];
       a[0][0] = pack2(dz4[0][0], dz4[0][1]);
       a[0][1] = pack2(dz4[0][2], dz4[0][3]);
       a[0][2] = 0u;
       a[0][3] = 0u;
-      float dz[8][4];
+      store_tile8(S.t.dz4t, col, a[0][0], a[0][1]);
+#pragma unroll
       for (int layer = 2; layer >= 0; --layer) {
-        const int ks = layer == 2 ? 1 : 4;
+        float dz[8][4];
 #pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          dz[t][0] = dz[t][1] = dz[t][2] = dz[t][3] = 0.0f;
-          for (int s = 0; s < ks; ++s) {
-            const __nv_bfloat16* wr = layer == 2 ? &S.w.w4t[8 * t + g][0]
-                                      : layer == 1 ? &S.w.w3t[8 * t + g][16 * s]
-                                                   : &S.w.w2t[8 * t + g][16 * s];
-            mma(dz[t], a[s], ld2(wr + 2 * q), ld2(wr + 8 + 2 * q));
+        for (int t = 0; t < 8; ++t) dz[t][0] = dz[t][1] = dz[t][2] = dz[t][3] = 0.0f;
+        if (layer == 2) {
+#pragma unroll
+          for (int t = 0; t < 8; t += 4) {
+            uint32_t b[4];   // rows = outputs: tiles t .. t + 3, upper half of K zero
+            ldsm4<true>(b, &S.w.w4[lane & 7][8 * (t + (lane >> 3))]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) mma(dz[t + k], a[0], b[k], 0u);
           }
-          // dZ = dA * SiLU'(Z)
+        } else {
+          const __nv_bfloat16 (*w)[H + PK] = layer == 1 ? S.w.w3 : S.w.w2;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) dz[t][e] *= wz->ds[layer][4 * t + e][lane];
-        }
-        store_dz(S.t.dzt[layer], col, dz, 8);
-        accumulate_db(dz, 8, H, &S.gb[GB1 + H * layer]);
-        if (layer > 0) {
+          for (int s = 0; s < 4; ++s)
 #pragma unroll
-          for (int s = 0; s < 4; ++s) {
-            a[s][0] = pack2(dz[2 * s][0], dz[2 * s][1]);
-            a[s][1] = pack2(dz[2 * s][2], dz[2 * s][3]);
-            a[s][2] = pack2(dz[2 * s + 1][0], dz[2 * s + 1][1]);
-            a[s][3] = pack2(dz[2 * s + 1][2], dz[2 * s + 1][3]);
-          }
+            for (int t = 0; t < 8; t += 2) {
+              uint32_t b[4];
+              ldsm4<true>(b, &w[16 * s + 8 * ((lane >> 3) & 1) + (lane & 7)][8 * t + 8 * (lane >> 4)]);
+              mma(dz[t], a[s], b[0], b[1]);
+              mma(dz[t + 1], a[s], b[2], b[3]);
+            }
         }
+        // dZ = dA * SiLU'(Z)
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) dz[t][e] *= ds[layer][4 * t + e];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          a[s][0] = pack2(dz[2 * s][0], dz[2 * s][1]);
+          a[s][1] = pack2(dz[2 * s][2], dz[2 * s][3]);
+          a[s][2] = pack2(dz[2 * s + 1][0], dz[2 * s + 1][1]);
+          a[s][3] = pack2(dz[2 * s + 1][2], dz[2 * s + 1][3]);
+        }
+        store_units(S.t.dzt[layer], col, a);
+        accumulate_db(dz, &S.gb[GB1 + H * layer]);
       }
     }
     __syncthreads();   // the round's tiles are complete
     const int m0 = 16 * warp;
-    block_dw(S.t.dzt[0], S.t.xt, m0, 0, 1, H, IN, grad + OW1);
-    block_dw(S.t.dzt[1], S.t.at[0], m0, 0, 8, H, H, grad + OW2);
-    block_dw(S.t.dzt[2], S.t.at[1], m0, 0, 8, H, H, grad + OW3);
-    block_dw(S.t.dz4t, S.t.at[2], 0, m0, 2, OUT, H, grad + OW4);
+    block_dw<1>(S.t.dzt[0], S.t.xt, m0, 0, H, IN, grad + OW1);
+    block_dw<8>(S.t.dzt[1], S.t.at[0], m0, 0, H, H, grad + OW2);
+    block_dw<8>(S.t.dzt[2], S.t.at[1], m0, 0, H, H, grad + OW3);
+    block_dw<2>(S.t.dz4t, S.t.at[2], 0, m0, OUT, H, grad + OW4);
     __syncthreads();   // tiles are rewritten by the next round
   }
 #pragma unroll
@@ -582,7 +599,7 @@ __global__ void __launch_bounds__(THREADS) k_mlp_infer(const __nv_bfloat16* pb, 
                                                        float* probs, double* g_out,
                                                        double eps) {
   __shared__ WeightsSmem W;
-  load_weights<false>(W, pb, pf);
+  load_weights(W, pb, pf);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
   const int64_t chunks = (n + 15) / 16;
@@ -635,7 +652,8 @@ __global__ void k_adam(float* p, float* m, float* v, const float* grad, __nv_bfl
 // SM.  Separate launches took 36 us a step (index draw 2.4, memsets, gradient
 // 22, Adam 3.4 and the gaps between them) for work that needs a fraction of
 // a microsecond at the tensor cores' rate: the step is a chain of latencies,
-// and this kernel shortens it to 21 us.  Each step a block draws its own
+// and this kernel shortens it to 14 us (21 before its passes took matrix loads
+// and stores).  Each step a block draws its own
 // rows, adds its share of the gradient and, after a grid barrier, takes the
 // Adam step of its own slice of the parameters; a second barrier publishes
 // them.  Gradient, loss and Adam arithmetic are those of the separate kernels.
