@@ -64,40 +64,53 @@ __device__ __forceinline__ double f64_of(float f) {
 // 1/r for r in the FP32 normal range: the FP32 hardware reciprocal y0
 // (relative error e0 below 2^-22), e = 1 - r y0, y = y0 (1 + e + e^2):
 // relative error e0^3 < 2^-66.  3 FP64 instructions.
-__device__ __forceinline__ double rcp_seeded(double r, float rf) {
+__device__ __forceinline__ double rcp_seeded(double r, float rf, const OpReg& op) {
   float yf;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(rf));
   const double y0 = f64_of(yf);
-  const double e = fma(-r, y0, 1.0);
+  const double e = fma(-r, y0, op.one());
   return fma(y0, fma(e, e, e), y0);
 }
 
 // ---------------------------------------------------------------------------
 // Potentials (Sec. 3.2 items 1-3).  The FP64 forms with the table
 // exponential: V, V' and, on request, V'' at r, given 1/r (ri) and an FP32
-// copy of r (rf) for the exponential's table index.
+// copy of r (rf) for the exponential's table index.  The work is bound by
+// the FP64 pipe, so products are DFMAs on registers (regop.cuh), and LJ
+// (12,6) and (8,6) take shared powers of 1/r^2 (SHARED; 4 products instead of
+// 11) wherever the energy error, a difference at rounding level, is not
+// formed from them.
 // ---------------------------------------------------------------------------
-template <bool D2>
+template <bool D2, bool SHARED>
 __device__ __forceinline__ void pot_tab(const DevPair& q, double r, double ri, float rf,
-                                        const double* __restrict__ T, double* V, double* dV,
-                                        double* d2V) {
+                                        const double* __restrict__ T, const OpReg& op, double* V,
+                                        double* dV, double* d2V) {
   if (q.kind == QCAMS_MORSE) {
     // x = e^{-alpha (r - re)}: V = De x (x - 2), V' = 2 alpha De x (1 - x),
     // V'' = 2 alpha^2 De x (2x - 1)
-    const double x = texp_hint(fma(-q.c0, r, q.c1), fmaf(-q.ef0, rf, q.ef1), T);
-    *V = q.c3 * (x * (x - 2.0));
-    *dV = q.c2 * fma(-x, x, x);
-    if (D2) *d2V = (q.c2 * q.c0) * (x * fma(2.0, x, -1.0));
+    const double x = texp_hint(fma(-q.c0, r, q.c1), fmaf(-q.ef0, rf, q.ef1), T, op);
+    *V = op.mul(q.c3, op.mul(x, x - 2.0));
+    *dV = op.mul(q.c2, fma(-x, x, x));
+    if (D2) *d2V = op.mul(op.mul(q.c2, q.c0), op.mul(x, fma(2.0, x, -1.0)));
   } else if (q.kind == QCAMS_LJ) {
-    const double rm = ipow(ri, q.m), rn = ipow(ri, q.n);
-    *V = fma(q.c0, rm, -q.c1 * rn);
-    *dV = fma(q.c3, rn, -q.c2 * rm) * ri;
+    double rm, rn;
+    if (SHARED && q.n == 6 && (q.m == 12 || q.m == 8)) {
+      const double ri2 = op.mul(ri, ri), ri4 = op.mul(ri2, ri2);
+      rn = op.mul(ri4, ri2);
+      const double h = q.m == 12 ? rn : ri4;
+      rm = op.mul(h, h);
+    } else {
+      rm = ipow(ri, q.m);
+      rn = ipow(ri, q.n);
+    }
+    *V = fma(q.c0, rm, -op.mul(q.c1, rn));
+    *dV = op.mul(fma(q.c3, rn, -op.mul(q.c2, rm)), ri);
     if (D2) *d2V = fma((q.m + 1.0) * q.c2, rm, -(q.n + 1.0) * q.c3 * rn) * (ri * ri);
   } else {
-    const double ex = texp_hint(-q.c1 * r, -q.ef0 * rf, T);
-    const double ri2 = ri * ri, ri6 = ri2 * ri2 * ri2;
-    *V = fma(q.c0, ex, -q.c4 * ri6);
-    *dV = fma(q.c3 * ri6, ri, -q.c2 * ex);
+    const double ex = texp_hint(op.mul(-q.c1, r), -q.ef0 * rf, T, op);
+    const double ri2 = op.mul(ri, ri), ri6 = op.mul(op.mul(ri2, ri2), ri2);
+    *V = fma(q.c0, ex, -op.mul(q.c4, ri6));
+    *dV = fma(op.mul(q.c3, ri6), ri, -op.mul(q.c2, ex));
     if (D2) *d2V = fma(q.c2 * q.c1, ex, -7.0 * q.c3 * ri6 * ri2);
   }
 }
@@ -202,36 +215,38 @@ __device__ double root_finish(F32 f32, FD fd, F64 f64, double a, double b, doubl
 // false: level solver) or from the shared-memory table T (TAB = true:
 // product analysis).
 template <bool TAB>
-__device__ __forceinline__ double pot_V_(const DevPair& q, double r, const double* T) {
+__device__ __forceinline__ double pot_V_(const DevPair& q, double r, const double* T,
+                                         const OpReg& op) {
   if (!TAB) return pot_V(q, r);
   const float rf = f32_of(r);
   double V, dV;
-  pot_tab<false>(q, r, rcp_seeded(r, rf), rf, T, &V, &dV, nullptr);
+  pot_tab<false, false>(q, r, rcp_seeded(r, rf, op), rf, T, op, &V, &dV, nullptr);
   return V;
 }
 // V_eff = V + L2/(2 mu r^2); inv_mu = 1/mu (used by TAB = true, which
 // multiplies by host-computed reciprocals instead of dividing).
 template <bool TAB>
 __device__ __forceinline__ double veff_(const DevPair& q, double mu, double inv_mu, double L2,
-                                        double r, const double* T) {
+                                        double r, const double* T, const OpReg& op) {
   if (!TAB) {
     const double ri = rsqrt(r * r);   // 1/r^2 from a reciprocal square root: no division
     return pot_V(q, r) + (0.5 * L2 / mu) * (ri * ri);
   }
   const float rf = f32_of(r);
-  const double ri = rcp_seeded(r, rf);
+  const double ri = rcp_seeded(r, rf, op);
   double V, dV;
-  pot_tab<false>(q, r, ri, rf, T, &V, &dV, nullptr);
-  return fma(0.5 * L2 * inv_mu, ri * ri, V);
+  pot_tab<false, true>(q, r, ri, rf, T, op, &V, &dV, nullptr);
+  return fma(0.5 * L2 * inv_mu, op.mul(ri, ri), V);
 }
 // g(r) = r^3 V'(r)
 template <bool TAB>
-__device__ __forceinline__ double gfun_(const DevPair& q, double r, const double* T) {
+__device__ __forceinline__ double gfun_(const DevPair& q, double r, const double* T,
+                                        const OpReg& op) {
   if (!TAB) return r * r * r * pot_dV(q, r);
   const float rf = f32_of(r);
   double V, dV;
-  pot_tab<false>(q, r, rcp_seeded(r, rf), rf, T, &V, &dV, nullptr);
-  return r * r * r * dV;
+  pot_tab<false, true>(q, r, rcp_seeded(r, rf, op), rf, T, op, &V, &dV, nullptr);
+  return op.mul(op.mul(op.mul(r, r), r), dV);
 }
 
 // Outer barrier of the effective potential V + L2/(2 mu r^2): the root
@@ -240,7 +255,8 @@ __device__ __forceinline__ double gfun_(const DevPair& q, double r, const double
 // Returns false when L2/mu >= g_max (no well).
 template <bool TAB>
 __device__ bool barrier_top(const DevPair& q, const DevShape& sh, double mu, double inv_mu,
-                            double L2, const double* T, double* r_top, double* thr) {
+                            double L2, const double* T, const OpReg& op, double* r_top,
+                            double* thr) {
   if (L2 <= 0.0) {
     *r_top = INFINITY;
     *thr = 0.0;
@@ -248,7 +264,7 @@ __device__ bool barrier_top(const DevPair& q, const DevShape& sh, double mu, dou
   }
   const double c = TAB ? L2 * inv_mu : L2 / mu;
   if (!(c < sh.g_max)) return false;
-  auto G = [&](double r) { return gfun_<TAB>(q, r, T) - c; };
+  auto G = [&](double r) { return gfun_<TAB>(q, r, T, op) - c; };
   double a = sh.r_peak, b = 2.0 * sh.r_peak, gb = G(b);
   for (int it = 0; it < 60 && gb >= 0.0; ++it) {
     a = b;
@@ -267,8 +283,8 @@ __device__ bool barrier_top(const DevPair& q, const DevShape& sh, double mu, dou
     auto GD = [&](double r, double* d1) {
       const float rf = f32_of(r);
       double V, dV, d2V;
-      pot_tab<true>(q, r, rcp_seeded(r, rf), rf, T, &V, &dV, &d2V);
-      const double r2 = r * r;
+      pot_tab<true, true>(q, r, rcp_seeded(r, rf, op), rf, T, op, &V, &dV, &d2V);
+      const double r2 = op.mul(r, r);
       *d1 = r2 * fma(r, d2V, 3.0 * dV);
       return fma(r2 * r, dV, -c);
     };
@@ -276,7 +292,7 @@ __device__ bool barrier_top(const DevPair& q, const DevShape& sh, double mu, dou
   } else {
     *r_top = illinois(G, a, b, G(a), gb);
   }
-  *thr = veff_<TAB>(q, mu, inv_mu, L2, *r_top, T);
+  *thr = veff_<TAB>(q, mu, inv_mu, L2, *r_top, T, op);
   return true;
 }
 
@@ -284,7 +300,7 @@ __device__ bool barrier_top(const DevPair& q, const DevShape& sh, double mu, dou
 // threshold).  Returns false when L2/mu >= g_max (no well).
 __device__ bool eff_well(const DevPair& q, const DevShape& sh, double mu, double L2,
                          double* r_min, double* r_top, double* thr) {
-  if (!barrier_top<false>(q, sh, mu, 0.0, L2, nullptr, r_top, thr)) return false;
+  if (!barrier_top<false>(q, sh, mu, 0.0, L2, nullptr, OpReg{}, r_top, thr)) return false;
   if (L2 <= 0.0) {
     *r_min = sh.r_eq;
     return true;
@@ -302,8 +318,8 @@ __device__ bool eff_well(const DevPair& q, const DevShape& sh, double mu, double
 template <bool TAB>
 __device__ bool turning_points(const DevPair& q, const DevShape& sh, double mu, double inv_mu,
                                double L2, double E, double r_in, double r_top, const double* T,
-                               double* rm, double* rp) {
-  auto f = [&](double r) { return veff_<TAB>(q, mu, inv_mu, L2, r, T) - E; };
+                               const OpReg& op, double* rm, double* rp) {
+  auto f = [&](double r) { return veff_<TAB>(q, mu, inv_mu, L2, r, T, op) - E; };
   double fin = f(r_in);
   if (!(fin < 0.0)) return false;
   // inner: V_eff rises steeply toward small r (Buckingham: up to r_b)
@@ -327,9 +343,9 @@ __device__ bool turning_points(const DevPair& q, const DevShape& sh, double mu, 
   // f'(r) = V'(r) - 2 a / r^3
   auto fd = [&](double r, double* d1) {
     const float rf = f32_of(r);
-    const double ri = rcp_seeded(r, rf), ri2 = ri * ri;
+    const double ri = rcp_seeded(r, rf, op), ri2 = op.mul(ri, ri);
     double V, dV;
-    pot_tab<false>(q, r, ri, rf, T, &V, &dV, nullptr);
+    pot_tab<false, true>(q, r, ri, rf, T, op, &V, &dV, nullptr);
     *d1 = fma(-2.0 * a2, ri2 * ri, dV);
     return fma(a2, ri2, V) - E;
   };
@@ -361,7 +377,8 @@ __device__ bool turning_points(const DevPair& q, const DevShape& sh, double mu, 
 // E - V_eff below 2^-126, where sqrt contributes below 1e-19, are dropped).
 template <int NG, bool TAB, bool PERIOD>
 __device__ void action_period(const DevPair& q, double mu, double inv_mu, double L2, double E,
-                              double rm, double rp, const double* T, double* act, double* per) {
+                              double rm, double rp, const double* T, const OpReg& op, double* act,
+                              double* per) {
   const double c = 0.5 * (rp + rm), d = 0.5 * (rp - rm);
   const double a = TAB ? 0.5 * L2 * inv_mu : L2 / (2.0 * mu);
   double sa = 0.0, sp = 0.0;
@@ -374,14 +391,14 @@ __device__ void action_period(const DevPair& q, double mu, double inv_mu, double
       const double r = sgn ? fma(-d, sn, c) : fma(d, sn, c);
       if (TAB) {
         const float rf = f32_of(r);
-        const double ri = rcp_seeded(r, rf);
+        const double ri = rcp_seeded(r, rf, op);
         double V, dV;
-        pot_tab<false>(q, r, ri, rf, T, &V, &dV, nullptr);
-        const double g = fma(-a, ri * ri, E) - V;
+        pot_tab<false, true>(q, r, ri, rf, T, op, &V, &dV, nullptr);
+        const double g = fma(-V, op.one(), fma(-a, op.mul(ri, ri), E));
         if (g > 0x1.0p-126) {
           float gf;
-          const double rg = rsqrt_seeded(g, gf);
-          sa = fma(wc, g * rg, sa);
+          const double rg = rsqrt_seeded(g, gf, op);
+          sa = fma(wc, op.mul(g, rg), sa);
           if (PERIOD) sp = fma(wc, rg, sp);
         }
       } else {
@@ -413,20 +430,22 @@ __device__ void action_period(const DevPair& q, double mu, double inv_mu, double
 //    r_top (g is unimodal there), so g(r) < L2/mu at r > r_peak means
 //    r > r_top: the pair is outside its barrier.
 __device__ __forceinline__ bool pair_candidate(const DevPair& q, const DevShape& sh, double mu,
-                                               double L2, double E, double r, const double* T) {
+                                               double L2, double E, double r, const double* T,
+                                               const OpReg& op) {
   // E >= L2 / (2 mu r_peak^2), L2 / mu >= g_max and g(r) < L2 / mu, multiplied out
   if (!sh.ok || (2.0 * mu) * (sh.r_peak * sh.r_peak) * E >= L2) return false;
   if (!(L2 < sh.g_max * mu)) return false;
-  return !(r > sh.r_peak && gfun_<true>(q, r, T) * mu < L2);
+  return !(r > sh.r_peak && gfun_<true>(q, r, T, op) * mu < L2);
 }
 // pair_bound: the test itself for a candidate.  Sets r_top for the
 // turning-point search.
 __device__ bool pair_bound(const DevPair& q, const DevShape& sh, double mu, double inv_mu,
-                           double L2, double E, double r, const double* T, double* r_top) {
+                           double L2, double E, double r, const double* T, const OpReg& op,
+                           double* r_top) {
   double thr;
-  if (!barrier_top<true>(q, sh, mu, inv_mu, L2, T, r_top, &thr)) return false;
+  if (!barrier_top<true>(q, sh, mu, inv_mu, L2, T, op, r_top, &thr)) return false;
   bool b = E < thr && r < *r_top;
-  if (q.kind == QCAMS_BUCK) b = b && r > sh.r_b && E < veff_<true>(q, mu, inv_mu, L2, sh.r_b, T);
+  if (q.kind == QCAMS_BUCK) b = b && r > sh.r_b && E < veff_<true>(q, mu, inv_mu, L2, sh.r_b, T, op);
   return b;
 }
 
@@ -438,7 +457,7 @@ __device__ bool pair_bound(const DevPair& q, const DevShape& sh, double mu, doub
 // Gaussian-binning width sigma (host-computed).
 __device__ void analyze_lane(const SysSet& sys, const DevShape* shapes, double gb_c1,
                              double gb_c2, const DevBatch& B, int64_t i,
-                             const double* __restrict__ sT) {
+                             const double* __restrict__ sT, const OpReg& op) {
   const int st = B.status[i];
   const int sid = B.sys_id[i];
   int cls = QCAMS_CLS_FAIL;
@@ -466,10 +485,10 @@ __device__ void analyze_lane(const SysSet& sys, const DevShape* shapes, double g
       const double mu = S.mu_pair[k];
       const double s2 = fma(r[0], r[0], fma(r[1], r[1], r[2] * r[2]));
       float rf;
-      d[k] = s2 * rsqrt_seeded(s2, rf);
+      d[k] = s2 * rsqrt_seeded(s2, rf, op);
       // pairs beyond the FP32 range of r^2 (never met) fall back to sqrt
       if (!(d[k] == d[k])) d[k] = sqrt(s2);
-      const double V = pot_V_<true>(S.pair[k], d[k], sT);
+      const double V = pot_V_<true>(S.pair[k], d[k], sT, op);
       Vsum += V;
       const double Lx = r[1] * v[2] - r[2] * v[1];
       const double Ly = r[2] * v[0] - r[0] * v[2];
@@ -485,12 +504,13 @@ __device__ void analyze_lane(const SysSet& sys, const DevShape* shapes, double g
       // candidate per lane at a time: nearly every lane has at most one, and
       // the lanes of a warp search theirs together whichever pair it is
       // (1 M lanes of all arrangements: 4.83 ms with a search per pair, now
-      // 4.35 ms).
+      // 4.35 ms; 3.8 ms with the products as register DFMAs and the shared
+      // LJ powers).
       unsigned cand = 0;
 #pragma unroll
       for (int k = 0; k < 3; ++k)
         cand |= pair_candidate(S.pair[k], shapes[sid * 3 + k], S.mu_pair[k], L2p[k], Ep[k], d[k],
-                               sT) ? 1u << k : 0u;
+                               sT, op) ? 1u << k : 0u;
       int nb = 0, which = 0;
       double E = 0.0, L2 = 0.0, r = 0.0, r_top = INFINITY;
       for (; cand; cand &= cand - 1) {
@@ -501,7 +521,7 @@ __device__ void analyze_lane(const SysSet& sys, const DevShape* shapes, double g
         const double rk = k == 0 ? d[0] : (k == 1 ? d[1] : d[2]);
         double top;
         if (pair_bound(S.pair[k], shapes[sid * 3 + k], S.mu_pair[k], S.inv_mu_pair[k], L2k, Ek, rk,
-                       sT, &top)) {
+                       sT, op, &top)) {
           ++nb;
           which = k;
           E = Ek;
@@ -521,7 +541,7 @@ __device__ void analyze_lane(const SysSet& sys, const DevShape* shapes, double g
         const DevPair& q = S.pair[which];
         const DevShape sh = shapes[sid * 3 + which];
         double r_in = r;
-        if (!(veff_<true>(q, mu, inv_mu, L2, r, sT) < E)) {
+        if (!(veff_<true>(q, mu, inv_mu, L2, r, sT, op) < E)) {
           // at a turning point within rounding: split at the well bottom
           double rmin, rt, thr;
           if (!eff_well(q, sh, mu, L2, &rmin, &rt, &thr)) rmin = sh.r_eq;
@@ -529,14 +549,14 @@ __device__ void analyze_lane(const SysSet& sys, const DevShape* shapes, double g
         }
         double rm, rp, act, per;
         vp = -0.5;
-        if (turning_points<true>(q, sh, mu, inv_mu, L2, E, r_in, r_top, sT, &rm, &rp)) {
-          action_period<kGL32, true, false>(q, mu, inv_mu, L2, E, rm, rp, sT, &act, &per);
+        if (turning_points<true>(q, sh, mu, inv_mu, L2, E, r_in, r_top, sT, op, &rm, &rp)) {
+          action_period<kGL32, true, false>(q, mu, inv_mu, L2, E, rm, rp, sT, op, &act, &per);
           vp = fma(S.s2mu_pi[which], act, -0.5);   // sqrt(2 mu) / pi * act - 1/2
         }
         {  // j' (j' + 1) = L2: j' = (sqrt(1 + 4 L2) - 1) / 2
           const double s4 = fma(4.0, L2, 1.0);
           float sf;
-          double sq = s4 * rsqrt_seeded(s4, sf);
+          double sq = s4 * rsqrt_seeded(s4, sf, op);
           if (!(sq == sq)) sq = sqrt(s4);
           jp = fma(0.5, sq, -0.5);
         }

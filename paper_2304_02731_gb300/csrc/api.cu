@@ -388,6 +388,7 @@ __device__ DevLevel solve_level(const DevPair& q, const DevShape& sh, double mu,
   DevLevel L{};
   L.ok = 0;
   if (!sh.ok) return L;
+  const OpReg none{};   // unused by the TAB = false forms
   const double L2 = (double)j * (double)(j + 1);
   double r_min, r_top, Etop;
   if (!eff_well(q, sh, mu, L2, &r_min, &r_top, &Etop)) return L;
@@ -395,8 +396,8 @@ __device__ DevLevel solve_level(const DevPair& q, const DevShape& sh, double mu,
   const double s2mu = sqrt(2.0 * mu);
   double lo = Vmin, hi = Etop - 1e-10 * (Etop - Vmin);
   double rm, rp, act, per;
-  if (!turning_points<false>(q, sh, mu, 0.0, L2, hi, r_min, r_top, nullptr, &rm, &rp)) return L;
-  action_period<kGL128, false, true>(q, mu, 0.0, L2, hi, rm, rp, nullptr, &act, &per);
+  if (!turning_points<false>(q, sh, mu, 0.0, L2, hi, r_min, r_top, nullptr, none, &rm, &rp)) return L;
+  action_period<kGL128, false, true>(q, mu, 0.0, L2, hi, rm, rp, nullptr, none, &act, &per);
   if (-0.5 + s2mu / kPi * act < v) return L;
   // harmonic first guess
   double k2 = pot_d2V(q, r_min) + 3.0 * L2 / (mu * r_min * r_min * r_min * r_min);
@@ -404,8 +405,8 @@ __device__ DevLevel solve_level(const DevPair& q, const DevShape& sh, double mu,
   if (!(E > lo && E < hi)) E = 0.5 * (lo + hi);
   bool ok = false;
   for (int it = 0; it < 200; ++it) {
-    if (!turning_points<false>(q, sh, mu, 0.0, L2, E, r_min, r_top, nullptr, &rm, &rp)) break;
-    action_period<kGL128, false, true>(q, mu, 0.0, L2, E, rm, rp, nullptr, &act, &per);
+    if (!turning_points<false>(q, sh, mu, 0.0, L2, E, r_min, r_top, nullptr, none, &rm, &rp)) break;
+    action_period<kGL128, false, true>(q, mu, 0.0, L2, E, rm, rp, nullptr, none, &act, &per);
     const double f = -0.5 + s2mu / kPi * act - v;
     if (f < 0) lo = E; else hi = E;
     double En = E - f * 2.0 * kPi / (s2mu * per);
@@ -418,8 +419,8 @@ __device__ DevLevel solve_level(const DevPair& q, const DevShape& sh, double mu,
     E = En;
   }
   if (!ok) return L;
-  if (!turning_points<false>(q, sh, mu, 0.0, L2, E, r_min, r_top, nullptr, &rm, &rp)) return L;
-  action_period<kGL128, false, true>(q, mu, 0.0, L2, E, rm, rp, nullptr, &act, &per);
+  if (!turning_points<false>(q, sh, mu, 0.0, L2, E, r_min, r_top, nullptr, none, &rm, &rp)) return L;
+  action_period<kGL128, false, true>(q, mu, 0.0, L2, E, rm, rp, nullptr, none, &act, &per);
   L.E = E;
   L.r_minus = rm;
   L.r_plus = rp;
@@ -541,7 +542,7 @@ __device__ bool warp_well(const DevPair& q, const DevShape& sh, double mu, doubl
   *r_min = __shfl_sync(0xffffffffu, root, 1);
   if (!far) {
     *r_top = __shfl_sync(0xffffffffu, root, 0);
-    *thr = veff_<false>(q, mu, 0.0, L2, *r_top, nullptr);
+    *thr = veff_<false>(q, mu, 0.0, L2, *r_top, nullptr, OpReg{});
   }
   return true;
 }
@@ -550,7 +551,7 @@ __device__ bool warp_well(const DevPair& q, const DevShape& sh, double mu, doubl
 // the inner root in the even lanes and the outer in the odd ones).
 __device__ bool warp_turning_points(const DevPair& q, const DevShape& sh, double mu, double L2,
                                     double E, double r_in, double r_top, double* root) {
-  auto f = [&](double r) { return veff_<false>(q, mu, 0.0, L2, r, nullptr) - E; };
+  auto f = [&](double r) { return veff_<false>(q, mu, 0.0, L2, r, nullptr, OpReg{}) - E; };
   const double fin = f(r_in);
   if (!(fin < 0.0)) return false;
   const bool outer = threadIdx.x & 1, fixed = outer ? isfinite(r_top) : q.kind == QCAMS_BUCK;
@@ -786,10 +787,13 @@ __global__ void k_init(SysSet sys, const DevLevel* levels, const double* E_col, 
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(128) k_analyze(SysSet sys, const DevShape* shapes,
                                                  double gb_c1, double gb_c2, DevBatch B) {
-  __shared__ double sT[kExpTableSize];
-  load_exp_table(sT);
+  __shared__ double sT[kExpTableSize], sK[kOpRegs];
+  op_reg_fill(sK);
+  load_exp_table(sT);   // ends with a barrier
+  OpReg op;
+  op.load(sK);
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < B.n) analyze_lane(sys, shapes, gb_c1, gb_c2, B, i, sT);
+  if (i < B.n) analyze_lane(sys, shapes, gb_c1, gb_c2, B, i, sT, op);
 }
 
 // ---------------------------------------------------------------------------
