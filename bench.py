@@ -63,8 +63,8 @@ KERNEL_SOURCES = {
     32: ["integrate32.cu", "dp5_tableau.cuh"],
 }
 COUNTS_SOURCE_SHA256 = {
-    64: "cf67eb8adb5624b72744b7ef0d6d4d0e2fea000478fff561090cccdf7322210e",
-    32: "d9cbe3757a6014589cdc38132e600b44ad5e99066d6bdb99841805d6197d8421",
+    64: "c5c711b08e4c160ee1e340674749742f91cf64cb3f74faff5867c834b0e0c21f",
+    32: "493f2ca84977c5e0b6e09d372d6e9d5d1ccc543957470b9b0cb5e2370225a9f3",
 }
 # DRAM bytes per trajectory of the integrator: ncu dram__bytes_read.sum +
 # dram__bytes_write.sum of the same FP64 profile case (1,110,784 B read,
@@ -77,6 +77,19 @@ DRAM_BYTES_PER_LANE = 1110784 / 3840
 # The same for the FP32 kernel (559,360 B read, no table): its state is
 # loaded as (value, compensation) pairs from the same FP64 arrays.
 DRAM_BYTES_PER_LANE_FP32 = 559360 / 3840
+
+
+def integrator_launches(precision, persistent, n):
+    """Kernels of one integrator run: the queue order (3), the start step and
+    the stages that a batch of n lanes takes (csrc/integrate.cu); init,
+    shapes, analysis and reduction are 8 more."""
+    import torch
+    per_sm = n / torch.cuda.get_device_properties(0).multi_processor_count
+    if precision == 32:
+        return 4 if persistent == 1 and per_sm > 512 else 1
+    if persistent not in (0, 1):
+        return 1
+    return 7 if per_sm > 120 else 4 if per_sm > 80 else 3 if per_sm > 20 else 2
 
 
 def kernel_sources_sha256(precision: int) -> str:
@@ -513,7 +526,7 @@ def run_ours(args):
                    "parallelism": (f"id-range shards x{world} + int64 all_reduce of the "
                                    f"histograms" if world > 1 else "single GPU")},
         "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e,
-        "gpu_launches": 8 * args.steps,
+        "gpu_launches": (8 + integrator_launches(args.precision, integ.persistent, wl.n)) * args.steps,
         "clocks": clock_info,
         "outcomes": {"cls_counts_Q_RAC_RBC_D_AMBIG_FAIL": cls_counts,
                      "merged_cls_counts_all_ranks": merged_counts,

@@ -562,7 +562,8 @@ template <bool MORSE, bool ONE, int MINB>
 __global__ void __launch_bounds__(128, MINB) k_integrate32_persistent(SysSetF sys,
                                                                 const DevShape* shapes,
                                                                 IntegParams ip, DevBatch B,
-                                                                unsigned long long* counters) {
+                                                                unsigned long long* counters,
+                                                                const long long* list) {
   const unsigned lane = threadIdx.x & 31u;
   unsigned long long rhs = 0, steps = 0;
   Lane32 L;
@@ -580,7 +581,7 @@ __global__ void __launch_bounds__(128, MINB) k_integrate32_persistent(SysSetF sy
         const int64_t k = (int64_t)(base + __popc(want & ((1u << lane) - 1u)));
         if (k >= B.n) exhausted = true;
         else {
-          idx = k;
+          idx = list ? list[k] : k;
           have = load<MORSE, ONE>(sys, shapes, ip, B, idx, L, rhs);
         }
       }
@@ -658,12 +659,21 @@ cudaError_t launch32_persistent(const SysSetF& sf, const DevShape* shapes, const
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
       &per_sm, k_integrate32_persistent<MORSE, ONE, MINB>, block, 0);
   if (e != cudaSuccess) return e;
+  const long long* list = nullptr;
+  // More lanes than are resident at once: the slowest collisions first
+  // (figures at launch_queue_order).
+  if (b.n > 4 * 128 * (int64_t)ctx.sm_count && lists_usable(b)) {
+    long long* order = reinterpret_cast<long long*>(b.vprime);
+    e = launch_queue_order(b, order, reinterpret_cast<unsigned*>(b.jprime), ctx.counters + 3, st);
+    if (e != cudaSuccess) return e;
+    list = order;
+  }
   long long grid = (long long)(per_sm < 1 ? 1 : per_sm) * ctx.sm_count;
   const long long need_blocks = (b.n + block - 1) / block;
   if (grid > need_blocks) grid = need_blocks;
   if (grid < 1) grid = 1;
   k_integrate32_persistent<MORSE, ONE, MINB><<<(unsigned)grid, block, 0, st>>>(sf, shapes, ip, b,
-                                                                              ctx.counters);
+                                                                              ctx.counters, list);
   return cudaGetLastError();
 }
 

@@ -695,7 +695,7 @@ __global__ void __launch_bounds__(kQueueBlock, G == 3 ? 3 : 4)
         } else {
           idx = q.list_in ? q.list_in[k] : k;
           st = B.status[idx];
-          started = q.list_in && (st & kHandoff);
+          started = q.handed_on && (st & kHandoff);
           const int s_in = B.sys_id[idx];
           const bool run = started || runnable(st), ok = s_in >= 0 && s_in < sys.n;
           fresh = run && ok;

@@ -87,6 +87,7 @@ struct StageQueue {
   long long* list_out = nullptr;
   unsigned long long* n_out = nullptr;
   long long keep = 0;
+  bool handed_on = false;                     // list_in came from an earlier stage
 };
 // Whether a stage with n source entries hands on now (same in all lanes).
 __device__ __forceinline__ bool stage_over(const StageQueue& q, long long n, int lane) {
@@ -99,6 +100,13 @@ __device__ __forceinline__ bool stage_over(const StageQueue& q, long long n, int
 // Lane status bits of a handed-on trajectory (never seen by a caller).
 constexpr int kHandoff = 0x40, kHandoffRejected = 0x80;
 constexpr int kCounters = 32;   // work counters of one run
+
+// Lists of lanes kept in two of the batch's output arrays during a run
+// (integrate.cu): whether the batch's arrays allow it, and the queue order of
+// its lanes (scratch: 16 KB; *n_out receives the list's length).
+bool lists_usable(const DevBatch& b);
+cudaError_t launch_queue_order(const DevBatch& b, long long* list, unsigned* scratch,
+                               unsigned long long* n_out, cudaStream_t st);
 
 // `lanes` = 3 or 6 lanes per trajectory, bit for bit the one-thread kernels'
 // results (integrate_grp.cu); at most n_max trajectories in the source, all

@@ -95,3 +95,26 @@ def test_one_buffer_for_several_outputs(Q):
         runs.append(_values(b))
     for k in ("y", "t", "h", "dE", "status", "cls", "nsteps", "nrej", "vt", "jt"):
         assert np.array_equal(runs[0][k], runs[1][k]), k
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("study", ["morse", "mixed"])
+def test_fp32_queue_order(Q, study):
+    """FP32 batches beyond what the GPU holds at once are taken slowest
+    collisions first: each lane as in a batch that is taken as it comes."""
+    import torch
+    w = _morse() if study == "morse" else W.mixed_ca_h(n=98_304 + 1, seed=5)
+    integ = Q.make_integ(**W.INTEG_FP32, precision=32, persistent=True)
+    start = Q.Batch.empty(w.n, "cuda", sys_id=w.sys_id)
+    Q.init_states(w.systems, start, w.E, w.b, w.v, w.j, w.R0, w.seed)
+    start.f64["t_scale"][3] = 0.0                # ends at its first step
+    big = _subset(Q, start, torch.arange(w.n, device="cuda"))
+    Q.run_batch(w.systems, big, integ)
+    whole = _values(big)
+    idx = torch.as_tensor(np.r_[0:7, 40_000:42_001, w.n - 5:w.n], device="cuda")
+    part = _subset(Q, start, idx)
+    Q.run_batch(w.systems, part, integ)
+    got = _values(part)
+    for k in FIELDS:
+        want = whole[k][..., idx.cpu().numpy()]
+        assert np.array_equal(got[k], want, equal_nan=got[k].dtype.kind == "f"), k
