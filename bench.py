@@ -63,7 +63,7 @@ KERNEL_SOURCES = {
     32: ["integrate32.cu", "dp5_tableau.cuh"],
 }
 COUNTS_SOURCE_SHA256 = {
-    64: "c5c711b08e4c160ee1e340674749742f91cf64cb3f74faff5867c834b0e0c21f",
+    64: "1ce3dfbc27c1fe570895340b07dbf712687f3e729d3a10d1e301bf61d694be23",
     32: "493f2ca84977c5e0b6e09d372d6e9d5d1ccc543957470b9b0cb5e2370225a9f3",
 }
 # DRAM bytes per trajectory of the integrator: ncu dram__bytes_read.sum +

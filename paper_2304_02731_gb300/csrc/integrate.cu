@@ -544,23 +544,36 @@ __global__ void __launch_bounds__(128) k_start_step(SysSet sys, IntegParams ip, 
 // the long-lived complexes; a long trajectory that is taken last runs alone
 // at the end.  A counting sort over kOrderBuckets buckets (the leading float
 // bits of t_scale, 16 to the octave): the order within a bucket is free, and
-// results do not depend on the order at all.  It moves 24 bytes a lane, which
-// is little beside the run: with it 200,000 mixed lanes at scattered energies
-// take 610 ms instead of 766 (FP64), and 1,000,000 labelling lanes 28.9 ms
-// instead of 35.5 (FP32); a sweep of equal cells 110.7 ms with and without.
+// results do not depend on the order at all.  Lanes that already come that way
+// (a sweep of rising energies) keep their own order, since neighbours of equal
+// length finish together: 221,184 of them took 0.35 % more when shuffled.
+// It moves 40 bytes a lane, which is little beside the run: with it 200,000
+// mixed lanes at scattered energies take 612 ms instead of 763 (FP64), and
+// 1,000,000 labelling lanes 28.6 ms instead of 38.4 (FP32).
 constexpr int kOrderBuckets = 4096, kOrderBlock = 1024, kOrderChunk = 4096;
 
 __device__ __forceinline__ int order_bucket(const DevBatch& B, int64_t i) {
   return (int)((__float_as_uint((float)B.t_scale[i]) >> 19) & (kOrderBuckets - 1));
 }
 
+// Bucket counts; count[kOrderBuckets] becomes 1 if a lane has a slower one
+// next to it or half a batch behind it, by more than four buckets (a quarter
+// of an octave): the vibrational phase moves R, and so t_scale, by up to ten
+// percent among the lanes of a cell.
 __global__ void __launch_bounds__(kOrderBlock) k_order_count(DevBatch B, unsigned* count) {
   __shared__ unsigned h[kOrderBuckets];
+  const int64_t half = B.n / 2;
+  bool mixed = false;
   for (int k = threadIdx.x; k < kOrderBuckets; k += kOrderBlock) h[k] = 0u;
   __syncthreads();
   for (int64_t i = blockIdx.x * (int64_t)kOrderBlock + threadIdx.x; i < B.n;
-       i += (int64_t)gridDim.x * kOrderBlock)
-    atomicAdd(&h[order_bucket(B, i)], 1u);
+       i += (int64_t)gridDim.x * kOrderBlock) {
+    const int k = order_bucket(B, i);
+    mixed |= i + 1 < B.n && k + 4 < order_bucket(B, i + 1);
+    mixed |= i + half < B.n && k + 4 < order_bucket(B, i + half);
+    atomicAdd(&h[k], 1u);
+  }
+  if (mixed) count[kOrderBuckets] = 1u;
   __syncthreads();
   for (int k = threadIdx.x; k < kOrderBuckets; k += kOrderBlock)
     if (h[k]) atomicAdd(&count[k], h[k]);
@@ -602,6 +615,11 @@ __global__ void __launch_bounds__(kOrderBlock) k_order_place(DevBatch B, unsigne
                                                              long long* list) {
   __shared__ unsigned h[kOrderBuckets];
   const int64_t base = (int64_t)blockIdx.x * kOrderChunk;
+  if (next[kOrderBuckets] == 0u) {   // in order as they come
+    for (int64_t i = base + threadIdx.x; i < base + kOrderChunk && i < B.n; i += kOrderBlock)
+      list[i] = i;
+    return;
+  }
   for (int k = threadIdx.x; k < kOrderBuckets; k += kOrderBlock) h[k] = 0u;
   __syncthreads();
   int bucket[kOrderChunk / kOrderBlock];
@@ -823,7 +841,7 @@ cudaError_t launch_integrate_shape(const SysSet& sys, const DevShape* shapes,
 
 cudaError_t launch_queue_order(const DevBatch& b, long long* list, unsigned* scratch,
                                unsigned long long* n_out, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(scratch, 0, kOrderBuckets * sizeof(unsigned), st);
+  cudaError_t e = cudaMemsetAsync(scratch, 0, (kOrderBuckets + 1) * sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
   const int64_t chunks = (b.n + kOrderChunk - 1) / kOrderChunk;
   k_order_count<<<(unsigned)(chunks < 304 ? chunks : 304), kOrderBlock, 0, st>>>(b, scratch);
@@ -874,7 +892,7 @@ namespace {
 //    step when each sub-partition has one warp).
 // 12,288 sweep lanes take 460 ms this way, 572 ms with three lanes to the
 // end, 660 ms without packing and 1,250 ms in the one-thread kernel alone;
-// 200,000 mixed lanes 610 ms (766 without the queue order) against 1,440 ms.
+// 200,000 mixed lanes 612 ms (763 without the queue order) against 1,440 ms.
 struct Stage {
   int lanes;         // lanes per trajectory (1: the persistent kernel)
   int keep_per_sm;   // hands on at this many trajectories per SM (0: none)
