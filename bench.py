@@ -63,8 +63,8 @@ KERNEL_SOURCES = {
     32: ["integrate32.cu", "dp5_tableau.cuh"],
 }
 COUNTS_SOURCE_SHA256 = {
-    64: "1ce3dfbc27c1fe570895340b07dbf712687f3e729d3a10d1e301bf61d694be23",
-    32: "493f2ca84977c5e0b6e09d372d6e9d5d1ccc543957470b9b0cb5e2370225a9f3",
+    64: "11739afbfbcc33e4bae9fe47ce58383f551317ddf4ff075736ec254c1577b4fe",
+    32: "1f1f476a60b80403d10ad407c867c5c3107bf21770a4aefbbd1addb6c36f9731",
 }
 # DRAM bytes per trajectory of the integrator: ncu dram__bytes_read.sum +
 # dram__bytes_write.sum of the same FP64 profile case (1,110,784 B read,

@@ -841,6 +841,7 @@ cudaError_t launch_integrate_shape(const SysSet& sys, const DevShape* shapes,
 
 cudaError_t launch_queue_order(const DevBatch& b, long long* list, unsigned* scratch,
                                unsigned long long* n_out, cudaStream_t st) {
+  static_assert(8 * kOrderMinLanes >= 4 * (kOrderBuckets + 1), "counts fit in jprime");
   cudaError_t e = cudaMemsetAsync(scratch, 0, (kOrderBuckets + 1) * sizeof(unsigned), st);
   if (e != cudaSuccess) return e;
   const int64_t chunks = (b.n + kOrderChunk - 1) / kOrderChunk;
@@ -915,7 +916,7 @@ cudaError_t launch_stages(const SysSet& sys, const DevShape* shapes, const Integ
   StageQueue q;
   long long* list[2] = {reinterpret_cast<long long*>(b.vprime),
                         reinterpret_cast<long long*>(b.jprime)};
-  if (lists && b.n > kOrderMinPerSm * sms) {   // slowest collisions first
+  if (lists && b.n > kOrderMinPerSm * sms && b.n >= kOrderMinLanes) {   // slowest collisions first
     cudaError_t e = launch_queue_order(b, list[0], reinterpret_cast<unsigned*>(b.jprime),
                                        ctx.counters + 3, st);
     if (e != cudaSuccess) return e;

@@ -662,7 +662,7 @@ cudaError_t launch32_persistent(const SysSetF& sf, const DevShape* shapes, const
   const long long* list = nullptr;
   // More lanes than are resident at once: the slowest collisions first
   // (figures at launch_queue_order).
-  if (b.n > 4 * 128 * (int64_t)ctx.sm_count && lists_usable(b)) {
+  if (b.n > 4 * 128 * (int64_t)ctx.sm_count && b.n >= kOrderMinLanes && lists_usable(b)) {
     long long* order = reinterpret_cast<long long*>(b.vprime);
     e = launch_queue_order(b, order, reinterpret_cast<unsigned*>(b.jprime), ctx.counters + 3, st);
     if (e != cudaSuccess) return e;

@@ -103,7 +103,9 @@ constexpr int kCounters = 32;   // work counters of one run
 
 // Lists of lanes kept in two of the batch's output arrays during a run
 // (integrate.cu): whether the batch's arrays allow it, and the queue order of
-// its lanes (scratch: 4,097 words; *n_out receives the list's length).
+// its lanes (scratch: 4,097 words, which jprime holds from kOrderMinLanes lanes
+// on; *n_out receives the list's length).
+constexpr int64_t kOrderMinLanes = 4096;
 bool lists_usable(const DevBatch& b);
 cudaError_t launch_queue_order(const DevBatch& b, long long* list, unsigned* scratch,
                                unsigned long long* n_out, cudaStream_t st);
