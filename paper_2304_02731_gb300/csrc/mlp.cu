@@ -410,9 +410,11 @@ __device__ __forceinline__ void block_dw(const __nv_bfloat16 (*dzt)[LDT],
 }
 
 // Bias gradients of a 64-unit layer: the sums over the 16 samples of dZ's
-// columns, added to gb.  The 16 columns of a lane quad are reduced over its
-// eight row lanes by halving (14 shuffles), which leaves lane (g, q) with
-// columns 8 g + 2 q and + 1.
+// columns, added to gb.  A column's order of sums is that of a butterfly over
+// the eight row lanes: rows g and g + 8, then lanes g ^ 1, g ^ 2 and g ^ 4.
+// The 16 columns of a lane quad take those three steps by halving (14
+// shuffles where butterflies take 48), which leaves lane (g, q) with columns
+// 8 r + 2 q and + 1, r being g with its three bits reversed.
 __device__ __forceinline__ void accumulate_db(const float (*dz)[4], float* gb) {
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
   float s[8][2];
@@ -422,18 +424,19 @@ __device__ __forceinline__ void accumulate_db(const float (*dz)[4], float* gb) {
     s[t][1] = dz[t][1] + dz[t][3];
   }
 #pragma unroll
-  for (int half = 4; half > 0; half >>= 1) {
-    const bool up = g & half;
+  for (int bit = 1, half = 4; half > 0; bit <<= 1, half >>= 1) {
+    const bool up = g & bit;
 #pragma unroll
     for (int t = 0; t < half; ++t)
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         const float send = up ? s[t][e] : s[t + half][e], keep = up ? s[t + half][e] : s[t][e];
-        s[t][e] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * half);
+        s[t][e] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * bit);
       }
   }
-  atomicAdd(&gb[8 * g + 2 * q], s[0][0]);
-  atomicAdd(&gb[8 * g + 2 * q + 1], s[0][1]);
+  const int r = (g & 1) << 2 | (g & 2) | g >> 2;
+  atomicAdd(&gb[8 * r + 2 * q], s[0][0]);
+  atomicAdd(&gb[8 * r + 2 * q + 1], s[0][1]);
 }
 // The same for the 4 outputs (columns 0-3 of one tile).
 __device__ __forceinline__ void accumulate_db4(const float* dz, float* gb) {
