@@ -143,8 +143,7 @@ __device__ __forceinline__ float sigm(float z) { return __fdividef(1.0f, 1.0f + 
 // Weights to shared memory (blockDim.x == THREADS).  With p 16-byte aligned
 // every matrix starts on a 16-byte boundary: each thread issues all of its
 // 16-byte loads of 8-element row segments first, then stores each segment
-// to its row.  Otherwise, element loads.  All loads go to L2: the training
-// kernel's other blocks rewrite the parameters between its steps.
+// to its row.  Otherwise, element loads.
 __device__ void load_weights(WeightsSmem& W, const __nv_bfloat16* p, const float* pf) {
   const __nv_bfloat16 zero = __float2bfloat16(0.0f);
   if ((reinterpret_cast<uintptr_t>(p) & 15u) == 0) {
@@ -161,7 +160,7 @@ __device__ void load_weights(WeightsSmem& W, const __nv_bfloat16* p, const float
       else if (i < N1 + N2) off = OW2 + 8 * (i - N1);
       else if (i < N1 + 2 * N2) off = OW3 + 8 * (i - N1 - N2);
       else if (i < NSEG) off = OW4 + 8 * (i - N1 - 2 * N2);
-      if (i < NSEG) v[k] = __ldcg(reinterpret_cast<const uint4*>(p + off));
+      if (i < NSEG) v[k] = *reinterpret_cast<const uint4*>(p + off);
     }
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
@@ -180,29 +179,26 @@ __device__ void load_weights(WeightsSmem& W, const __nv_bfloat16* p, const float
     }
     for (int i = threadIdx.x; i < (8 - OUT) * H; i += blockDim.x) W.w4[OUT + i / H][i % H] = zero;
   } else {
-    auto ld = [&](int k) {
-      return __ushort_as_bfloat16(__ldcg(reinterpret_cast<const unsigned short*>(p) + k));
-    };
     for (int i = threadIdx.x; i < H * 16; i += blockDim.x) {
       const int r = i / 16, c = i % 16;
-      W.w1[r][c] = c < IN ? ld(OW1 + r * IN + c) : zero;
+      W.w1[r][c] = c < IN ? p[OW1 + r * IN + c] : zero;
     }
     for (int i = threadIdx.x; i < H * H; i += blockDim.x) {
       const int r = i / H, c = i % H;
-      W.w2[r][c] = ld(OW2 + i);
-      W.w3[r][c] = ld(OW3 + i);
+      W.w2[r][c] = p[OW2 + i];
+      W.w3[r][c] = p[OW3 + i];
     }
     for (int i = threadIdx.x; i < 8 * H; i += blockDim.x) {
       const int r = i / H, c = i % H;
-      W.w4[r][c] = r < OUT ? ld(OW4 + r * H + c) : zero;
+      W.w4[r][c] = r < OUT ? p[OW4 + r * H + c] : zero;
     }
   }
   for (int i = threadIdx.x; i < H; i += blockDim.x) {
-    W.b1[i] = __ldcg(pf + OB1 + i);
-    W.b2[i] = __ldcg(pf + OB2 + i);
-    W.b3[i] = __ldcg(pf + OB3 + i);
+    W.b1[i] = pf[OB1 + i];
+    W.b2[i] = pf[OB2 + i];
+    W.b3[i] = pf[OB3 + i];
   }
-  if (threadIdx.x < 8) W.b4[threadIdx.x] = threadIdx.x < OUT ? __ldcg(pf + OB4 + threadIdx.x) : 0.0f;
+  if (threadIdx.x < 8) W.b4[threadIdx.x] = threadIdx.x < OUT ? pf[OB4 + threadIdx.x] : 0.0f;
 }
 
 // Features of the 16 rows handled by this lane's fragment rows: either from
@@ -211,15 +207,13 @@ struct CellGrid {
   int n_b2, n_cth, n_phi, n_eta, n_chi;
   float E, v, j, b2_max;
 };
-// Minibatch rows: row i is sample i, or (draw) a uniform one of `n`, from
-// Philox4x32-10 with key = seed and counter (i, step_lo, step_hi, 4); the
-// 64-bit word w1:w0 is mapped by the high half of w * n (bias <= n / 2^64).
+// Minibatch rows: row i is a uniform one of `n` samples, from Philox4x32-10
+// with key = seed and counter (i, step_lo, step_hi, 4); the 64-bit word w1:w0
+// is mapped by the high half of w * n (bias <= n / 2^64).
 struct RowSrc {
-  bool draw;
   int64_t n;
   uint64_t seed, step;
   __device__ __forceinline__ int64_t at(int64_t i) const {
-    if (!draw) return i;
     const uint4 w = philox4x32_10(
         make_uint4((uint32_t)i, (uint32_t)step, (uint32_t)(step >> 32), 4u),
         make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
@@ -453,35 +447,27 @@ __device__ __forceinline__ void accumulate_db4(const float* dz, float* gb) {
   }
 }
 
-// Shared state of a gradient block before its first round (ends without a
-// barrier).
-template <int CPW>
-__device__ void grad_begin(TrainSmem<CPW>& S, const __nv_bfloat16* pb, const float* pf) {
-  load_weights(S.w, pb, pf);
-  for (int i = threadIdx.x; i < NGB; i += blockDim.x) S.gb[i] = 0.0f;
-}
-// Padding rows of the X^T and dZ4^T tiles (never written by the passes).
-template <int CPW>
-__device__ void grad_pad(TrainSmem<CPW>& S) {
-  constexpr int LDT = BlockTiles<CPW>::LDT;
-  const __nv_bfloat16 zero = __float2bfloat16(0.0f);
-  for (int i = threadIdx.x; i < (16 - IN) * LDT; i += blockDim.x) S.t.xt[IN + i / LDT][i % LDT] = zero;
-  for (int i = threadIdx.x; i < (16 - 8) * LDT; i += blockDim.x) S.t.dz4t[8 + i / LDT][i % LDT] = zero;
-}
-
-// This block's share of the gradient of the mean cross-entropy over n rows
-// (rows.at(r) the sample behind row r).  Block rounds of RS samples: each
+// Gradient of the mean cross-entropy over n rows: samples 0 .. n - 1 or, with
+// DRAW, the minibatch rows.at(0 .. n - 1).  Block rounds of RS samples: each
 // warp carries its chunks of 16 through the forward and backward passes
 // (activations and errors to the block tiles, bias gradients to shared FP32
 // sums), then the four weight gradients of the round are formed as block
 // GEMMs (warp w: rows 16w .. 16w+15 of dW1..dW3, columns 16w .. 16w+15 of
 // dW4) and added to the global gradient.
-template <int CPW>
-__device__ void grad_rounds(TrainSmem<CPW>& S, const Std& sd, const float* x,
-                            const uint8_t* label, const RowSrc& rows, int64_t n, float* grad,
-                            float* loss) {
-  constexpr int RS = BlockTiles<CPW>::RS;
-  if ((int64_t)blockIdx.x * RS >= n) return;   // no round for this block
+template <int CPW, bool DRAW>
+__global__ void __launch_bounds__(THREADS) k_mlp_grad(const __nv_bfloat16* pb, const float* pf,
+                                                      Std sd, const float* x,
+                                                      const uint8_t* label, RowSrc rows,
+                                                      int64_t n, float* grad, float* loss) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  TrainSmem<CPW>& S = *reinterpret_cast<TrainSmem<CPW>*>(smem_raw);
+  constexpr int RS = BlockTiles<CPW>::RS, LDT = BlockTiles<CPW>::LDT;
+  load_weights(S.w, pb, pf);
+  for (int i = threadIdx.x; i < NGB; i += blockDim.x) S.gb[i] = 0.0f;
+  // padding rows of the X^T and dZ4^T tiles (never written by the passes)
+  const __nv_bfloat16 zero = __float2bfloat16(0.0f);
+  for (int i = threadIdx.x; i < (16 - IN) * LDT; i += blockDim.x) S.t.xt[IN + i / LDT][i % LDT] = zero;
+  for (int i = threadIdx.x; i < (16 - 8) * LDT; i += blockDim.x) S.t.dz4t[8 + i / LDT][i % LDT] = zero;
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
   const float inv_n = 1.0f / (float)n;
@@ -493,7 +479,7 @@ __device__ void grad_rounds(TrainSmem<CPW>& S, const Std& sd, const float* x,
       const int64_t base = rnd * RS + col;
       float lg[4], ds[3][32];
       const int64_t r0 = base + g, r1 = base + g + 8;
-      const int64_t s0 = rows.at(r0), s1 = rows.at(r1);
+      const int64_t s0 = DRAW ? rows.at(r0) : r0, s1 = DRAW ? rows.at(r1) : r1;
       forward16<true, CPW>(S.w, ds, &S.t, col, x, s0, s1, n, base, nullptr, sd, lg);
       // softmax cross-entropy and dZ4 = (p - onehot) / n; rows past n and
       // rows without a target have dZ4 = 0 and so add nothing below
@@ -584,18 +570,6 @@ __device__ void grad_rounds(TrainSmem<CPW>& S, const Std& sd, const float* x,
   }
 }
 
-template <int CPW>
-__global__ void __launch_bounds__(THREADS) k_mlp_grad(const __nv_bfloat16* pb, const float* pf,
-                                                      Std sd, const float* x,
-                                                      const uint8_t* label, int64_t n,
-                                                      float* grad, float* loss) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  TrainSmem<CPW>& S = *reinterpret_cast<TrainSmem<CPW>*>(smem_raw);
-  grad_pad<CPW>(S);
-  grad_begin<CPW>(S, pb, pf);
-  grad_rounds<CPW>(S, sd, x, label, RowSrc{false, n, 0, 0}, n, grad, loss);
-}
-
 __global__ void __launch_bounds__(THREADS) k_mlp_infer(const __nv_bfloat16* pb, const float* pf,
                                                        Std sd, const float* x, int64_t n,
                                                        CellGrid grid, int use_grid,
@@ -632,97 +606,20 @@ __global__ void __launch_bounds__(THREADS) k_mlp_infer(const __nv_bfloat16* pb, 
   }
 }
 
-// One parameter's Adam step (beta1 0.9, beta2 0.999, eps 1e-8; c1, c2 the
-// bias corrections).
-__device__ __forceinline__ void adam_one(int i, float gr, float* p, float* m, float* v,
-                                         __nv_bfloat16* pb, float lr, float c1, float c2) {
-  const float mi = 0.9f * m[i] + 0.1f * gr;
-  const float vi = 0.999f * v[i] + 0.001f * gr * gr;
-  m[i] = mi;
-  v[i] = vi;
-  const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
-  p[i] = pi;
-  pb[i] = __float2bfloat16(pi);
-}
-
-__global__ void k_adam(float* p, float* m, float* v, const float* grad, __nv_bfloat16* pb,
-                       float lr, float c1, float c2) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < NP; i += gridDim.x * blockDim.x)
-    adam_one(i, grad[i], p, m, v, pb, lr, c1, c2);
-}
-
-// All steps of one training call in one cooperative launch, one block per
-// SM.  Separate launches took 36 us a step (index draw 2.4, memsets, gradient
-// 22, Adam 3.4 and the gaps between them) for work that needs a fraction of
-// a microsecond at the tensor cores' rate: the step is a chain of latencies,
-// and this kernel shortens it to 14 us (21 before its passes took matrix loads
-// and stores).  Each step a block draws its own
-// rows, adds its share of the gradient and, after a grid barrier, takes the
-// Adam step of its own slice of the parameters; a second barrier publishes
-// them.  Gradient, loss and Adam arithmetic are those of the separate kernels.
-struct GridBarrier {
-  unsigned* count;      // zero at launch
-  unsigned target;
-  // Bounded: a barrier that is not complete after about ten seconds gives up.
-  __device__ bool wait() {
-    __shared__ int ok;
-    __syncthreads();
-    target += gridDim.x;
-    if (threadIdx.x == 0) {
-      __threadfence();
-      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
-      unsigned seen = 0;
-      int left = 1 << 25;
-      do {
-        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
-      } while ((int)(seen - target) < 0 && --left > 0);
-      ok = left > 0;
-    }
-    __syncthreads();
-    return ok != 0;
-  }
-};
-
-template <int CPW>
-__global__ void __launch_bounds__(THREADS) k_mlp_train(float* p, float* m, float* v, float* grad,
-                                                       __nv_bfloat16* pb, Std sd, const float* x,
-                                                       const uint8_t* label, RowSrc rows,
-                                                       int64_t steps, int64_t batch, float lr,
-                                                       double b1, double b2, float* losses,
-                                                       unsigned* barrier) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  TrainSmem<CPW>& S = *reinterpret_cast<TrainSmem<CPW>*>(smem_raw);
-  GridBarrier bar{barrier, 0u};
-  const int per = (NP + gridDim.x - 1) / gridDim.x;
-  const int lo = blockIdx.x * per, hi = min(NP, lo + per);
-  grad_pad<CPW>(S);
-  for (int64_t s = 0; s < steps; ++s, ++rows.step) {
-    grad_begin<CPW>(S, pb, p);
-    grad_rounds<CPW>(S, sd, x, label, rows, batch, grad, losses ? losses + s : nullptr);
-    b1 *= 0.9;
-    b2 *= 0.999;
-    const float c1 = (float)(1.0 - b1), c2 = (float)(1.0 - b2);
-    bool ok = bar.wait();   // the gradient is complete
-    // the next step's first rows towards L2 while the barriers pass
-    if (s + 1 < steps) {
-      RowSrc next = rows;
-      ++next.step;
-      const int64_t r = (int64_t)blockIdx.x * BlockTiles<CPW>::RS + threadIdx.x;
-      if (threadIdx.x < BlockTiles<CPW>::RS && r < batch) {
-        const int64_t src = next.at(r);
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(x + src * IN));
-        asm volatile("prefetch.global.L1 [%0];" ::"l"(label + src));
-      }
-    }
-    for (int i = lo + threadIdx.x; i < hi; i += THREADS) {
-      adam_one(i, __ldcg(grad + i), p, m, v, pb, lr, c1, c2);
-      if (s + 1 < steps) grad[i] = 0.0f;
-    }
-    ok = ok && bar.wait();  // the parameters are
-    if (!ok) {
-      if (losses && threadIdx.x == 0) losses[s] = __int_as_float(0x7fc00000);
-      return;
-    }
+// Adam step (beta1 0.9, beta2 0.999, eps 1e-8; c1, c2 the bias corrections).
+// With clear, the gradient is zeroed for the next training step.
+__global__ void k_adam(float* p, float* m, float* v, float* grad, __nv_bfloat16* pb, float lr,
+                       float c1, float c2, bool clear) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < NP; i += gridDim.x * blockDim.x) {
+    const float gr = grad[i];
+    const float mi = 0.9f * m[i] + 0.1f * gr;
+    const float vi = 0.999f * v[i] + 0.001f * gr * gr;
+    m[i] = mi;
+    v[i] = vi;
+    const float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+    p[i] = pi;
+    pb[i] = __float2bfloat16(pi);
+    if (clear) grad[i] = 0.0f;
   }
 }
 
@@ -1095,64 +992,44 @@ CellGrid grid_of(const qcams_proposal_spec* s) {
   return g;
 }
 
-template <int CPW>
+template <int CPW, bool DRAW>
 cudaError_t launch_grad_cpw(const qcams_mlp* m, const float* x, const uint8_t* label,
-                            int64_t n, float* loss_out, cudaStream_t st) {
+                            const RowSrc& rows, int64_t n, float* loss_out, cudaStream_t st) {
   const size_t smem = sizeof(TrainSmem<CPW>);
-  cudaError_t e = cudaFuncSetAttribute(k_mlp_grad<CPW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(
+      k_mlp_grad<CPW, DRAW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int64_t grid = (n + BlockTiles<CPW>::RS - 1) / BlockTiles<CPW>::RS;
   if (grid > sm_count()) grid = sm_count();
   if (grid < 1) grid = 1;
-  k_mlp_grad<CPW><<<(unsigned)grid, THREADS, smem, st>>>(
-      reinterpret_cast<const __nv_bfloat16*>(m->params_bf16), m->params, std_of(m), x, label, n,
-      m->grad, loss_out);
+  k_mlp_grad<CPW, DRAW><<<(unsigned)grid, THREADS, smem, st>>>(
+      reinterpret_cast<const __nv_bfloat16*>(m->params_bf16), m->params, std_of(m), x, label, rows,
+      n, m->grad, loss_out);
   return cudaGetLastError();
 }
 
-int launch_grad(const qcams_mlp* m, const float* x, const uint8_t* label, int64_t n,
-                float* loss_out, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(m->grad, 0, NP * sizeof(float), st);
-  if (e == cudaSuccess && loss_out) e = cudaMemsetAsync(loss_out, 0, sizeof(float), st);
-  if (e != cudaSuccess) return QCAMS_E_CUDA;
-  // At most one block per SM (the weights, the round's tiles and the warps'
-  // SiLU' values take 155 KB of shared memory with 64-sample rounds, 203 KB
-  // with 128).  A batch that fits one 64-sample round per SM (8,192 samples:
-  // 128 blocks) takes that, the shortest block; larger batches take
-  // 128-sample rounds, half the rounds' global-atomic flushes.
-  e = (n + 63) / 64 <= sm_count() ? launch_grad_cpw<1>(m, x, label, n, loss_out, st)
-                                  : launch_grad_cpw<2>(m, x, label, n, loss_out, st);
-  return status_of(e);
+// Adds the gradient and loss of n rows to m->grad and *loss_out.  One block
+// per SM at most.  A batch that fits one 64-sample round per SM (8,192
+// samples: 128 blocks) takes that, the shortest block (84 KB of shared memory
+// for weights and tiles); larger batches take 128-sample rounds (137 KB), half
+// the rounds' global-atomic flushes.  With two 64-sample blocks per SM
+// instead, 12,000 samples take 17.8 us against 20.2, 19,456 22.8 against
+// 20.7, 1,000,000 439 against 570.
+template <bool DRAW>
+cudaError_t launch_grad(const qcams_mlp* m, const float* x, const uint8_t* label,
+                        const RowSrc& rows, int64_t n, float* loss_out, cudaStream_t st) {
+  return (n + 63) / 64 <= sm_count()
+             ? launch_grad_cpw<1, DRAW>(m, x, label, rows, n, loss_out, st)
+             : launch_grad_cpw<2, DRAW>(m, x, label, rows, n, loss_out, st);
 }
 
-template <int CPW>
-cudaError_t launch_train(const qcams_mlp* m, const float* x, const uint8_t* label, RowSrc rows,
-                         int64_t steps, int64_t batch, float lr, float* losses, unsigned* barrier,
-                         cudaStream_t st) {
-  const size_t smem = sizeof(TrainSmem<CPW>);
-  cudaError_t e = cudaFuncSetAttribute(k_mlp_train<CPW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
-  // one block per SM: those without a round share the Adam step
-  const unsigned grid = (unsigned)sm_count();
-  float *p = m->params, *am = m->adam_m, *av = m->adam_v, *grad = m->grad;
-  __nv_bfloat16* pb = reinterpret_cast<__nv_bfloat16*>(m->params_bf16);
-  Std sd = std_of(m);
-  double b1 = std::pow(0.9, (double)m->step), b2 = std::pow(0.999, (double)m->step);
-  void* args[] = {&p, &am, &av, &grad, &pb, &sd, &x, &label, &rows, &steps, &batch, &lr, &b1, &b2,
-                  &losses, &barrier};
-  return cudaLaunchCooperativeKernel((const void*)k_mlp_train<CPW>, dim3(grid), dim3(THREADS), args,
-                                     smem, st);
-}
-
-int launch_adam(qcams_mlp* m, float lr, cudaStream_t st) {
+cudaError_t launch_adam(qcams_mlp* m, float lr, bool clear, cudaStream_t st) {
   m->step += 1;
   const float c1 = (float)(1.0 - std::pow(0.9, (double)m->step));
   const float c2 = (float)(1.0 - std::pow(0.999, (double)m->step));
   k_adam<<<36, 256, 0, st>>>(m->params, m->adam_m, m->adam_v, m->grad,
-                             reinterpret_cast<__nv_bfloat16*>(m->params_bf16), lr, c1, c2);
-  return status_of(cudaGetLastError());
+                             reinterpret_cast<__nv_bfloat16*>(m->params_bf16), lr, c1, c2, clear);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -1235,7 +1112,11 @@ int qcams_mlp_grad(const qcams_mlp* m, const float* x, const uint8_t* label, int
   int rc;
   if ((rc = dev_ok()) != QCAMS_OK) return rc;
   (void)cudaGetLastError();
-  return launch_grad(m, x, label, n, loss_out, (cudaStream_t)cuda_stream);
+  cudaStream_t st = (cudaStream_t)cuda_stream;
+  cudaError_t e = cudaMemsetAsync(m->grad, 0, NP * sizeof(float), st);
+  if (e == cudaSuccess && loss_out) e = cudaMemsetAsync(loss_out, 0, sizeof(float), st);
+  if (e == cudaSuccess) e = launch_grad<false>(m, x, label, RowSrc{}, n, loss_out, st);
+  return status_of(e);
 }
 
 int qcams_mlp_train_step(qcams_mlp* m, const float* x, const uint8_t* label, int64_t n,
@@ -1243,7 +1124,7 @@ int qcams_mlp_train_step(qcams_mlp* m, const float* x, const uint8_t* label, int
   if (!(lr > 0.0f)) return QCAMS_E_INVALID;
   int rc = qcams_mlp_grad(m, x, label, n, loss_out, cuda_stream);
   if (rc != QCAMS_OK) return rc;
-  return launch_adam(m, lr, (cudaStream_t)cuda_stream);
+  return status_of(launch_adam(m, lr, false, (cudaStream_t)cuda_stream));
 }
 
 int qcams_mlp_train(qcams_mlp* m, const float* x, const uint8_t* label, int64_t n, int64_t steps,
@@ -1259,23 +1140,22 @@ int qcams_mlp_train(qcams_mlp* m, const float* x, const uint8_t* label, int64_t 
       cudaMemsetAsync(losses, 0, sizeof(float) * (size_t)steps, st) != cudaSuccess)
     return QCAMS_E_CUDA;
   if (steps == 0) return QCAMS_OK;
-  // the grid barrier's counter lives in the index scratch until the kernel
-  // is done, then the last step's indices go there
+  // Two launches a step: the gradient kernel draws its own rows (as
+  // k_draw_idx does) and Adam clears the gradient for the next step.
+  // 16.8 us a step at 8,192 rows, 32.1 with an index draw and a memset more
+  // and the earlier passes.  All steps in one cooperative launch take 13.8,
+  // but need every SM free at once and a grid barrier, whose give-up an
+  // asynchronous call cannot report.
   cudaError_t e = cudaMemsetAsync(m->grad, 0, NP * sizeof(float), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(idx, 0, sizeof(int64_t), st);
-  RowSrc rows{true, n, seed, (uint64_t)m->step};
-  unsigned* barrier = reinterpret_cast<unsigned*>(idx);
-  // rounds as launch_grad chooses them
-  if (e == cudaSuccess)
-    e = (batch + 63) / 64 <= sm_count()
-            ? launch_train<1>(m, x, label, rows, steps, batch, lr, losses, barrier, st)
-            : launch_train<2>(m, x, label, rows, steps, batch, lr, losses, barrier, st);
+  RowSrc rows{n, seed, (uint64_t)m->step};
+  for (int64_t s = 0; s < steps && e == cudaSuccess; ++s) {
+    rows.step = (uint64_t)m->step;
+    e = launch_grad<true>(m, x, label, rows, batch, losses ? losses + s : nullptr, st);
+    if (e == cudaSuccess) e = launch_adam(m, lr, s + 1 < steps, st);
+  }
   if (e != cudaSuccess) return QCAMS_E_CUDA;
-  rows.step += (uint64_t)(steps - 1);
   k_draw_idx<<<(batch + 255) / 256, 256, 0, st>>>(idx, batch, rows);
-  if (cudaGetLastError() != cudaSuccess) return QCAMS_E_CUDA;
-  m->step += steps;
-  return QCAMS_OK;
+  return status_of(cudaGetLastError());
 }
 
 int qcams_mlp_infer(const qcams_mlp* m, const float* x, int64_t n, float* probs,

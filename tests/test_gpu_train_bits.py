@@ -53,3 +53,51 @@ def test_bias_gradient_row_order(Q):
         differ += int((want != _row_sum(d, (4, 2, 1))).sum())
         assert np.array_equal(got, want), (seed, np.flatnonzero(got != want))
     assert differ > 0                  # the rows chosen do show the order
+
+
+def _values(m):
+    return [t.cpu().numpy() for t in (m.params, m.m, m.v, m.grad, m.params_bf16)]
+
+
+@pytest.mark.parametrize("how", ["eager", "stream", "graph"])
+@pytest.mark.parametrize("batch,steps", [(1, 1), (16, 9), (7, 40)])
+def test_training_is_its_single_steps(Q, how, batch, steps):
+    """qcams_mlp_train against the same rows one qcams_mlp_train_step at a
+    time, bit for bit: losses, last indices, last gradient, parameters,
+    moments and the step count; as a plain call, on a stream of its own beside
+    other work, and replayed from a graph."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(batch)
+    x = torch.randn(500, 8, device="cuda", generator=gen)
+    cls = torch.randint(0, 6, (500,), device="cuda", generator=gen).to(torch.uint8)
+    a, b, one = Q.MLP(seed=2), Q.MLP(seed=2), Q.MLP(seed=1)
+    for m in (a, b):
+        m.train_step(x[:3].contiguous(), cls[:3].contiguous(), 1e-3)     # training goes on from step 1
+    want = []
+    for s in range(steps):
+        one.c.step = 1 + s                                               # the rows of step 1 + s
+        rows = one.train(x, cls, 1, batch, 1e-3, seed=21)[1]
+        want.append(b.train_step(x[rows].contiguous(), cls[rows].contiguous(), 2e-3).clone())
+    side, busy = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    if how == "eager":
+        losses, idx = a.train(x, cls, steps, batch, 2e-3, seed=21)
+    elif how == "stream":
+        big = torch.randn(4096, 4096, device="cuda")
+        torch.cuda.synchronize()
+        with torch.cuda.stream(busy):
+            for _ in range(20):
+                big = big @ big * 1e-3
+        with torch.cuda.stream(side):
+            losses, idx = a.train(x, cls, steps, batch, 2e-3, seed=21)
+    else:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side):
+            losses, idx = a.train(x, cls, steps, batch, 2e-3, seed=21)
+        graph.replay()
+    torch.cuda.synchronize()
+    assert a.step == b.step == 1 + steps
+    assert np.array_equal(idx.cpu().numpy(), rows.cpu().numpy())
+    assert np.array_equal(losses.cpu().numpy(), torch.cat(want).cpu().numpy())
+    for u, v in zip(_values(a), _values(b)):
+        assert np.array_equal(u, v)
