@@ -825,6 +825,16 @@ struct SlotRec {
   unsigned long long gb[3 * 64], w[8], w2[8];
 };
 
+// 64-bit add in shared memory as two 32-bit ones, the carry from the first's
+// old value.  A 64-bit shared atomic is a compare-and-swap loop, which the few
+// words of the weight sums serialise: 2 M weighted lanes of sorted cells took
+// 105 us with it, 38 this way.
+__device__ __forceinline__ void shared_add64(unsigned long long* p, unsigned long long x) {
+  unsigned* q = reinterpret_cast<unsigned*>(p);   // low word first
+  const unsigned lo = (unsigned)x, old = atomicAdd(q, lo);
+  atomicAdd(q + 1, (unsigned)(x >> 32) + (old + lo < old ? 1u : 0u));
+}
+
 template <bool WEIGHTED>
 __global__ void __launch_bounds__(kReduceBlock) k_reduce(DevBatch B, int n_cells,
                                                          unsigned long long* hist) {
@@ -857,8 +867,8 @@ __global__ void __launch_bounds__(kReduceBlock) k_reduce(DevBatch B, int n_cells
     if (WEIGHTED) {
       const double wv = B.isw[i];
       if (slot >= 0) {
-        atomicAdd(&sh[slot].w[k], fixp(wv));
-        atomicAdd(&sh[slot].w2[k], fixp(wv * wv));
+        shared_add64(&sh[slot].w[k], fixp(wv));
+        shared_add64(&sh[slot].w2[k], fixp(wv * wv));
       } else {
         atomicAdd(&H[QCAMS_H_W + k], fixp(wv));
         atomicAdd(&H[QCAMS_H_W2 + k], fixp(wv * wv));
@@ -870,7 +880,7 @@ __global__ void __launch_bounds__(kReduceBlock) k_reduce(DevBatch B, int n_cells
     } else if (slot >= 0) {
       atomicAdd(&sh[slot].vt[64 * k + v], 1u);
       atomicAdd(&sh[slot].jt[256 * k + jj], 1u);
-      atomicAdd(&sh[slot].gb[64 * k + v], fixp(B.gbw[i]));
+      shared_add64(&sh[slot].gb[64 * k + v], fixp(B.gbw[i]));
     } else {
       atomicAdd(&H[QCAMS_H_VT + 64 * k + v], 1ull);
       atomicAdd(&H[QCAMS_H_JT + 256 * k + jj], 1ull);
