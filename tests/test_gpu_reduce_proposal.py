@@ -53,6 +53,49 @@ def test_reduce_matches_counts(Q, n, n_cells, weighted, sort):
     assert np.array_equal(cells, host, equal_nan=True)
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [0, 1, 513, 1024, 1025, 131_072, 131_073])
+@pytest.mark.parametrize("n_cells,weighted", [(1, False), (2, True), (9, False), (9, True)])
+def test_histograms_without_cross_sections(Q, n, n_cells, weighted):
+    """A call of up to 1,024 lanes that wants no cross sections adds every entry
+    in one launch, one of up to 131,072 gives a block 512 lanes: the records
+    are those of the lanes taken in halves with cross sections, added up."""
+    import torch
+    weighted = weighted and n > 0        # without lanes there is no weight array to pass
+    rng = np.random.default_rng(n)
+    cell = rng.integers(-1, n_cells + 1, n).astype(np.int32)
+    b = Q.Batch.empty(n, "cuda", cell=cell, isw=rng.uniform(0, 3000, n) if weighted else None)
+    for dst, lo, hi in ((b.cls, 0, 8), (b.vt, -3, 90), (b.jt, -3, 400)):
+        dst.copy_(torch.as_tensor(rng.integers(lo, hi, n)))
+    b.f64["gbw"].copy_(torch.as_tensor(rng.uniform(0, 9, n)))
+    one = np.ones(n_cells)
+    got, _, _ = Q.reduce_xsec(b, n_cells, weighted=weighted, finalize=False)
+    want = torch.zeros_like(got)
+    for lo, hi in ((0, n // 2), (n // 2, n)):
+        h = Q.Batch.empty(hi - lo, "cuda", cell=cell[lo:hi],
+                          isw=b.isw[lo:hi].cpu().numpy() if weighted else None)
+        for k in ("cls", "vt", "jt"):
+            getattr(h, k).copy_(getattr(b, k)[lo:hi])
+        h.f64["gbw"].copy_(b.f64["gbw"][lo:hi])
+        want += Q.reduce_xsec(h, n_cells, one, one, 0 * one, 1, weighted=weighted and hi > lo)[0]
+    assert torch.equal(got, want)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,most", [(1, 6.0), (2000, 14.0)])
+def test_small_reductions_take_few_passes(Q, n, most):
+    """Time of small calls without cross sections, in microseconds: a memset and
+    one kernel for one lane (two kernels take 1.2 us more), and for 2,000 lanes
+    about ten atomics one after the other at 0.7 us and two launches."""
+    cell = np.arange(n) % 5
+    b = Q.Batch.empty(n, "cuda", cell=cell, isw=np.ones(n))
+    import torch
+    hist = torch.empty(5 * Q.H_STRIDE, dtype=torch.int64, device="cuda")
+    us = _graph_us(lambda: Q.reduce_xsec(b, 5, hist_out=hist, finalize=False))
+    print(f"\nreduce of {n} lanes: {us:.2f} us")
+    assert us < most
+
+
 def _graph_us(f, reps=20):
     """Device time of one call, from a graph of `reps`."""
     import torch
