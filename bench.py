@@ -64,7 +64,7 @@ KERNEL_SOURCES = {
 }
 COUNTS_SOURCE_SHA256 = {
     64: "11739afbfbcc33e4bae9fe47ce58383f551317ddf4ff075736ec254c1577b4fe",
-    32: "1f1f476a60b80403d10ad407c867c5c3107bf21770a4aefbbd1addb6c36f9731",
+    32: "4a133bb64ef2a1dd7b05426b98f303eee879916774013995d569b5d017d7d1ff",
 }
 # DRAM bytes per trajectory of the integrator: ncu dram__bytes_read.sum +
 # dram__bytes_write.sum of the same FP64 profile case (1,110,784 B read,

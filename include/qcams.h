@@ -143,10 +143,11 @@ typedef struct {
   int32_t persistent;  /* 0 and 1: FP64 adaptive runs choose the launch by the
                           batch (one thread per trajectory with a refill
                           queue, or three and six lanes per trajectory; the
-                          results are the same bits on every path); FP32: 1 =
-                          persistent refill-queue launch (finished lanes take
-                          the next trajectory from a device counter), 0 = one
-                          thread per trajectory;
+                          results are the same bits on every path); FP32: 0 =
+                          one thread per trajectory, 1 = for batches several
+                          times what the GPU holds a persistent refill-queue
+                          launch (finished lanes take the next trajectory
+                          from a device counter), the same bits;
                           2 = three lanes per trajectory, 3 = six lanes
                           per trajectory, from start to end (FP64 adaptive
                           steps only, else QCAMS_E_INVALID; block and

@@ -552,18 +552,16 @@ __global__ void __launch_bounds__(128) k_integrate32_plain(SysSetF sys, const De
   flush(rhs, steps, counters);
 }
 
-// MINB resident blocks per SM cap the registers: the all-Morse kernel takes
+// The resident blocks per SM cap the registers: the all-Morse kernel takes
 // 121, four blocks of 128 threads (five, at 96 registers, spill and run the
-// sweep in 115.8 ms against 110.7); the generic one 120 or, with five blocks
-// and 100 bytes of spills, 96: 35.8 against 37.9 ms for 1 M lanes, but 8.4
-// against 8.3 ms for 9,999, which four blocks per SM hold at once and whose
-// longest lanes set the time.
-template <bool MORSE, bool ONE, int MINB>
-__global__ void __launch_bounds__(128, MINB) k_integrate32_persistent(SysSetF sys,
-                                                                const DevShape* shapes,
-                                                                IntegParams ip, DevBatch B,
-                                                                unsigned long long* counters,
-                                                                const long long* list) {
+// sweep in 115.8 ms against 110.7; with several systems the four-block cap
+// costs 32 bytes of spills: 1 M lanes of two systems 38.4 ms, of one 36.6);
+// the generic one 120 or, with five blocks and 100 bytes of spills, 96: 35.8
+// against 37.9 ms for 1 M lanes.
+template <bool MORSE, bool ONE>
+__global__ void __launch_bounds__(128, MORSE ? 4 : 5)
+    k_integrate32_persistent(SysSetF sys, const DevShape* shapes, IntegParams ip, DevBatch B,
+                             unsigned long long* counters, const long long* list) {
   const unsigned lane = threadIdx.x & 31u;
   unsigned long long rhs = 0, steps = 0;
   Lane32 L;
@@ -649,7 +647,7 @@ SysSetF to_float(const SysSet& in) {
   return o;
 }
 
-template <bool MORSE, bool ONE, int MINB>
+template <bool MORSE, bool ONE>
 cudaError_t launch32_persistent(const SysSetF& sf, const DevShape* shapes, const IntegParams& ip,
                                 const DevBatch& b, Ctx& ctx, cudaStream_t st) {
   const int block = 128;
@@ -657,12 +655,11 @@ cudaError_t launch32_persistent(const SysSetF& sf, const DevShape* shapes, const
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &per_sm, k_integrate32_persistent<MORSE, ONE, MINB>, block, 0);
+      &per_sm, k_integrate32_persistent<MORSE, ONE>, block, 0);
   if (e != cudaSuccess) return e;
   const long long* list = nullptr;
-  // More lanes than are resident at once: the slowest collisions first
-  // (figures at launch_queue_order).
-  if (b.n > 4 * 128 * (int64_t)ctx.sm_count && b.n >= kOrderMinLanes && lists_usable(b)) {
+  // the slowest collisions first (figures at launch_queue_order)
+  if (b.n >= kOrderMinLanes && lists_usable(b)) {
     long long* order = reinterpret_cast<long long*>(b.vprime);
     e = launch_queue_order(b, order, reinterpret_cast<unsigned*>(b.jprime), ctx.counters + 3, st);
     if (e != cudaSuccess) return e;
@@ -672,18 +669,27 @@ cudaError_t launch32_persistent(const SysSetF& sf, const DevShape* shapes, const
   const long long need_blocks = (b.n + block - 1) / block;
   if (grid > need_blocks) grid = need_blocks;
   if (grid < 1) grid = 1;
-  k_integrate32_persistent<MORSE, ONE, MINB><<<(unsigned)grid, block, 0, st>>>(sf, shapes, ip, b,
-                                                                              ctx.counters, list);
+  k_integrate32_persistent<MORSE, ONE><<<(unsigned)grid, block, 0, st>>>(sf, shapes, ip, b,
+                                                                        ctx.counters, list);
   return cudaGetLastError();
 }
 
 template <bool MORSE, bool ONE>
 cudaError_t launch32(const SysSetF& sf, const DevShape* shapes, const IntegParams& ip,
                      const DevBatch& b, int persistent, Ctx& ctx, cudaStream_t st) {
-  if (persistent)
-    return !MORSE && b.n > 4 * 128 * (int64_t)ctx.sm_count
-               ? launch32_persistent<MORSE, ONE, MORSE ? 4 : 5>(sf, shapes, ip, b, ctx, st)
-               : launch32_persistent<MORSE, ONE, 4>(sf, shapes, ip, b, ctx, st);
+  // The queue pays once a batch is several times what the GPU holds (384 to
+  // 640 lanes per SM): below, there is little to refill, its attempts are
+  // slower than those of one thread per lane, and its slowest lanes, taken
+  // first, share warps and SMs.  Milliseconds, queue / one thread each:
+  //   sweep, all energies       60,000 16.2 / 9.2, 125,000 21.0 / 12.9,
+  //                             260,000 22.0 / 20.1, 300,000 21.3 / 22.4
+  //   three generic systems     125,000 20.2 / 16.3, 260,000 25.2 / 22.7,
+  //                             300,000 22.9 / 23.9
+  //   LJ(12,6), one system      100,000 13.3 / 12.1, 125,000 12.8 / 13.6,
+  //                             150,000 13.6 / 13.0, 175,000 12.7 / 14.3
+  constexpr int64_t queue_per_sm = !MORSE && ONE ? 1024 : 1792;
+  if (persistent && b.n > queue_per_sm * ctx.sm_count)
+    return launch32_persistent<MORSE, ONE>(sf, shapes, ip, b, ctx, st);
   const unsigned grid = (unsigned)((b.n + 127) / 128);
   k_integrate32_plain<MORSE, ONE><<<grid, 128, 0, st>>>(sf, shapes, ip, b, ctx.counters);
   return cudaGetLastError();
