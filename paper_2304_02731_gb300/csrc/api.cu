@@ -449,6 +449,13 @@ struct LevelSmem {
   int more;
 };
 
+// The warps of a level's block meet at different places of the code (the
+// first one in its iteration, the others in their loop), which __syncthreads
+// does not allow for: a barrier of its own with the number of threads.
+__device__ __forceinline__ void level_barrier() {
+  asm volatile("barrier.sync 1, %0;" ::"n"(kLevelBlock) : "memory");
+}
+
 // V and V' of a pair in one evaluation (Morse without the cancellation of
 // De (1 - x)^2 - De at large r, where high levels have their outer ends).
 __device__ __forceinline__ void pot_VdV(const DevPair& q, double r, double* V, double* dV) {
@@ -508,9 +515,9 @@ __device__ __forceinline__ void level_integrals(const DevPair& q, double a, doub
     S.d = d;
     S.more = 1;
   }
-  __syncthreads();
+  level_barrier();
   level_points(q, a, S);
-  __syncthreads();
+  level_barrier();
   const int k = threadIdx.x & 1;
   const double s = (S.sum[0][k] + S.sum[1][k]) + (S.sum[2][k] + S.sum[3][k]);
   *act = 0.5 * kPi * d * __shfl_sync(0xffffffffu, s, 0);
@@ -607,10 +614,10 @@ __device__ qcams_level solve_level_block(const DevPair& q, const DevShape& sh, d
   const double a = L2 / (2.0 * mu);
   if (threadIdx.x >= 32) {
     for (;;) {
-      __syncthreads();
+      level_barrier();
       if (!S.more) return L;
       level_points(q, a, S);
-      __syncthreads();
+      level_barrier();
     }
   }
   double r_min, r_top, Etop, out, act, per;
@@ -655,7 +662,7 @@ __device__ qcams_level solve_level_block(const DevPair& q, const DevShape& sh, d
     }
   }
   if (threadIdx.x == 0) S.more = 0;
-  __syncthreads();
+  level_barrier();
   return L;
 }
 
