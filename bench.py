@@ -63,7 +63,7 @@ KERNEL_SOURCES = {
     32: ["integrate32.cu", "dp5_tableau.cuh"],
 }
 COUNTS_SOURCE_SHA256 = {
-    64: "11739afbfbcc33e4bae9fe47ce58383f551317ddf4ff075736ec254c1577b4fe",
+    64: "d6c334d67295a982fd79ac4c0465ee863138bb82b05456a9e6299ea919624425",
     32: "4a133bb64ef2a1dd7b05426b98f303eee879916774013995d569b5d017d7d1ff",
 }
 # DRAM bytes per trajectory of the integrator: ncu dram__bytes_read.sum +

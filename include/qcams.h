@@ -391,21 +391,27 @@ int qcams_run_batch_noalloc(const qcams_system* sys, int32_t n_sys, const qcams_
  * status READY) representative of the workload, ideally the workload
  * itself when it is small; the integrator runs on it, from the same saved
  * initial state, with at most `max_attempts` step attempts per lane, once
- * for every supported (block, blocks_per_sm) variant of the persistent
- * launch and, when the sample has no more lanes than one warp per SM
- * sub-partition (SM count x 128) or max_attempts is not below
- * integ->max_steps (an uncapped run), once for each lane-group launch
- * (persistent = 2 and 3, one warp per block); the attempted lane-steps per
- * second are measured with CUDA events.  (A larger capped sample cannot
- * show the lane-group kernels' tails: their warps run until their longest
- * trajectory ends, without refill.)  The sample's state is restored afterwards.  results
+ * for every supported (block, blocks_per_sm) shape and, when the sample has
+ * no more lanes than one warp per SM sub-partition (SM count x 128) or
+ * max_attempts is not below integ->max_steps (an uncapped run), once for each
+ * lane-group launch (persistent = 2 and 3, one warp per block); the attempted
+ * lane-steps per second are measured with CUDA events.  (A larger capped
+ * sample cannot show the lane-group kernels' tails: their warps run until
+ * their longest trajectory ends, without refill.)  With all-Morse systems the
+ * shapes are those of the one-thread kernel, which serves large batches;
+ * other systems' runs have no use for them, and their one mode-1 run is
+ * listed for every shape.  The sample's state is restored afterwards.  results
  * (host, room for QCAMS_TUNE_MAX_VARIANTS entries) receives one entry per
  * launch, *n_results their number, and *best a copy of *integ with the
- * fastest launch (its persistent, block and blocks_per_sm).  Persistent
- * shapes within 2 % of the fastest persistent shape count as a tie, which
- * goes to the smallest block (then the fewest blocks per SM); a lane-group
- * launch is chosen only if it is strictly the fastest.  Synchronous;
- * allocates a temporary copy of the sample state (~121 bytes per lane) with
+ * fastest launch (its persistent, block and blocks_per_sm).  Shapes within
+ * 2 % of the fastest shape count as a tie, which goes to the smallest block
+ * (then the fewest blocks per SM).  A lane-group launch is chosen only if it
+ * is faster than mode 1 on the sample; mode 1 is timed for that as
+ * qcams_run_batch runs it, except on uncapped all-Morse samples of more than
+ * SM count x 128 lanes, where the fastest shape stands for it (the staged run
+ * of such a batch can be the fastest of all: 20,000 plain-study lanes take
+ * 240 ms in mode 1, 271 with three lanes, 281 with six).  Synchronous;
+ * allocates a temporary copy of the sample state (~137 bytes per lane) with
  * cudaMallocAsync.
  */
 #define QCAMS_TUNE_MAX_VARIANTS 16

@@ -354,10 +354,9 @@ __device__ void lane_store(const SysSet& sys, const DevBatch& B, int64_t i, cons
 // irrelevant to a step-size controller); accept / reject is a select, so
 // the warp does not diverge.  The minimum step is checked by exponents: h
 // fails below 8-16 ulp(t).
-template <bool MORSE>
-__device__ __forceinline__ void lane_attempt(const SysSet& sys, const DevShape* shapes,
-                                             const IntegParams& ip, const double* __restrict__ T,
-                                             LaneState& L, const OpReg& op, const double* sB) {
+__device__ __forceinline__ void lane_attempt(const SysSet& sys, const IntegParams& ip,
+                                             const double* __restrict__ T, LaneState& L,
+                                             const OpReg& op, const double* sB) {
   const DevSys& S = sys.s[L.sid];
   {
     const int eh = (__double2hiint(L.h) >> 20) & 0x7ff;
@@ -369,7 +368,7 @@ __device__ __forceinline__ void lane_attempt(const SysSet& sys, const DevShape* 
   }
   double xn[6], vn[6], s2[3];
   float er[6], ev[6];
-  dp_step<MORSE>(S, T, L.rho, L.vel, L.acc, L.h, xn, vn, er, ev, s2, op, sB);
+  dp_step<true>(S, T, L.rho, L.vel, L.acc, L.h, xn, vn, er, ev, s2, op, sB);
   unsigned bad = 0, ignore = 0;
   float sum = 0.f;
   const float rt = ip.rtol_f, at = ip.atol_f;
@@ -414,17 +413,9 @@ __device__ __forceinline__ void lane_attempt(const SysSet& sys, const DevShape* 
   const float radial = fmaf(signed_f(L.rho[3]), signed_f(L.vel[3]),
                             fmaf(signed_f(L.rho[4]), signed_f(L.vel[4]),
                                  signed_f(L.rho[5]) * signed_f(L.vel[5])));
-  bool collapse = false;
-  if (!MORSE) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-      collapse |= S.pair[k].kind == QCAMS_BUCK &&
-                  dbits(s2[k]) < dbits(shapes[L.sid * 3 + k].r_b2);
-  }
   int st = L.status;
   st = (accept && dbits(L.t) >= dbits(L.tmax)) ? QCAMS_LANE_DONE_TMAX : st;
   st = (accept && smax > dbits(ip.r_stop2) && radial > 0.0f) ? QCAMS_LANE_DONE_RSTOP : st;
-  st = (accept && collapse) ? QCAMS_LANE_FAIL_COLLAPSE : st;
   st = (st == QCAMS_LANE_RUNNING && (long long)(L.nacc + L.nrej) >= ip.max_steps)
            ? QCAMS_LANE_FAIL_MAXSTEPS : st;
   L.status = st;
@@ -447,11 +438,10 @@ __device__ __forceinline__ void flush_counters(unsigned long long rhs, unsigned 
 // of its idle lanes with one atomicAdd (ballot + popc + shuffle).  With
 // q.keep > 0 the lanes that are left when the queue is empty are handed on
 // (StageQueue).
-template <bool MORSE, int BLOCK, int MINB>
-__global__ void __launch_bounds__(BLOCK, MINB) k_integrate_persistent(SysSet sys, const DevShape* shapes,
-                                                              IntegParams ip, DevBatch B,
-                                                              unsigned long long* counters,
-                                                              StageQueue q) {
+template <int BLOCK, int MINB>
+__global__ void __launch_bounds__(BLOCK, MINB)
+    k_integrate_persistent(SysSet sys, IntegParams ip, DevBatch B, unsigned long long* counters,
+                           StageQueue q) {
   __shared__ double sT[kExpTableSize], sK[kOpRegs], sB[8];
   op_reg_fill(sK);
   if (threadIdx.x < 8) sB[threadIdx.x] = kT.b[threadIdx.x];
@@ -478,7 +468,7 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_integrate_persistent(SysSet sys
           exhausted = true;
         } else {
           idx = q.list_in ? q.list_in[k] : k;
-          have = lane_load<MORSE>(sys, ip, sT, B, idx, L, rhs, op);
+          have = lane_load<true>(sys, ip, sT, B, idx, L, rhs, op);
           skip = !have;
         }
       }
@@ -494,19 +484,19 @@ __global__ void __launch_bounds__(BLOCK, MINB) k_integrate_persistent(SysSet sys
       if (have) {
         rhs += 6ull * L.calls;
         steps += L.calls;
-        lane_store<MORSE>(sys, B, idx, L, true);
+        lane_store<true>(sys, B, idx, L, true);
         q.list_out[at + __popc(pass & ((1u << lane) - 1u))] = idx;
       }
       break;
     }
-    if (have) lane_attempt<MORSE>(sys, shapes, ip, sT, L, op, sB);
+    if (have) lane_attempt(sys, ip, sT, L, op, sB);
     const bool done = have && L.status != QCAMS_LANE_RUNNING;
     const unsigned ended = __ballot_sync(FULL, done);
     if (ended) {
       if (done) {
         rhs += 6ull * L.calls;
         steps += L.calls;
-        lane_store<MORSE>(sys, B, idx, L);
+        lane_store<true>(sys, B, idx, L);
         have = false;
       }
       if (lane == 0) atomicAdd(q.retired, (unsigned long long)__popc(ended));
@@ -770,35 +760,32 @@ int find_variant(int block, int minb) {
   return -1;
 }
 
-template <bool MORSE, int BLOCK, int MINB>
-cudaError_t launch_shape(const SysSet& sys, const DevShape* shapes, const IntegParams& ip,
-                         const DevBatch& b, int sm_count, unsigned long long* counters,
-                         const StageQueue& q, cudaStream_t st) {
+template <int BLOCK, int MINB>
+cudaError_t launch_shape(const SysSet& sys, const IntegParams& ip, const DevBatch& b, int sm_count,
+                         unsigned long long* counters, const StageQueue& q, cudaStream_t st) {
   int per_sm = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &per_sm, k_integrate_persistent<MORSE, BLOCK, MINB>, BLOCK, 0);
+      &per_sm, k_integrate_persistent<BLOCK, MINB>, BLOCK, 0);
   if (e != cudaSuccess) return e;
   if (per_sm < 1) per_sm = 1;
   long long grid = (long long)per_sm * sm_count;
   const long long need = (b.n + BLOCK - 1) / BLOCK;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
-  k_integrate_persistent<MORSE, BLOCK, MINB><<<(unsigned)grid, BLOCK, 0, st>>>(
-      sys, shapes, ip, b, counters, q);
+  k_integrate_persistent<BLOCK, MINB><<<(unsigned)grid, BLOCK, 0, st>>>(sys, ip, b, counters, q);
   return cudaGetLastError();
 }
 
-template <bool MORSE>
-cudaError_t launch_variant(int v, const SysSet& sys, const DevShape* shapes,
-                           const IntegParams& ip, const DevBatch& b, int sm_count,
-                           unsigned long long* counters, const StageQueue& q, cudaStream_t st) {
+cudaError_t launch_variant(int v, const SysSet& sys, const IntegParams& ip, const DevBatch& b,
+                           int sm_count, unsigned long long* counters, const StageQueue& q,
+                           cudaStream_t st) {
   switch (v) {
-    case 0: return launch_shape<MORSE, 128, 1>(sys, shapes, ip, b, sm_count, counters, q, st);
-    case 1: return launch_shape<MORSE, 64, 1>(sys, shapes, ip, b, sm_count, counters, q, st);
-    case 2: return launch_shape<MORSE, 128, 3>(sys, shapes, ip, b, sm_count, counters, q, st);
-    case 3: return launch_shape<MORSE, 64, 6>(sys, shapes, ip, b, sm_count, counters, q, st);
-    case 4: return launch_shape<MORSE, 64, 7>(sys, shapes, ip, b, sm_count, counters, q, st);
-    case 5: return launch_shape<MORSE, 256, 1>(sys, shapes, ip, b, sm_count, counters, q, st);
+    case 0: return launch_shape<128, 1>(sys, ip, b, sm_count, counters, q, st);
+    case 1: return launch_shape<64, 1>(sys, ip, b, sm_count, counters, q, st);
+    case 2: return launch_shape<128, 3>(sys, ip, b, sm_count, counters, q, st);
+    case 3: return launch_shape<64, 6>(sys, ip, b, sm_count, counters, q, st);
+    case 4: return launch_shape<64, 7>(sys, ip, b, sm_count, counters, q, st);
+    case 5: return launch_shape<256, 1>(sys, ip, b, sm_count, counters, q, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -824,19 +811,16 @@ cudaError_t launch_ff_dot_check(const double* a, const double* w, int m, double*
   return cudaGetLastError();
 }
 
-cudaError_t launch_integrate_shape(const SysSet& sys, const DevShape* shapes,
-                                   const IntegParams& ip, const DevBatch& b, int block,
-                                   int blocks_per_sm, Ctx& ctx, cudaStream_t st) {
+cudaError_t launch_integrate_shape(const SysSet& sys, const IntegParams& ip, const DevBatch& b,
+                                   int block, int blocks_per_sm, Ctx& ctx, cudaStream_t st) {
   const int v = find_variant(block, blocks_per_sm);
-  if (v < 0) return cudaErrorInvalidValue;
+  if (v < 0 || !all_morse(sys)) return cudaErrorInvalidValue;
   cudaError_t e = cudaMemsetAsync(ctx.counters, 0, kCounters * sizeof(unsigned long long), st);
   if (e != cudaSuccess) return e;
   StageQueue q;
   q.head = ctx.counters + 4;
   q.retired = ctx.counters + 5;
-  return all_morse(sys)
-             ? launch_variant<true>(v, sys, shapes, ip, b, ctx.sm_count, ctx.counters, q, st)
-             : launch_variant<false>(v, sys, shapes, ip, b, ctx.sm_count, ctx.counters, q, st);
+  return launch_variant(v, sys, ip, b, ctx.sm_count, ctx.counters, q, st);
 }
 
 cudaError_t launch_queue_order(const DevBatch& b, long long* list, unsigned* scratch,
@@ -937,7 +921,7 @@ cudaError_t launch_stages(const SysSet& sys, const DevShape* shapes, const Integ
     q.keep = lists ? keep : 0;
     cudaError_t e = cudaSuccess;
     if (g.lanes == 1) {
-      e = launch_variant<MORSE>(variant, sys, shapes, ip, b, ctx.sm_count, ctx.counters, q, st);
+      e = launch_variant(variant, sys, ip, b, ctx.sm_count, ctx.counters, q, st);
     } else {
       if (!started) {
         k_start_step<MORSE>
@@ -995,38 +979,25 @@ bool integrate_shape_supported(int block, int blocks_per_sm) {
   return find_variant(block, blocks_per_sm) >= 0;
 }
 
-cudaError_t integrate_variant_regs(int v, bool morse, int* regs) {
+cudaError_t integrate_variant_info(int v, int* regs, int* blocks_per_sm) {
   cudaFuncAttributes a;
   cudaError_t e = cudaErrorInvalidValue;
-#define QCAMS_REGS(M, B, N) e = cudaFuncGetAttributes(&a, k_integrate_persistent<M, B, N>)
+#define QCAMS_INFO(B, N)                                              \
+  e = cudaFuncGetAttributes(&a, k_integrate_persistent<B, N>);        \
+  if (e == cudaSuccess)                                               \
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(                \
+        blocks_per_sm, k_integrate_persistent<B, N>, B, 0)
   switch (v) {
-    case 0: if (morse) QCAMS_REGS(true, 128, 1); else QCAMS_REGS(false, 128, 1); break;
-    case 1: if (morse) QCAMS_REGS(true, 64, 1); else QCAMS_REGS(false, 64, 1); break;
-    case 2: if (morse) QCAMS_REGS(true, 128, 3); else QCAMS_REGS(false, 128, 3); break;
-    case 3: if (morse) QCAMS_REGS(true, 64, 6); else QCAMS_REGS(false, 64, 6); break;
-    case 4: if (morse) QCAMS_REGS(true, 64, 7); else QCAMS_REGS(false, 64, 7); break;
-    case 5: if (morse) QCAMS_REGS(true, 256, 1); else QCAMS_REGS(false, 256, 1); break;
+    case 0: QCAMS_INFO(128, 1); break;
+    case 1: QCAMS_INFO(64, 1); break;
+    case 2: QCAMS_INFO(128, 3); break;
+    case 3: QCAMS_INFO(64, 6); break;
+    case 4: QCAMS_INFO(64, 7); break;
+    case 5: QCAMS_INFO(256, 1); break;
     default: break;
   }
-#undef QCAMS_REGS
+#undef QCAMS_INFO
   if (e == cudaSuccess) *regs = a.numRegs;
-  return e;
-}
-
-cudaError_t integrate_variant_occupancy(int v, bool morse, int* blocks_per_sm) {
-  cudaError_t e = cudaErrorInvalidValue;
-#define QCAMS_OCC(M, B, N) \
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_integrate_persistent<M, B, N>, B, 0)
-  switch (v) {
-    case 0: if (morse) QCAMS_OCC(true, 128, 1); else QCAMS_OCC(false, 128, 1); break;
-    case 1: if (morse) QCAMS_OCC(true, 64, 1); else QCAMS_OCC(false, 64, 1); break;
-    case 2: if (morse) QCAMS_OCC(true, 128, 3); else QCAMS_OCC(false, 128, 3); break;
-    case 3: if (morse) QCAMS_OCC(true, 64, 6); else QCAMS_OCC(false, 64, 6); break;
-    case 4: if (morse) QCAMS_OCC(true, 64, 7); else QCAMS_OCC(false, 64, 7); break;
-    case 5: if (morse) QCAMS_OCC(true, 256, 1); else QCAMS_OCC(false, 256, 1); break;
-    default: break;
-  }
-#undef QCAMS_OCC
   return e;
 }
 

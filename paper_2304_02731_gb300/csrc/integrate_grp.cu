@@ -825,6 +825,18 @@ cudaError_t grouped_func_info(int lanes, bool all_morse, int* regs, int* blocks_
   return e;
 }
 
+cudaError_t queue_func_info(bool all_morse, int* regs, int* blocks_per_sm) {
+  cudaFuncAttributes a;
+  cudaError_t e = all_morse ? cudaFuncGetAttributes(&a, k_integrate_queue<true, 3>)
+                            : cudaFuncGetAttributes(&a, k_integrate_queue<false, 3>);
+  if (e != cudaSuccess) return e;
+  *regs = a.numRegs;
+  return all_morse ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                         blocks_per_sm, k_integrate_queue<true, 3>, kQueueBlock, 0)
+                   : cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                         blocks_per_sm, k_integrate_queue<false, 3>, kQueueBlock, 0);
+}
+
 cudaError_t launch_integrate_grouped(const SysSet& sys, const DevShape* shapes,
                                      const IntegParams& ip, const DevBatch& b, int lanes,
                                      unsigned long long* counters, cudaStream_t st,

@@ -60,11 +60,10 @@ cudaError_t launch_analyze(const SysSet& ss, const DevShape* shapes, double gb_s
 cudaError_t launch_integrate(const SysSet& sys, const DevShape* shapes, const IntegParams& ip,
                              const DevBatch& b, int precision, int persistent, int block,
                              int blocks_per_sm, Ctx& ctx, cudaStream_t st);
-// The FP64 persistent kernel of one launch shape alone, from first to last
-// lane (the autotuner's measurement).
-cudaError_t launch_integrate_shape(const SysSet& sys, const DevShape* shapes,
-                                   const IntegParams& ip, const DevBatch& b, int block,
-                                   int blocks_per_sm, Ctx& ctx, cudaStream_t st);
+// The one-thread FP64 kernel (all-Morse) of one launch shape alone, from first
+// to last lane (the autotuner's measurement of the shapes).
+cudaError_t launch_integrate_shape(const SysSet& sys, const IntegParams& ip, const DevBatch& b,
+                                   int block, int blocks_per_sm, Ctx& ctx, cudaStream_t st);
 
 // FP64 integrator for small batches, `lanes` = 3 or 6 lanes per trajectory
 // (integrate_grp.cu).
@@ -120,6 +119,8 @@ cudaError_t launch_integrate_queue(const SysSet& sys, const DevShape* shapes,
 
 // Registers per thread and resident blocks per SM of the lane-group kernel.
 cudaError_t grouped_func_info(int lanes, bool all_morse, int* regs, int* blocks_per_sm);
+// The same of the three-lane queue.
+cudaError_t queue_func_info(bool all_morse, int* regs, int* blocks_per_sm);
 
 // FP32 integrator with compensated state updates (integrate32.cu).
 cudaError_t launch_integrate32(const SysSet& sys, const DevShape* shapes, const IntegParams& ip,
@@ -134,8 +135,7 @@ void noalloc_forget_device(int dev);
 int integrate_variant_count();
 void integrate_variant_shape(int v, int* block, int* blocks_per_sm);
 bool integrate_shape_supported(int block, int blocks_per_sm);
-cudaError_t integrate_variant_regs(int v, bool morse, int* regs);
-cudaError_t integrate_variant_occupancy(int v, bool morse, int* blocks_per_sm);
+cudaError_t integrate_variant_info(int v, int* regs, int* blocks_per_sm);
 bool integrate_all_morse(const SysSet& sys);
 
 }  // namespace qcams

@@ -451,9 +451,9 @@ def fma_peak(precision: int = 64, stream=None) -> float:
 
 
 def autotune(systems, sample: Batch, integ: Integ, max_attempts: int = 1500, stream=None):
-    """qcams_autotune: measure every launch (the persistent shapes and the
-    three- and six-lane groups) on an initialised sample batch; returns (best
-    Integ, list of per-launch result dicts)."""
+    """qcams_autotune: measure every launch (the one-thread kernel's shapes and
+    the three- and six-lane groups) on an initialised sample batch; returns
+    (best Integ, list of per-launch result dicts)."""
     arr = systems_array(systems)
     res = (TuneResult * 16)()
     nres = C.c_int32()
