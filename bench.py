@@ -5,8 +5,9 @@ One step = one pass of the whole path over one batch: initial conditions
 trajectory to its stop rule, product analysis, histogram reduction and cross
 sections.  Default workload: the batched H2 + Ca sweep, 16 collision
 energies x 24 impact parameters x 8,192 trajectories = 3,145,728
-trajectories, FP64, in one persistent refill-queue launch.  Inputs (the SoA
-state, ~600 MB) are larger than L2, so no flush is needed between steps.
+trajectories, FP64, launch mode 1 (one thread per trajectory from a refill
+queue, the last trajectories in lane groups).  Inputs (the SoA state, ~600 MB)
+are larger than L2, so no flush is needed between steps.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
@@ -38,16 +39,18 @@ if ROOT not in sys.path:
 # Per-step operation counts of the integrators' Morse kernels, from ncu's
 # sass counters (smsp__sass_thread_inst_executed_op_{dfma,dmul,dadd,ffma,
 # fmul,fadd}_pred_on.sum and smsp__sass_thread_inst_executed.sum, divided by
-# the launch's attempted lane-steps) on the 3,840-lane sweep subset capped
-# at 3,000 attempts (bench.py --lanes 4096 --max-steps 3000 --persistent 0).
-# Each set holds the SHA-256 of the kernel sources it was measured on; the
-# bench recomputes it and marks the roofline's counts stale when the
-# sources have changed since.
+# the launch's attempted lane-steps).  Each set holds the SHA-256 of the
+# kernel sources it was measured on; the bench recomputes it and marks the
+# roofline's counts stale when the sources have changed since.
 #   FP64: 342 multiply-adds, 137 products and 37 sums per step (six
 #   right-hand sides included; products and sums issue as DFMAs too) = 516
-#   FP64-pipe instructions of the one-thread kernel, 858 FLOP.  The
-#   DFMA-chain peak runs one DFMA per pipe slot, so pipe_frac below is the
-#   fraction of the FP64 pipe's instruction rate the kernel uses.
+#   FP64-pipe instructions of the one-thread kernel, 858 FLOP.  Checked on the
+#   first k_integrate_persistent launch of "bench.py --lanes 98304 --max-steps
+#   100", where the autotuner runs that kernel alone: 5.149e9 over 9,830,400
+#   lane-steps = 523.7, the 516 and a hundredth of each lane's starting step.
+#   The DFMA-chain peak runs one DFMA per pipe slot, so pipe_frac below is the
+#   fraction of the FP64 pipe's instruction rate the kernel uses; it is
+#   reported for runs whose first stage is the one-thread kernel.
 FP64_FLOP_PER_STEP = 858
 FP64_INSTR_PER_STEP = 516
 #   FP32: 393 multiply-adds, 178 products and 39 sums = 1,004 FLOP and one
@@ -58,38 +61,38 @@ FP64_INSTR_PER_STEP = 516
 FP32_FLOP_PER_STEP = 1004
 FP32_THREAD_INSTR_PER_STEP = 628
 KERNEL_SOURCES = {
-    64: ["integrate.cu", "elem64.cuh", "ff.cuh", "texp.cuh", "exp2_table.inc",
+    64: ["integrate.cu", "integrate_grp.cu", "elem64.cuh", "ff.cuh", "texp.cuh", "exp2_table.inc",
          "dp5_tableau.cuh", "step_ctrl.cuh", "pair_force.cuh", "regop.cuh"],
     32: ["integrate32.cu", "dp5_tableau.cuh"],
 }
 COUNTS_SOURCE_SHA256 = {
-    64: "d6c334d67295a982fd79ac4c0465ee863138bb82b05456a9e6299ea919624425",
-    32: "4a133bb64ef2a1dd7b05426b98f303eee879916774013995d569b5d017d7d1ff",
+    64: "59f5303cd5ecce0b674d6e6f417074e69aa932133a9bb00a6fc440d22a0c3c6b",
+    32: "e32052676aff67b078d3851bfe3de6baef8de151f02049e17bc7508e86a8d9f1",
 }
-# DRAM bytes per trajectory of the integrator: ncu dram__bytes_read.sum +
-# dram__bytes_write.sum of the same FP64 profile case (1,110,784 B read,
-# nothing written back during the launch, for 3,840 lanes), per lane: the
-# state is loaded once, everything else is in registers; the 16 KB
-# exponential table is read from DRAM once and served from L2 to the other
-# blocks.  The figure also holds the fetch of the kernel's code, a fixed
-# cost per launch.
-DRAM_BYTES_PER_LANE = 1110784 / 3840
-# The same for the FP32 kernel (559,360 B read, no table): its state is
-# loaded as (value, compensation) pairs from the same FP64 arrays.
-DRAM_BYTES_PER_LANE_FP32 = 559360 / 3840
+# DRAM bytes per trajectory of an integrator run: ncu dram__bytes_read.sum +
+# dram__bytes_write.sum over all its kernels on 1,572,864 sweep lanes capped
+# at 40 attempts (200 MB of state; bench.py --lanes 1572864 --max-steps 40
+# --tune 0): the queue order 12.6 MB, the one-thread kernel 226.0 read and
+# 129.7 written, the lane-group stages 7.8.  The state is loaded and stored
+# once, everything else is in registers; part of the stores stays in L2.
+DRAM_BYTES_PER_LANE = (12598784 + 21504 + 7936 + 225990912 + 129674752
+                       + 5508608 + 1772288 + 535808) / 1572864
+# The same with --precision 32: order 12.6 MB, queue 222.6 read, 127.3 written.
+DRAM_BYTES_PER_LANE_FP32 = (12602368 + 21504 + 8192 + 222643456 + 127280896) / 1572864
 
 
-def integrator_launches(precision, persistent, n):
-    """Kernels of one integrator run: the queue order (3), the start step and
-    the stages that a batch of n lanes takes (csrc/integrate.cu); init,
-    shapes, analysis and reduction are 8 more."""
-    import torch
-    per_sm = n / torch.cuda.get_device_properties(0).multi_processor_count
-    if precision == 32:
-        return 4 if persistent == 1 and per_sm > 512 else 1
-    if persistent not in (0, 1):
-        return 1
-    return 7 if per_sm > 120 else 4 if per_sm > 80 else 3 if per_sm > 20 else 2
+def launch_text(Q, wl, integ):
+    """The launches that integrate a run of wl, in words."""
+    kernels, lanes = Q.debug_run_plan(wl.systems, integ, wl.n)
+    many = {1: "one thread", 3: "three lanes", 6: "six lanes"}
+    if integ.persistent >= 2:
+        return (f"{many[lanes[0]]} per trajectory, one warp "
+                f"({10 if lanes[0] == 3 else 5} trajectories) per block")
+    if integ.precision == 32:
+        return "refill queue, one thread per trajectory" if kernels > 1 else "one thread per trajectory"
+    text = "refill queue, stages of " + ", ".join(many[k] for k in lanes) + " per trajectory"
+    return text + (f", block {integ.block or 128} x {integ.blocks_per_sm or 1}/SM variant"
+                   if lanes[0] == 1 else "")
 
 
 def kernel_sources_sha256(precision: int) -> str:
@@ -133,8 +136,9 @@ def parse():
                     help="32: FP32 integrator with Kahan-compensated updates "
                          "(rtol 1e-6, atol 1e-8), FP64 everywhere else")
     ap.add_argument("--persistent", type=int, default=1, choices=[0, 1, 2, 3],
-                    help="0: one thread per trajectory; 1: persistent refill queue; "
-                         "2 / 3: three / six lanes per trajectory (FP64, small batches)")
+                    help="launch mode: 0, 1: staged refill queue (FP64); one thread per "
+                         "trajectory, refill queue (FP32); 2 / 3: three / six lanes per "
+                         "trajectory (FP64)")
     ap.add_argument("--block", type=int, default=0)
     ap.add_argument("--blocks-per-sm", type=int, default=0)
     ap.add_argument("--tune", type=int, default=1,
@@ -462,14 +466,16 @@ def run_ours(args):
                                f"(qcams_fma_peak), this run",
                 "traffic": ((DRAM_BYTES_PER_LANE if args.precision == 64 else DRAM_BYTES_PER_LANE_FP32)
                             * wl.n if args.workload == "sweep" else None),
-                "traffic_note": "ncu dram bytes of the 3,840-lane profile case scaled by lanes"}
+                "traffic_note": "ncu dram bytes of a 1,572,864-lane sweep scaled by lanes"}
     if args.workload in ("sweep", "plain"):
         # FLOP counts are those of the Morse kernel (H2 + Ca systems)
         ach = flop_per_step * steps_per_launch / (avg_integ_ms * 1e-3)
         roofline.update(achieved=ach / 1e12, frac=ach / peak, flop_per_step=flop_per_step)
         if args.precision == 64:
-            rate = FP64_INSTR_PER_STEP * steps_per_launch / (avg_integ_ms * 1e-3)
-            roofline.update(fp64_instr_per_step=FP64_INSTR_PER_STEP, pipe_frac=rate / (peak / 2))
+            if Q.debug_run_plan(wl.systems, integ, wl.n)[1][0] == 1 and integ.persistent < 2:
+                rate = FP64_INSTR_PER_STEP * steps_per_launch / (avg_integ_ms * 1e-3)
+                roofline.update(fp64_instr_per_step=FP64_INSTR_PER_STEP,
+                                pipe_frac=rate / (peak / 2))
         else:
             props = torch.cuda.get_device_properties(dev)
             mhz = (clock_info or {}).get("sm_mhz") or 2070.0
@@ -507,13 +513,8 @@ def run_ours(args):
         "scaling": "weak", "vs_baseline": None, "dtype": f"f{args.precision}",
         "data": "synthetic",
         "config": {"workload": wl.name, "trajectories_per_gpu": wl.n,
-                   "launch": {0: "one thread/lane", 1: "persistent refill queue",
-                              2: "three lanes/trajectory",
-                              3: "six lanes/trajectory"}[integ.persistent]
-                   + (", CUDA graph" if graph is not None else "")
-                   + (f", block {integ.block or 128} x {integ.blocks_per_sm or 1}/SM variant"
-                      if integ.persistent < 2 else
-                      f", one warp ({10 if integ.persistent == 2 else 5} trajectories) per block"),
+                   "launch": launch_text(Q, wl, integ)
+                   + (", CUDA graph" if graph is not None else ""),
                    "autotune": tune,
                    "rtol": wl.integ["rtol"], "atol": wl.integ["atol"],
                    "arithmetic": ("FP64 state, forces and new-state sums; stage corrections, "
@@ -526,7 +527,10 @@ def run_ours(args):
                    "parallelism": (f"id-range shards x{world} + int64 all_reduce of the "
                                    f"histograms" if world > 1 else "single GPU")},
         "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e,
-        "gpu_launches": (8 + integrator_launches(args.precision, integ.persistent, wl.n)) * args.steps,
+        # beside those that integrate: init 4 (shapes, marks, levels, states), shapes,
+        # analysis, and the reduction's 2 (1 up to 1,024 lanes)
+        "gpu_launches": (6 + (2 if wl.n > 1024 else 1)
+                         + Q.debug_run_plan(wl.systems, integ, wl.n)[0]) * args.steps,
         "clocks": clock_info,
         "outcomes": {"cls_counts_Q_RAC_RBC_D_AMBIG_FAIL": cls_counts,
                      "merged_cls_counts_all_ranks": merged_counts,
@@ -587,18 +591,15 @@ def time_steps(Q, wl, integ, steps, warmup, dev):
     return {"workload": wl.name, "trajectories": wl.n, "steps": steps, "warmup": warmup,
             "value": wl.n / (ms * 1e-3), "unit": "trajectories/s", "ms_per_step": ms,
             "integrate_ms": float(np.mean(integ_ms)), "analyze_ms": float(np.mean(analyze_ms)),
-            "launch": (f"{'three' if integ.persistent == 2 else 'six'} lanes per trajectory, "
-                       "CUDA graph" if integ.persistent >= 2 else
-                       f"persistent refill queue, CUDA graph, block {integ.block or 128} x "
-                       f"{integ.blocks_per_sm or 1}/SM variant"),
+            "launch": launch_text(Q, wl, integ) + ", CUDA graph",
             "cls_counts_Q_RAC_RBC_D_AMBIG_FAIL": cls, "clocks": clock_info}
 
 
 def run_extras(args, dev):
     """Short measurements of the other workloads after the headline sweep
     (single GPU, outside its timed region): the 1,000-lane plain study (the
-    autotuner's launch, and one thread per trajectory for comparison) and
-    the 2,000,000-lane mixed study in FP64 (autotuned launch shape), the
+    autotuner's launch, and launch mode 1 for comparison) and the
+    2,000,000-lane mixed study in FP64 (the autotuner's launch), the
     sweep with the FP32 integrator, and the learned-proposal study."""
     import torch
     from paper_2304_02731_gb300 import qcams as Q
@@ -616,8 +617,8 @@ def run_extras(args, dev):
     wl = W.plain_h2_ca()
     out["plain_fp64"] = time_steps(Q, wl, tuned(wl, Q.make_integ(**wl.integ, persistent=True)),
                                    5, 3, dev)
-    out["plain_fp64_one_thread"] = time_steps(
-        Q, wl, Q.make_integ(**wl.integ, persistent=True, block=64, blocks_per_sm=1), 5, 3, dev)
+    out["plain_fp64_mode1"] = time_steps(Q, wl, Q.make_integ(**wl.integ, persistent=True), 5, 3,
+                                         dev)
     wl = W.sweep_h2_ca()
     wl.integ = dict(W.INTEG_FP32)
     wl.name += "_fp32"

@@ -57,6 +57,17 @@ int qcams_debug_ff_dot(const double* a, const double* w, int32_t m, double* out,
                        int64_t n, void* cuda_stream);
 
 /*
+ * Diagnostic: the kernels that qcams_run_batch launches to integrate n lanes
+ * of these systems with these parameters on the current device (outputs that
+ * do not overlap; the potential shapes and the analysis are one kernel each
+ * beside them).  *n_kernels is their number; lanes[0 .. *n_stages) receives
+ * the lanes per trajectory of those that take steps, in order (host arrays;
+ * room for 8).  Host-only and synchronous.
+ */
+int qcams_debug_run_plan(const qcams_system* sys, int32_t n_sys, const qcams_integ* integ,
+                         int64_t n, int32_t* n_kernels, int32_t* n_stages, int32_t lanes[8]);
+
+/*
  * Whether the per-device context of the current device exists: *out = 1 if
  * a call that uses it (qcams_levels, qcams_init_states, qcams_run_batch,
  * qcams_analyze, qcams_autotune, qcams_last_run_stats) has created it since

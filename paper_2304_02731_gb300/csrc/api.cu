@@ -1603,6 +1603,24 @@ int qcams_debug_ff_dot(const double* a, const double* w, int32_t m, double* out,
   return cuda_status(launch_ff_dot_check(a, w, m, out, out_f, n, (cudaStream_t)cuda_stream));
 }
 
+int qcams_debug_run_plan(const qcams_system* sys, int32_t n_sys, const qcams_integ* integ,
+                         int64_t n, int32_t* n_kernels, int32_t* n_stages, int32_t lanes[8]) {
+  if (n < 0 || !n_kernels || !n_stages || !lanes) return QCAMS_E_INVALID;
+  SysSet ss;
+  IntegParams ip;
+  int rc = make_sysset(sys, n_sys, &ss);
+  if (rc != QCAMS_OK) return rc;
+  if ((rc = make_integ_params(integ, &ip)) != QCAMS_OK) return rc;
+  int sms = 0, dev = 0, stages = 0, per[8] = {0};
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return QCAMS_E_NODEVICE;
+  *n_kernels = integrate_plan(ss, ip, integ->precision, integ->persistent, n, sms, per, &stages);
+  *n_stages = stages;
+  for (int k = 0; k < 8; ++k) lanes[k] = k < stages ? per[k] : 0;
+  return QCAMS_OK;
+}
+
 int qcams_debug_context_exists(int32_t* out) {
   if (!out) return QCAMS_E_INVALID;
   int dev = 0;

@@ -58,8 +58,10 @@
 namespace qcams {
 namespace {
 
-// Coefficients in the constant bank: a DFMA takes a constant-bank operand at
-// full rate, so indexing this table with compile-time indices costs nothing.
+// Coefficients in the constant bank, indexed at compile time.  A DFMA with a
+// constant-bank operand takes 76 cycles instead of 64 (regop.cuh), so only the
+// few products formed once per step read it directly; the weights b, which
+// multiply every component, are staged in shared memory for register loads.
 __constant__ RknTab kT = make_rkn_tab();
 
 // The coefficients of the float-float sums as float pairs.
@@ -537,7 +539,8 @@ __global__ void __launch_bounds__(128) k_start_step(SysSet sys, IntegParams ip, 
 // results do not depend on the order at all.  Lanes that already come that way
 // (a sweep of rising energies) keep their own order, since neighbours of equal
 // length finish together: 221,184 of them took 0.35 % more when shuffled.
-// It moves 40 bytes a lane, which is little beside the run: with it 200,000
+// It reads t_scale three times and writes and reads a list entry, 40 bytes a
+// lane, of which 8 come from DRAM (1.6 M lanes: the list stays in L2): with it 200,000
 // mixed lanes at scattered energies take 612 ms instead of 763 (FP64), and
 // 1,000,000 labelling lanes 28.6 ms instead of 38.4 (FP32).
 constexpr int kOrderBuckets = 4096, kOrderBlock = 1024, kOrderChunk = 4096;
@@ -890,17 +893,39 @@ constexpr int kOneThreadMinPerSm = 512;
 constexpr int kOrderMinPerSm = 120;
 static_assert(4 + 4 * kNumStages <= kCounters, "a counter block per stage");
 
+// The stages that a batch of n lanes takes.
+struct StagePlan {
+  bool order = false;          // takes the queue order
+  int n = 0;                   // stages, from first to last:
+  int stage[kNumStages];       // index into kStages
+  int64_t bound[kNumStages];   // the most trajectories it can meet
+  int64_t keep[kNumStages];    // hands on at this many (0: runs to the end)
+};
+StagePlan plan_stages(bool morse, bool lists, int64_t n, int64_t sms) {
+  StagePlan p;
+  p.order = lists && n > kOrderMinPerSm * sms && n >= kOrderMinLanes;
+  int64_t bound = n;
+  for (int s = 0; s < kNumStages; ++s) {
+    const int64_t keep = kStages[s].keep_per_sm * sms;
+    if (kStages[s].lanes == 1 ? !(morse && lists && n >= kOneThreadMinPerSm * sms) : bound <= keep)
+      continue;
+    p.stage[p.n] = s;
+    p.bound[p.n] = bound;
+    p.keep[p.n] = lists ? keep : 0;
+    if (p.keep[p.n++] == 0) break;
+    bound = keep < bound ? keep : bound;
+  }
+  return p;
+}
+
 template <bool MORSE>
 cudaError_t launch_stages(const SysSet& sys, const DevShape* shapes, const IntegParams& ip,
                           const DevBatch& b, int variant, Ctx& ctx, cudaStream_t st) {
-  const int64_t sms = ctx.sm_count;
-  const bool lists = lists_usable(b);
-  int64_t bound = b.n;   // the most trajectories the next stage can meet
-  bool started = false;
+  const StagePlan plan = plan_stages(MORSE, lists_usable(b), b.n, ctx.sm_count);
   StageQueue q;
   long long* list[2] = {reinterpret_cast<long long*>(b.vprime),
                         reinterpret_cast<long long*>(b.jprime)};
-  if (lists && b.n > kOrderMinPerSm * sms && b.n >= kOrderMinLanes) {   // slowest collisions first
+  if (plan.order) {   // slowest collisions first
     cudaError_t e = launch_queue_order(b, list[0], reinterpret_cast<unsigned*>(b.jprime),
                                        ctx.counters + 3, st);
     if (e != cudaSuccess) return e;
@@ -908,37 +933,32 @@ cudaError_t launch_stages(const SysSet& sys, const DevShape* shapes, const Integ
     q.n_in = ctx.counters + 3;
     std::swap(list[0], list[1]);
   }
-  for (int s = 0; s < kNumStages; ++s) {
-    const Stage& g = kStages[s];
-    const int64_t keep = g.keep_per_sm * sms;
-    if (g.lanes == 1 ? !(MORSE && lists && b.n >= kOneThreadMinPerSm * sms) : bound <= keep)
-      continue;
-    unsigned long long* c = ctx.counters + 4 + 4 * s;
+  for (int k = 0; k < plan.n; ++k) {
+    const int lanes = kStages[plan.stage[k]].lanes;
+    unsigned long long* c = ctx.counters + 4 + 4 * plan.stage[k];
     q.head = c;
     q.retired = c + 1;
     q.n_out = c + 2;
     q.list_out = list[0];
-    q.keep = lists ? keep : 0;
+    q.keep = plan.keep[k];
     cudaError_t e = cudaSuccess;
-    if (g.lanes == 1) {
+    if (lanes == 1) {
       e = launch_variant(variant, sys, ip, b, ctx.sm_count, ctx.counters, q, st);
     } else {
-      if (!started) {
+      if (k == 0) {
         k_start_step<MORSE>
             <<<(unsigned)((b.n + 127) / 128), 128, 0, st>>>(sys, ip, b, ctx.counters);
         e = cudaGetLastError();
       }
       if (e == cudaSuccess)
-        e = launch_integrate_queue(sys, shapes, ip, b, g.lanes, bound, ctx.sm_count,
+        e = launch_integrate_queue(sys, shapes, ip, b, lanes, plan.bound[k], ctx.sm_count,
                                    ctx.counters, q, st, MORSE);
     }
-    if (e != cudaSuccess || q.keep == 0) return e;
-    started = true;
+    if (e != cudaSuccess) return e;
     q.list_in = q.list_out;
     q.n_in = q.n_out;
     q.handed_on = true;
     std::swap(list[0], list[1]);
-    bound = keep < bound ? keep : bound;
   }
   return cudaSuccess;
 }
@@ -966,6 +986,25 @@ cudaError_t launch_integrate(const SysSet& sys, const DevShape* shapes, const In
   if (v < 0) return cudaErrorInvalidValue;
   return morse ? launch_stages<true>(sys, shapes, ip, b, v, ctx, st)
                : launch_stages<false>(sys, shapes, ip, b, v, ctx, st);
+}
+
+int integrate_plan(const SysSet& sys, const IntegParams& ip, int precision, int persistent,
+                   int64_t n, int sm_count, int lanes[8], int* n_stages) {
+  *n_stages = 1;
+  lanes[0] = 1;
+  if (n == 0) return *n_stages = 0;
+  const bool morse = all_morse(sys);
+  if (precision == 32) return integrate32_queue(morse, sys.n == 1, persistent, n, sm_count) ? 4 : 1;
+  if (ip.fixed_step) return 1;
+  if (persistent >= 2) {
+    lanes[0] = persistent == 2 ? 3 : 6;
+    return 1;
+  }
+  const StagePlan p = plan_stages(morse, true, n, sm_count);
+  static_assert(kNumStages <= 8, "room in lanes");
+  *n_stages = p.n;
+  for (int k = 0; k < p.n; ++k) lanes[k] = kStages[p.stage[k]].lanes;
+  return (p.order ? 3 : 0) + (lanes[0] == 1 ? 0 : 1) + p.n;
 }
 
 int integrate_variant_count() { return kNumVariants; }

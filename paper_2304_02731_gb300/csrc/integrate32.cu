@@ -674,21 +674,26 @@ cudaError_t launch32_persistent(const SysSetF& sf, const DevShape* shapes, const
   return cudaGetLastError();
 }
 
+// Whether a batch runs in the refill queue (mode 1).
+//
+// The queue pays once a batch is several times what the GPU holds (384 to
+// 640 lanes per SM): below, there is little to refill, its attempts are
+// slower than those of one thread per lane, and its slowest lanes, taken
+// first, share warps and SMs.  Milliseconds, queue / one thread each:
+//   sweep, all energies       60,000 16.2 / 9.2, 125,000 21.0 / 12.9,
+//                             260,000 22.0 / 20.1, 300,000 21.3 / 22.4
+//   three generic systems     125,000 20.2 / 16.3, 260,000 25.2 / 22.7,
+//                             300,000 22.9 / 23.9
+//   LJ(12,6), one system      100,000 13.3 / 12.1, 125,000 12.8 / 13.6,
+//                             150,000 13.6 / 13.0, 175,000 12.7 / 14.3
+bool queue_pays(bool morse, bool one, int persistent, int64_t n, int64_t sms) {
+  return persistent && n > (!morse && one ? 1024 : 1792) * sms;
+}
+
 template <bool MORSE, bool ONE>
 cudaError_t launch32(const SysSetF& sf, const DevShape* shapes, const IntegParams& ip,
                      const DevBatch& b, int persistent, Ctx& ctx, cudaStream_t st) {
-  // The queue pays once a batch is several times what the GPU holds (384 to
-  // 640 lanes per SM): below, there is little to refill, its attempts are
-  // slower than those of one thread per lane, and its slowest lanes, taken
-  // first, share warps and SMs.  Milliseconds, queue / one thread each:
-  //   sweep, all energies       60,000 16.2 / 9.2, 125,000 21.0 / 12.9,
-  //                             260,000 22.0 / 20.1, 300,000 21.3 / 22.4
-  //   three generic systems     125,000 20.2 / 16.3, 260,000 25.2 / 22.7,
-  //                             300,000 22.9 / 23.9
-  //   LJ(12,6), one system      100,000 13.3 / 12.1, 125,000 12.8 / 13.6,
-  //                             150,000 13.6 / 13.0, 175,000 12.7 / 14.3
-  constexpr int64_t queue_per_sm = !MORSE && ONE ? 1024 : 1792;
-  if (persistent && b.n > queue_per_sm * ctx.sm_count)
+  if (queue_pays(MORSE, ONE, persistent, b.n, ctx.sm_count))
     return launch32_persistent<MORSE, ONE>(sf, shapes, ip, b, ctx, st);
   const unsigned grid = (unsigned)((b.n + 127) / 128);
   k_integrate32_plain<MORSE, ONE><<<grid, 128, 0, st>>>(sf, shapes, ip, b, ctx.counters);
@@ -696,6 +701,10 @@ cudaError_t launch32(const SysSetF& sf, const DevShape* shapes, const IntegParam
 }
 
 }  // namespace
+
+bool integrate32_queue(bool all_morse, bool one, int persistent, int64_t n, int sm_count) {
+  return queue_pays(all_morse, one, persistent, n, sm_count);
+}
 
 cudaError_t launch_integrate32(const SysSet& sys, const DevShape* shapes, const IntegParams& ip,
                                const DevBatch& b, int persistent, Ctx& ctx, cudaStream_t st,

@@ -127,6 +127,15 @@ cudaError_t launch_integrate32(const SysSet& sys, const DevShape* shapes, const 
                                const DevBatch& b, int persistent, Ctx& ctx, cudaStream_t st,
                                bool all_morse);
 
+// Whether an FP32 batch of n lanes takes the refill queue.
+bool integrate32_queue(bool all_morse, bool one, int persistent, int64_t n, int sm_count);
+
+// The launches of launch_integrate for n lanes (outputs that do not overlap):
+// returns the number of kernels; lanes[0 .. *n_stages) receives the lanes per
+// trajectory of each kernel that integrates.
+int integrate_plan(const SysSet& sys, const IntegParams& ip, int precision, int persistent,
+                   int64_t n, int sm_count, int lanes[8], int* n_stages);
+
 // Drop the no-allocation entry point's cached scratch address for a device
 // (noalloc.cu); qcams_shutdown calls it.
 void noalloc_forget_device(int dev);

@@ -37,7 +37,7 @@ EXPORTS = ["qcams_status_string", "qcams_system_setup", "qcams_levels", "qcams_i
            "qcams_run_batch", "qcams_analyze", "qcams_reduce_xsec", "qcams_last_run_stats",
            "qcams_fma_peak", "qcams_device_info", "qcams_shutdown", "qcams_run_batch_noalloc",
            "qcams_debug_exp", "qcams_debug_force_math", "qcams_debug_ff_dot",
-           "qcams_debug_context_exists", "qcams_xsec_from_hist", "qcams_autotune", "qcams_mlp_init", "qcams_mlp_sync",
+           "qcams_debug_context_exists", "qcams_debug_run_plan", "qcams_xsec_from_hist", "qcams_autotune", "qcams_mlp_init", "qcams_mlp_sync",
            "qcams_mlp_features", "qcams_mlp_fit_standardizer", "qcams_mlp_grad",
            "qcams_mlp_train_step", "qcams_mlp_train", "qcams_mlp_infer", "qcams_build_proposal",
            "qcams_sample_proposal", "qcams_rate_constants", "qcams_gb_distribution"]
@@ -147,6 +147,8 @@ def lib():
                 "qcams_debug_force_math": (C.c_int, [V, D, D, V, V, V, I64, V]),
                 "qcams_debug_ff_dot": (C.c_int, [V, V, I32, V, V, I64, V]),
                 "qcams_debug_context_exists": (C.c_int, [P(I32)]),
+                "qcams_debug_run_plan": (C.c_int, [P(System), I32, P(Integ), I64, P(I32), P(I32),
+                                                   P(I32)]),
                 "qcams_autotune": (C.c_int, [P(System), I32, P(Integ), P(CBatch), I64,
                                              P(TuneResult), P(I32), P(Integ), V]),
                 "qcams_mlp_init": (C.c_int, [P(CMLP), C.c_uint64, V]),
@@ -508,6 +510,16 @@ def debug_context_exists() -> bool:
     out = C.c_int32(0)
     _check(lib().qcams_debug_context_exists(C.byref(out)), "qcams_debug_context_exists")
     return bool(out.value)
+
+
+def debug_run_plan(systems, integ: Integ, n: int):
+    """qcams_debug_run_plan: (kernels that integrate n lanes, lanes per
+    trajectory of each that takes steps)."""
+    arr = systems_array(systems)
+    kernels, stages, lanes = C.c_int32(), C.c_int32(), (C.c_int32 * 8)()
+    _check(lib().qcams_debug_run_plan(arr, len(systems), C.byref(integ), int(n), C.byref(kernels),
+                                      C.byref(stages), lanes), "qcams_debug_run_plan")
+    return kernels.value, list(lanes[:stages.value])
 
 
 def device_info():
