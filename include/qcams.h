@@ -23,11 +23,14 @@
  *     CUDA device (or managed) memory of the current device; "host" arrays
  *     are ordinary host memory.  The library keeps only a small per-device
  *     context (level table, potential shape table, work counters), created
- *     on first use with cudaMalloc and released by qcams_shutdown(); make
- *     the first call on a device before capturing any of its calls into a
- *     CUDA graph.  Calls that use the context on one device (qcams_levels,
- *     qcams_init_states, qcams_run_batch, qcams_analyze, qcams_autotune,
- *     qcams_last_run_stats) share it: serialise them on one stream.
+ *     on first use with cudaMalloc, and 1 MB of pinned host memory per
+ *     process, created by the first qcams_reduce_xsec that returns cross
+ *     sections; qcams_shutdown() releases both (a caller that resets a
+ *     device calls it first).  Make the first call on a device before
+ *     capturing any of its calls into a CUDA graph.  Calls that use the
+ *     context on one device (qcams_levels, qcams_init_states,
+ *     qcams_run_batch, qcams_analyze, qcams_autotune, qcams_last_run_stats)
+ *     share it: serialise them on one stream.
  *   - Streams: `cuda_stream` is a cudaStream_t (NULL = legacy default
  *     stream).  Calls only enqueue work on it and return without waiting,
  *     except where a function states that it synchronises.
@@ -484,14 +487,15 @@ int qcams_mlp_train_step(qcams_mlp* m, const float* x, const uint8_t* cls, int64
                          float lr, float* loss_out, void* cuda_stream);
 /*
  * `steps` minibatch Adam steps on the samples (x[n][8], cls[n]) as
- * qcams_mlp_train_step takes them, all on the device: before each step the
- * batch row indices idx[0..batch) (caller-owned device int64 scratch) are
- * drawn uniformly on [0, n) with replacement (Philox4x32-10, key = seed,
- * counter (i, step_lo, step_hi, 4) with step = m->step before the update;
- * index = high 64 bits of (w1:w0) * n), the gradient is taken over the
- * gathered rows and Adam updates the parameters.  losses (device float
- * [steps], optional) receives each step's minibatch loss.  On return idx
- * holds the last step's indices.  Asynchronous; capturable in a graph.
+ * qcams_mlp_train_step takes them, all on the device: for each step the
+ * batch row indices are drawn uniformly on [0, n) with replacement
+ * (Philox4x32-10, key = seed, counter (i, step_lo, step_hi, 4) with step =
+ * m->step before the update; index = high 64 bits of (w1:w0) * n), the
+ * gradient is taken over the gathered rows and Adam updates the parameters.
+ * losses (device float [steps], optional) receives each step's minibatch
+ * loss, idx[0..batch) (caller-owned device int64) the last step's indices.
+ * With at most 16 rows a minibatch has one result; with more, sums of its
+ * gradient are added in no fixed order.  Asynchronous; capturable in a graph.
  */
 int qcams_mlp_train(qcams_mlp* m, const float* x, const uint8_t* cls, int64_t n, int64_t steps,
                     int32_t batch, float lr, uint64_t seed, int64_t* idx, float* losses,
@@ -587,7 +591,8 @@ int qcams_fma_peak(int32_t precision, double* flops_per_s, void* cuda_stream);
 /* Device properties used for launch shapes: SM count and CC. */
 int qcams_device_info(int32_t* sm_count, int32_t* cc_major, int32_t* cc_minor);
 
-/* Release the per-device context of the current device. */
+/* Release the per-device context of the current device, and the process's
+ * pinned host memory (created again by the next call that needs it). */
 int qcams_shutdown(void);
 
 #ifdef __cplusplus

@@ -9,11 +9,12 @@
 // accumulator fragment of two adjacent 16x8 output tiles has exactly the
 // register layout of the A operand of a 16x16 slice, so a layer's SiLU output
 // is fed to the next layer's products without touching shared memory.  The
-// backward pass reuses the same fragments: dA = dZ W uses transposed weights
-// staged in shared memory.  Training leaves each block round's transposed
-// activations and errors in shared tiles; the weight gradients dW = dZ^T A
-// are then block GEMMs over the round's samples (K = 128), accumulated in
-// registers and added to the global gradient once per round.
+// backward pass reuses the same fragments: dA = dZ W reads the weight tiles
+// of the forward pass transposed (ldmatrix.trans).  Training leaves each block
+// round's transposed activations and errors in shared tiles; the weight
+// gradients dW = dZ^T A are then block GEMMs over the round's samples (K = 64
+// or 128), accumulated in registers and added to the global gradient once per
+// round.
 //
 // The network is ~9k multiply-adds per sample: negligible next to the
 // trajectory integration, so a warp-level mma kernel is enough here.
