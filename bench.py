@@ -66,7 +66,7 @@ KERNEL_SOURCES = {
     32: ["integrate32.cu", "dp5_tableau.cuh"],
 }
 COUNTS_SOURCE_SHA256 = {
-    64: "59f5303cd5ecce0b674d6e6f417074e69aa932133a9bb00a6fc440d22a0c3c6b",
+    64: "03f166477a14257d142e78ecdc556e39ad7cc72557ced5fbeb3314d0e4748489",
     32: "e32052676aff67b078d3851bfe3de6baef8de151f02049e17bc7508e86a8d9f1",
 }
 # DRAM bytes per trajectory of an integrator run: ncu dram__bytes_read.sum +

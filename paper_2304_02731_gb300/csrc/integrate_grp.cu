@@ -127,7 +127,7 @@ __device__ __forceinline__ float grp_norm_seq(const float* qr, const float* qv, 
 // The lanes of a warp hold different pairs, so the
 // generic form is one sequence for the Morse, Buckingham and (12,6) / (8,6)
 // Lennard-Jones kinds with selected operands instead of a branch per kind.
-template <bool MORSE>
+template <bool MORSE, bool SEQ>
 __device__ __forceinline__ double pair_u_grp(const DevPair& q, double s,
                                              const double* __restrict__ T,
                                              const OpReg& op) {
@@ -153,7 +153,7 @@ __device__ __forceinline__ double pair_u_grp(const DevPair& q, double s,
   const double B = fma(isM ? -x : q.c3, isM ? x : (isL ? ri6 : hh), isM ? x : -A);
   const double C = op.mul(B, isM ? A : ri2);
   double u = isB ? B : C;
-  if (general) u = pot_g(q, ri, s * ri);
+  if (general) u = SEQ ? lj_u(q, ri, op) : pot_g(q, ri, s * ri);
   return u;
 }
 
@@ -199,7 +199,7 @@ __device__ __forceinline__ void accel_grp(const Grp<G>& L,
   const double c2 = !SEQ || L.j == 0 ? rk[1] : (L.j == 1 ? rk[0] : rj);
   const double s = fma(c0, c0, fma(c1, c1, op.mul(c2, c2)));
   s_own = s;
-  const double u = pair_u_grp<MORSE>(L.q, s, T, op);
+  const double u = pair_u_grp<MORSE, SEQ>(L.q, s, T, op);
   if (G == 3) {
     const double f = op.mul(L.kf, u), h = op.mul(L.kh, u);
     const double f0 = __shfl_sync(FULL, f, L.base), f1 = __shfl_sync(FULL, f, L.base + 1),

@@ -13,6 +13,15 @@
 namespace qcams {
 namespace {
 
+// u of a Lennard-Jones pair with any exponents.  The difference's fused
+// product is written out: left to the compiler it is the other one in some
+// kernels, and the one-thread and lane-group forms would differ in the last
+// bit.
+template <class OP>
+__device__ __forceinline__ double lj_u(const DevPair& q, double ri, const OP& op) {
+  return op.mul(fma(-q.c2, ipow(ri, q.m), op.mul(q.c3, ipow(ri, q.n))), op.mul(ri, ri));
+}
+
 // The exponents' arguments take alpha r as (alpha s) (1/sqrt(s)): alpha s
 // is formed while the reciprocal square root is refined, so the argument
 // is one FP64 instruction after it instead of two (the same instruction
@@ -47,7 +56,7 @@ __device__ __forceinline__ double pair_u(const DevPair& q, double s, const doubl
     const double h = q.m == 12 ? ri6 : ri4;
     return op.mul(fma(q.c3, ri6, -op.mul(q.c2, op.mul(h, h))), ri2);
   }
-  return pot_g(q, ri, s * ri);
+  return lj_u(q, ri, op);
 }
 
 }  // namespace
